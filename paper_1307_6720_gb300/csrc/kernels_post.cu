@@ -149,6 +149,94 @@ __global__ void trace_kernel(TraceGeom G, const double* __restrict__ Bx, const d
     lengths[q] = len;
 }
 
+// The same lines with four lanes per line: lane a (a < 3) owns coordinate a
+// of the point and component a of B, the fourth mirrors the third; cell
+// indices, cell fractions and squares of B's components travel by shuffles
+// within the four.  Every value is formed by the operations of trace_dir in
+// their order, so the lines equal trace_kernel's bit for bit.
+//
+// Bound by the FP64 pipe (16 cycles of an SM's pipe per warp instruction,
+// whatever its active lanes) on few warps: one thread per line runs about 200
+// FP64 instructions per stage and 2048 lines fill 64 warps; here a warp
+// runs about 60 per stage for its eight lines and 2048 lines make 256 warps.
+// 2048 lines of 200 steps through a 129^3 field: 4.59 -> 1.82 ms; what is
+// left is the dependent FP64 chain of a stage (32 % of the pipe's cycles).
+__device__ __forceinline__ bool trace_dir4(const TraceGeom& G, const double* __restrict__ F, double L, double h, int n,
+                                           int a, int base, double dir, double r, double& v) {
+    const unsigned full = 0xffffffffu;
+    const bool in = r >= 0.0 && r <= L;
+    const double s = __ddiv_rn(r, h);
+    int i = int(floor(s));
+    if (i > n - 2) i = n - 2;
+    if (i < 0) i = 0;
+    const double f = sub(s, double(i));
+    const int cx = __shfl_sync(full, i, base), cy = __shfl_sync(full, i, base + 1), cz = __shfl_sync(full, i, base + 2);
+    const double f0 = __shfl_sync(full, f, base), f1 = __shfl_sync(full, f, base + 1), f2 = __shfl_sync(full, f, base + 2);
+    const size_t o = size_t(cx) + G.px * size_t(cy) + G.plane * size_t(cz);
+    double e[2][2];
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+            const size_t q = o + G.px * size_t(dy) + G.plane * size_t(dz);
+            e[dz][dy] = add(mul(F[q], sub(1.0, f0)), mul(F[q + 1], f0));
+        }
+    const double e0 = add(mul(e[0][0], sub(1.0, f1)), mul(e[0][1], f1));
+    const double e1 = add(mul(e[1][0], sub(1.0, f1)), mul(e[1][1], f1));
+    const double b = add(mul(e0, sub(1.0, f2)), mul(e1, f2));
+    const double bb = mul(b, b);
+    const double b0 = __shfl_sync(full, bb, base), b1 = __shfl_sync(full, bb, base + 1),
+                 b2 = __shfl_sync(full, bb, base + 2);
+    const double m = __dsqrt_rn(add(add(b0, b1), b2));
+    v = __ddiv_rn(mul(dir, b), m);
+    // every coordinate in the box (the four lanes of the line) and |B| > 0
+    const unsigned inside = __ballot_sync(full, in) >> base;
+    return (inside & 15u) == 15u && m > 0.0;
+}
+
+constexpr int TRACE4_THREADS = 32;
+
+__global__ void __launch_bounds__(TRACE4_THREADS)
+trace4_kernel(TraceGeom G, const double* __restrict__ Bx, const double* __restrict__ By, const double* __restrict__ Bz,
+              const double* __restrict__ seeds, int n, double ds, int max_steps, double dir, double* __restrict__ points,
+              int* __restrict__ lengths) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, base = lane & ~3, a = min(lane & 3, 2);
+    const int q = blockIdx.x * (TRACE4_THREADS / 4) + threadIdx.x / 4;
+    const bool line = q < n, own = line && (lane & 3) < 3;
+    const double* F = a == 0 ? Bx : a == 1 ? By : Bz;
+    const double L = a == 0 ? G.L[0] : a == 1 ? G.L[1] : G.L[2];
+    const int na = a == 0 ? G.n[0] : a == 1 ? G.n[1] : G.n[2];
+    const double h = __ddiv_rn(L, double(na - 1));
+    double r = line ? seeds[3 * size_t(q) + a] : 0.0;
+    double* out = points + size_t(line ? q : 0) * size_t(max_steps + 1) * 3 + a;
+    // the warp's lines advance together; a line that has ended idles
+    // (warp votes stand in statements of their own: every lane takes part)
+    const unsigned start = __ballot_sync(full, r >= 0.0 && r <= L) >> base;
+    bool alive = line && (start & 15u) == 15u;
+    int len = alive ? 1 : 0;
+    if (alive && own) out[0] = r;
+    const double hs = mul(0.5, ds), s6 = __ddiv_rn(ds, 6.0);
+    for (int step = 0; step < max_steps; ++step) {
+        const int any = __any_sync(full, alive);
+        if (!any) break;
+        double k1, k2, k3, k4;
+        bool ok = trace_dir4(G, F, L, h, na, a, base, dir, r, k1);
+        ok &= trace_dir4(G, F, L, h, na, a, base, dir, add(r, mul(hs, k1)), k2);
+        ok &= trace_dir4(G, F, L, h, na, a, base, dir, add(r, mul(hs, k2)), k3);
+        ok &= trace_dir4(G, F, L, h, na, a, base, dir, add(r, mul(ds, k3)), k4);
+        const double e = add(r, mul(s6, add(add(add(k1, mul(2.0, k2)), mul(2.0, k3)), k4)));
+        const unsigned taken = __ballot_sync(full, ok && e >= 0.0 && e <= L) >> base;
+        alive = alive && (taken & 15u) == 15u;
+        if (alive) {
+            r = e;
+            if (own) out[3 * size_t(len)] = e;
+            ++len;
+        }
+    }
+    if (line && (lane & 3) == 0) lengths[q] = len;
+}
+
 }  // namespace
 
 void launch_current(const Geom& g, double mu0, const double* Bx, const double* By, const double* Bz, double* jx,
@@ -162,12 +250,23 @@ void launch_current(const Geom& g, double mu0, const double* Bx, const double* B
     MHS_CUDA(cudaGetLastError());
 }
 
+// Four lanes per line up to the count of lines that gives the one-lane form a
+// warp per SM; past it the one-lane form's smaller total (no duplicated
+// square roots and votes) wins, as both then keep every SM's FP64 pipe busy.
+constexpr int TRACE4_LINES = 32 * 152;
+
 void launch_trace(int nx, int ny, int nz, double Lx, double Ly, double Lz, size_t px, size_t plane, const double* Bx,
                   const double* By, const double* Bz, const double* seeds, int n, double ds, int max_steps,
                   double dir, double* points, int* lengths, cudaStream_t st) {
     if (n <= 0) return;
     TraceGeom G{{nx, ny, nz}, {Lx, Ly, Lz}, px, plane};
-    trace_kernel<<<(n + 63) / 64, 64, 0, st>>>(G, Bx, By, Bz, seeds, n, ds, max_steps, dir, points, lengths);
+    if (n <= TRACE4_LINES) {
+        constexpr int per = TRACE4_THREADS / 4;
+        trace4_kernel<<<(n + per - 1) / per, TRACE4_THREADS, 0, st>>>(G, Bx, By, Bz, seeds, n, ds, max_steps, dir,
+                                                                      points, lengths);
+    } else {
+        trace_kernel<<<(n + 31) / 32, 32, 0, st>>>(G, Bx, By, Bz, seeds, n, ds, max_steps, dir, points, lengths);
+    }
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
 }

@@ -111,3 +111,29 @@ def test_field_lines_of_solution_host_buffers(M):
     with pytest.raises(M.MhsError):
         M.mhs_trace(h, seeds, -0.1, 10)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("extra", [1, 7, 8, 31])
+def test_field_lines_do_not_depend_on_the_number_of_lines(M, extra):
+    """Up to 4864 lines run four lanes to a line, more one lane to a line; the
+    lines are the same bit for bit (lines that leave the box, a seed outside
+    it and a ragged last warp among them)."""
+    import torch
+    rng = np.random.default_rng(extra)
+    shape, box = (17, 9, 13), (1.0, 0.7, 0.9)
+    B = [torch.from_numpy(rng.standard_normal(shape)).cuda() for _ in range(3)]
+    n, steps = 4864 + extra, 40
+    seeds = torch.from_numpy(rng.uniform(0.0, 1.0, (n, 3)) * np.array(box)).cuda()
+    seeds[3] = torch.tensor([2.0, 0.1, 0.1])
+
+    def trace(part):
+        pts = torch.full((len(part), steps + 1, 3), -7.0, dtype=torch.float64, device="cuda")
+        lens = torch.zeros(len(part), dtype=torch.int32, device="cuda")
+        M.mhs_trace_field(shape, box, *B, part.contiguous(), 0.02, steps, -1, pts, lens, torch.cuda.current_stream())
+        return pts, lens
+
+    p, l = trace(seeds)
+    for a, b in ((0, extra), (extra, n)):
+        pq, lq = trace(seeds[a:b])
+        assert torch.equal(pq, p[a:b]) and torch.equal(lq, l[a:b])
+    assert int(l[3]) == 0 and int((l > 1).sum()) > n // 2 and int((l < steps + 1).sum()) > 100
