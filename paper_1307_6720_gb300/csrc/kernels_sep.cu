@@ -33,64 +33,94 @@ namespace mhs {
 
 namespace {
 
-// C_b = scale A_b B_b (+ C_b): 64 x 64 output tile per block of 256 threads,
-// 4 x 4 outputs per thread (rows ty + 16 r, columns tx + 16 c), K staged
-// through shared memory 16 at a time; block (bx, by, bz) = (column tile, row
-// tile, batch).
-constexpr int TM = 64, TN = 64, TK = 16;
-
-template <typename T>
-__device__ __forceinline__ void gemm_body(const GemmArgs<T>& g, int bx, int by, int bz) {
-    __shared__ T As[TK][TM + 4];
-    __shared__ T Bs[TK][TN + 4];
+// C_b = scale A_b B_b (+ C_b): TB x TB output tile per block of 256 threads,
+// TB/16 x TB/16 outputs per thread (rows ty + 16 r, columns tx + 16 c), K
+// staged through shared memory TK at a time; block (bx, by, bz) = (column
+// tile, row tile, batch).  Every output is one FMA chain over increasing k,
+// whatever the tile, so the results do not depend on it.
+template <typename T, int TB, int TK>
+__device__ __forceinline__ void gemm_tile(const GemmArgs<T>& g, int bx, int by, int bz, T* smem) {
+    constexpr int R = TB / 16, LD = TB + (TB > 16 ? 4 : 1);
+    T* As = smem;               // [TK][LD]
+    T* Bs = smem + TK * LD;     // [TK][LD]
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int row0 = by * TM, col0 = bx * TN;
+    const int row0 = by * TB, col0 = bx * TB;
     const long long b = bz;
     const T* A = g.A + b * g.sA;
     const T* B = g.B + b * g.sB;
     T* C = g.C + b * g.sC;
-    T acc[4][4] = {};
+    T acc[R][R] = {};
     for (int k0 = 0; k0 < g.K; k0 += TK) {
-        // A tile: 64 rows x 16 k (k fastest in global memory)
-        for (int e = threadIdx.x; e < TM * TK; e += 256) {
+        // A tile: TB rows x TK k (k fastest in global memory)
+#pragma unroll 4
+        for (int e = threadIdx.x; e < TB * TK; e += 256) {
             const int r = e / TK, kk = e % TK;
             const int gr = row0 + r, gk = k0 + kk;
-            As[kk][r] = (gr < g.M && gk < g.K) ? A[gr * g.lda + gk] : T(0);
+            As[kk * LD + r] = (gr < g.M && gk < g.K) ? A[(long long)gr * g.lda + gk] : T(0);
         }
-        // B tile: 16 k x 64 columns (columns fastest)
-        for (int e = threadIdx.x; e < TK * TN; e += 256) {
-            const int kk = e / TN, c = e % TN;
+        // B tile: TK k x TB columns (columns fastest)
+#pragma unroll 4
+        for (int e = threadIdx.x; e < TK * TB; e += 256) {
+            const int kk = e / TB, c = e % TB;
             const int gk = k0 + kk, gc = col0 + c;
-            Bs[kk][c] = (gk < g.K && gc < g.N) ? B[gk * g.ldb + gc] : T(0);
+            Bs[kk * LD + c] = (gk < g.K && gc < g.N) ? B[(long long)gk * g.ldb + gc] : T(0);
         }
         __syncthreads();
+        const int kn = min(TK, g.K - k0);
+#pragma unroll 8
+        for (int kk = 0; kk < kn; ++kk) {
+            T a[R], bb[R];
 #pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-            T a[4], bb[4];
+            for (int r = 0; r < R; ++r) a[r] = As[kk * LD + ty + 16 * r];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+            for (int c = 0; c < R; ++c) bb[c] = Bs[kk * LD + tx + 16 * c];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bb[c] = Bs[kk][tx + 16 * c];
+            for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], bb[c], acc[r][c]);
+                for (int c = 0; c < R; ++c) acc[r][c] = fma(a[r], bb[c], acc[r][c]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
         const int gr = row0 + ty + 16 * r;
         if (gr >= g.M) continue;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < R; ++c) {
             const int gc = col0 + tx + 16 * c;
             if (gc < g.N) {
                 const T v = g.scale * acc[r][c];
-                C[gr * g.ldc + gc] = g.accumulate ? C[gr * g.ldc + gc] + v : v;
+                const long long at = (long long)gr * g.ldc + gc;
+                C[at] = g.accumulate ? C[at] + v : v;
             }
         }
     }
+}
+
+// The tile of a product (GemmArgs::tile).  FP64 products are bound by the
+// FP64 pipe, one FMA per output and k whatever the tile, and their rows are
+// short: 16 x 16 tiles waste little at ragged ends and spread a 47 x 39
+// plane over nine SMs instead of one (6.6 against 59 us per product, and 9.4
+// against 59 us for the 23 planes of a 49 x 41 x 25 level).
+// FP32 products take the largest tile that still gives two blocks per SM.
+constexpr int TK64 = 16, TK32 = 32, TK16 = 64;
+constexpr int GEMM_SMEM = 2 * TK32 * 36;   // the 32 x 32 tiles' two operands, the largest
+static_assert(GEMM_SMEM >= 2 * TK16 * 17 && GEMM_SMEM >= 2 * TK64 * 68, "shared memory of the other tiles");
+
+template <typename T>
+int gemm_tile_size(int M, int N, int batch) {
+    if (sizeof(T) == 8) return 16;
+    for (int tb : {64, 32})
+        if ((long long)((M + tb - 1) / tb) * ((N + tb - 1) / tb) * batch >= 2 * 152) return tb;
+    return 16;
+}
+
+template <typename T>
+__device__ __forceinline__ void gemm_body(const GemmArgs<T>& g, int bx, int by, int bz) {
+    __shared__ T smem[GEMM_SMEM];
+    if (g.tile == 16) gemm_tile<T, 16, TK16>(g, bx, by, bz, smem);
+    else if (g.tile == 32) gemm_tile<T, 32, TK32>(g, bx, by, bz, smem);
+    else gemm_tile<T, 64, TK64>(g, bx, by, bz, smem);
 }
 
 template <typename T>
@@ -391,7 +421,8 @@ SepStage<T> gemm_stage(const GemmArgs<T>& g, int batch) {
     s.kind = SEP_GEMM;
     s.gemm = g;
     s.threads = 256;
-    s.grid = dim3((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, batch);
+    const int tb = s.gemm.tile = gemm_tile_size<T>(g.M, g.N, batch);
+    s.grid = dim3((g.N + tb - 1) / tb, (g.M + tb - 1) / tb, batch);
     return s;
 }
 

@@ -347,6 +347,7 @@ struct GemmArgs {
     long long ldc = 0, sC = 0;
     T scale = T(1);
     int accumulate = 0;
+    int tile = 64;   // output tile of a block: 64, 32 or 16 (set with the launch grid)
 };
 // mode systems on transformed data t[k][slow][fast] (k < nzi; nzi = 1: the
 // lower-boundary division by cf mu_fast + cs mu_slow)

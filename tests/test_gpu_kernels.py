@@ -606,3 +606,24 @@ def test_zline_vcycle_parity(M, prec, cut):
     want = oracle.vcycle(pr, u, f, smoother="zline")
     assert _rel(got, want) < (1e-11 if prec == 0 else 1e-5)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shape", [(19, 35, 9), (35, 19, 21), (57, 57, 89), (41, 41, 321), (11, 7, 5)])
+def test_dense_transform_tiles(M, shape, prec):
+    """Dense sine transforms at the edges of their output tiles (16, 32 and 64:
+    one interior node past a tile, ragged ends, batches that select each
+    tile), against the separable direct solution formed with plain products."""
+    from oracle import exact
+    nx, ny, nz = shape
+    pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
+    f = np.random.default_rng(nx).standard_normal((nz, ny, nx))
+    if prec == 1:
+        f = f.astype(np.float32).astype(np.float64)
+    M.mhs_level_write(h, 3, 0, M.MHS_FIELD_U, prec, np.zeros(f.shape))
+    M.mhs_level_write(h, 3, 0, M.MHS_FIELD_F, prec, f)
+    M.mhs_level_op(h, 3, 0, M.MHS_OP_EXACT, prec)
+    got = _read(M, h, 3, 0, M.MHS_FIELD_U, prec)
+    want = exact.separable_solve3d(_level_problem(M, h, pr, 3, 0), np.zeros((ny, nx)), f)
+    assert _rel(got, want) < (1e-12 if prec == 0 else 2e-5)
+    M.mhs_destroy(h)
