@@ -41,14 +41,7 @@ mhs_status guarded(F&& f) {
     }
 }
 
-bool is_device_ptr(const void* p) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-}
+using mhs::is_device_ptr;
 
 mhs_atmos_params default_atmos() { return mhs_atmos_params{1.0, 0.5, 150.0, 5.0, 10.0}; }
 
@@ -371,52 +364,23 @@ mhs_status mhs_fields(mhs_handle h, double* Bx, double* By, double* Bz, double* 
     if (!h) return fail(MHS_ERR_INVALID_ARG, "handle is NULL");
     if (!h->have_solution) return fail(MHS_ERR_BAD_STATE, "no solution yet (call mhs_solve)");
     return guarded([&] {
-        mhs::ensure_field_buffers(h);
-        const mhs::Geom& g = h->h3.g[0];
-        {
-            const double nodes = double(g.nx) * g.ny * g.nz;
-            mhs::TimedScope t(h->timer, MHS_KT_FIELDS, 48.0 * nodes, 60.0 * nodes, h->stream);
-            mhs::launch_fields(g, h->alpha, h->atm, h->prof, h->h3.d[0].u, h->fld[0], h->fld[1], h->fld[2],
-                               h->fld[3], h->fld[4], (h->opts.flags & MHS_FLAG_BZ_MIMETIC) ? 1 : 0, h->stream);
-        }
         double* outs[5] = {Bx, By, Bz, p, rho};
+        mhs::recover_fields(h, outs);
         bool host = false;
-        for (int q = 0; q < 5; ++q) {
-            if (!outs[q]) continue;
-            copy_out(h, g, outs[q], h->fld[q], size_t(g.ny) * g.nz);
-            host = host || !is_device_ptr(outs[q]);
-        }
+        for (double* o : outs) host = host || (o && !is_device_ptr(o));
         if (host) MHS_CUDA(cudaStreamSynchronize(h->stream));
         return MHS_OK;
     });
-}
-
-// B of the latest solve into h->fld (the field recovery of mhs_fields)
-static void compute_fields(mhs_handle h) {
-    mhs::ensure_field_buffers(h);
-    const mhs::Geom& g = h->h3.g[0];
-    const double nodes = double(g.nx) * g.ny * g.nz;
-    mhs::TimedScope t(h->timer, MHS_KT_FIELDS, 48.0 * nodes, 60.0 * nodes, h->stream);
-    mhs::launch_fields(g, h->alpha, h->atm, h->prof, h->h3.d[0].u, h->fld[0], h->fld[1], h->fld[2], h->fld[3],
-                       h->fld[4], (h->opts.flags & MHS_FLAG_BZ_MIMETIC) ? 1 : 0, h->stream);
 }
 
 mhs_status mhs_current(mhs_handle h, double* jx, double* jy, double* jz, double* jmag, double* bmag) {
     if (!h) return fail(MHS_ERR_INVALID_ARG, "handle is NULL");
     if (!h->have_solution) return fail(MHS_ERR_BAD_STATE, "no solution yet (call mhs_solve)");
     return guarded([&] {
-        compute_fields(h);
-        mhs::ensure_post_buffers(h);
-        const mhs::Geom& g = h->h3.g[0];
-        mhs::launch_current(g, h->atm.mu0, h->fld[0], h->fld[1], h->fld[2], h->post[0], h->post[1], h->post[2],
-                            h->post[3], h->post[4], h->stream);
         double* outs[5] = {jx, jy, jz, jmag, bmag};
+        mhs::recover_current(h, outs);
         bool host = false;
-        for (int q = 0; q < 5; ++q) {
-            if (!outs[q]) continue;
-            copy_out(h, g, outs[q], h->post[q], size_t(g.ny) * g.nz);
-            host = host || !is_device_ptr(outs[q]);
-        }
+        for (double* o : outs) host = host || (o && !is_device_ptr(o));
         if (host) MHS_CUDA(cudaStreamSynchronize(h->stream));
         return MHS_OK;
     });
@@ -473,9 +437,9 @@ mhs_status mhs_trace(mhs_handle h, const double* seeds, int n, double ds, int ma
     const mhs_status s = check_trace_args(seeds, n, ds, max_steps, direction, points, lengths);
     if (s != MHS_OK) return s;
     return guarded([&] {
-        compute_fields(h);
+        mhs::recover_b(h);
         const mhs::Geom& g = h->h3.g[0];
-        trace_any(g.nx, g.ny, g.nz, h->Lx, h->Ly, h->Lz, size_t(g.px), g.plane, h->fld[0], h->fld[1], h->fld[2],
+        trace_any(g.nx, g.ny, g.nz, h->Lx, h->Ly, h->Lz, size_t(g.nx), size_t(g.nx) * g.ny, h->fld[0], h->fld[1], h->fld[2],
                   seeds, n, ds, max_steps, direction, points, lengths, h->stream);
         return MHS_OK;
     });

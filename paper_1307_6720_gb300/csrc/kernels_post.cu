@@ -14,6 +14,8 @@
 // arithmetic uses explicitly rounded FP64 operations (no fused
 // multiply-add), in a fixed order, so that a line depends only on B and the
 // seed, not on how the compiler schedules the arithmetic.
+#include <algorithm>
+
 #include "device_util.cuh"
 #include "mhs_internal.h"
 
@@ -23,31 +25,78 @@ namespace {
 
 constexpr int BX = 32, BY = 8;
 
-// d/dx_a at node t of n along one axis, element stride s
-__device__ __forceinline__ double dif1(const double* __restrict__ f, size_t c, size_t s, int t, int n, double inv2h) {
-    if (t == 0) return (-3.0 * f[c] + 4.0 * f[c + s] - f[c + 2 * s]) * inv2h;
-    if (t == n - 1) return (3.0 * f[c] - 4.0 * f[c - s] + f[c - 2 * s]) * inv2h;
-    return (f[c + s] - f[c - s]) * inv2h;
+// numerator of d/dx_a at node t of n along one axis, element stride s (times
+// 1/(2h): the derivative); the three-point form of either end and the central
+// one share their first two terms
+__device__ __forceinline__ double num1(const double* __restrict__ f, size_t c, ptrdiff_t s, int t, int n) {
+    const bool lo = t == 0, hi = t == n - 1, end = lo || hi;
+    const double w0 = lo ? -3.0 : hi ? 3.0 : -1.0, w1 = lo ? 4.0 : hi ? -4.0 : 1.0;
+    double v = fma(w1, f[hi ? c - s : c + s], w0 * f[end ? c : c - s]);
+    if (end) v += lo ? -f[c + 2 * s] : f[c - 2 * s];
+    return v;
 }
 
-__global__ void current_kernel(Geom g, double inv_mu0, const double* __restrict__ Bx, const double* __restrict__ By,
-                               const double* __restrict__ Bz, double* __restrict__ jx, double* __restrict__ jy,
-                               double* __restrict__ jz, double* __restrict__ jmag, double* __restrict__ bmag) {
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    if (i >= g.nx || j >= g.ny) return;
-    const double ix = 0.5 / g.hx, iy = 0.5 / g.hy, iz = 0.5 / g.hz;
-    const size_t sy = g.px, sz = g.plane;
-    for (int k = blockIdx.z; k < g.nz; k += gridDim.z) {
-        const size_t c = at(g, i, j, k);
-        const double cx = (dif1(Bz, c, sy, j, g.ny, iy) - dif1(By, c, sz, k, g.nz, iz)) * inv_mu0;
-        const double cy = (dif1(Bx, c, sz, k, g.nz, iz) - dif1(Bz, c, 1, i, g.nx, ix)) * inv_mu0;
-        const double cz = (dif1(By, c, 1, i, g.nx, ix) - dif1(Bx, c, sy, j, g.ny, iy)) * inv_mu0;
+// sqrt(m): an FP32 reciprocal square root refined by one coupled Newton
+// (Goldschmidt) step for g ~ sqrt(m), h ~ 1/(2 sqrt(m)) and one correction of
+// g by its residual, 8 FP64 instructions instead of about 22; the relative
+// error before the last rounding is below 2^-80.  Arguments outside the FP32
+// range (and 0, NaN) take the library's sqrt.
+__device__ __forceinline__ double sqrt_mid(double m) {
+    if (!(m > 1e-30 && m < 1e30)) return sqrt(m);
+    const float y = rsqrtf(float(m));
+    double g = m * double(y), h = double(0.5f * y);
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(fma(-g, g, m), h, g);
+}
+
+// j and the magnitudes on dense arrays; wx, wy, wz = 1/(2 h mu0).  A block
+// owns 256 consecutive nodes of a plane and `per` consecutive planes.  Bound
+// by the FP64 pipe (12 instructions per node for j, 22 for the two
+// magnitudes): the scale 1/mu0 is folded into the difference weights, and a
+// warp without an edge node takes plain central differences (129^3: 366 ->
+// 192 us).
+__global__ void __launch_bounds__(BX * BY)
+current_kernel(int nx, int ny, int nz, int per, double wx, double wy, double wz, const double* __restrict__ Bx,
+               const double* __restrict__ By, const double* __restrict__ Bz, double* __restrict__ jx,
+               double* __restrict__ jy, double* __restrict__ jz, double* __restrict__ jmag, double* __restrict__ bmag) {
+    const size_t sz = size_t(nx) * ny;
+    const size_t e = blockIdx.x * size_t(BX * BY) + threadIdx.x;
+    const bool node = e < sz;
+    const int j = node ? int(unsigned(e) / unsigned(nx)) : 0;
+    const int i = node ? int(unsigned(e) - unsigned(j) * unsigned(nx)) : 0;
+    const bool edge = node && (i == 0 || i == nx - 1 || j == 0 || j == ny - 1);
+    const int edges = __any_sync(0xffffffffu, edge);
+    if (!node) return;
+    const ptrdiff_t sy = nx;
+    const int k0 = blockIdx.y * per, k1 = min(nz, k0 + per);
+    size_t c = e + sz * size_t(k0);
+    for (int k = k0; k < k1; ++k, c += sz) {
+        double xy, xz, yx, yz, zx, zy;   // differences of B along x of By, Bz; y of Bx, Bz; z of Bx, By
+        if (edges || k == 0 || k == nz - 1) {
+            xy = num1(By, c, 1, i, nx);
+            xz = num1(Bz, c, 1, i, nx);
+            yx = num1(Bx, c, sy, j, ny);
+            yz = num1(Bz, c, sy, j, ny);
+            zx = num1(Bx, c, (ptrdiff_t)sz, k, nz);
+            zy = num1(By, c, (ptrdiff_t)sz, k, nz);
+        } else {
+            xy = By[c + 1] - By[c - 1];
+            xz = Bz[c + 1] - Bz[c - 1];
+            yx = Bx[c + sy] - Bx[c - sy];
+            yz = Bz[c + sy] - Bz[c - sy];
+            zx = Bx[c + sz] - Bx[c - sz];
+            zy = By[c + sz] - By[c - sz];
+        }
+        const double cx = fma(yz, wy, -(zy * wz));
+        const double cy = fma(zx, wz, -(xz * wx));
+        const double cz = fma(xy, wx, -(yx * wy));
         if (jx) jx[c] = cx;
         if (jy) jy[c] = cy;
         if (jz) jz[c] = cz;
-        if (jmag) jmag[c] = sqrt(cx * cx + cy * cy + cz * cz);
-        if (bmag) bmag[c] = sqrt(Bx[c] * Bx[c] + By[c] * By[c] + Bz[c] * Bz[c]);
+        if (jmag) jmag[c] = sqrt_mid(fma(cx, cx, fma(cy, cy, cz * cz)));
+        if (bmag) bmag[c] = sqrt_mid(fma(Bx[c], Bx[c], fma(By[c], By[c], Bz[c] * Bz[c])));
     }
 }
 
@@ -241,11 +290,12 @@ trace4_kernel(TraceGeom G, const double* __restrict__ Bx, const double* __restri
 
 void launch_current(const Geom& g, double mu0, const double* Bx, const double* By, const double* Bz, double* jx,
                     double* jy, double* jz, double* jmag, double* bmag, cudaStream_t st) {
-    int gz = g.nz;
-    const int tiles = ((g.nx + BX - 1) / BX) * ((g.ny + BY - 1) / BY);
-    if (gz * tiles > 152 * 16) gz = std::max(1, 152 * 16 / tiles);
-    const dim3 grid((g.nx + BX - 1) / BX, (g.ny + BY - 1) / BY, gz);
-    current_kernel<<<grid, dim3(BX, BY), 0, st>>>(g, 1.0 / mu0, Bx, By, Bz, jx, jy, jz, jmag, bmag);
+    // about eight blocks per SM, chunks of at most 16 planes
+    const long long pl = ((long long)g.nx * g.ny + BX * BY - 1) / (BX * BY);
+    const int per = int(std::min<long long>(16, std::max<long long>(1, pl * g.nz / (152 * 8))));
+    const double m = 1.0 / mu0;
+    current_kernel<<<dim3(unsigned(pl), (g.nz + per - 1) / per), BX * BY, 0, st>>>(
+        g.nx, g.ny, g.nz, per, 0.5 / g.hx * m, 0.5 / g.hy * m, 0.5 / g.hz * m, Bx, By, Bz, jx, jy, jz, jmag, bmag);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
 }

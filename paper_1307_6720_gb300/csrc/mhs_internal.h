@@ -243,8 +243,8 @@ struct mhs_ctx {
     int* flag = nullptr;           // device flags (non-finite input detection)
     int* flag_host = nullptr;      // pinned mirror
     double* staging = nullptr;     // FP64 staging buffer of the finest size (level hooks, lazily allocated)
-    double* fld[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // pitched Bx, By, Bz, p, rho
-    double* post[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; // pitched jx, jy, jz, |j|, |B| (on first use)
+    double* fld[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // dense Bx, By, Bz, p, rho (each on first use)
+    double* post[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; // dense jx, jy, jz, |j|, |B| (each on first use)
     bool have_bz = false, have_solution = false;
     bool f_zero_finest = true;     // the finest interior right-hand side is identically zero (no hook wrote it)
     std::vector<void*> allocations;
@@ -436,8 +436,8 @@ void launch_df_copy_plane(const Geom& g2, const float* hi2, const float* lo2, co
                           cudaStream_t st);
 
 // ---- fields (kernels_fields.cu) ----
-void launch_fields(const Geom& g, double alpha, const mhs_atmos_params& atm, const double* prof,
-                   const double* P, double* Bx, double* By, double* Bz, double* p, double* rho, int bz_mode,
-                   cudaStream_t st);
+// P pitched, the fields dense [nz][ny][nx]; p and rho may be NULL (not formed)
+void launch_fields(const Geom& g, double alpha, const double* prof, const double* P, double* Bx, double* By,
+                   double* Bz, double* p, double* rho, int bz_mode, cudaStream_t st);
 
 }  // namespace mhs

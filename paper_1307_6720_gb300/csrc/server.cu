@@ -149,22 +149,16 @@ void Server::start(const std::shared_ptr<Request>& q) {
     c->have_bz = true;
     solve_begin(c, r.tol, r.mode);
     const Geom& g = c->h3.g[0];
-    if (r.phi)
-        MHS_CUDA(cudaMemcpy2DAsync(r.phi, g.nx * sizeof(double), c->h3.d[0].u, g.px * sizeof(double),
-                                   g.nx * sizeof(double), size_t(g.ny) * g.nz, cudaMemcpyDefault, c->stream));
-    double* outs[5] = {r.Bx, r.By, r.Bz, r.p, r.rho};
-    bool any = false;
-    for (double* o : outs) any = any || o;
-    if (any) {
-        ensure_field_buffers(c);
-        launch_fields(g, c->alpha, c->atm, c->prof, c->h3.d[0].u, c->fld[0], c->fld[1], c->fld[2], c->fld[3],
-                      c->fld[4], (c->opts.flags & MHS_FLAG_BZ_MIMETIC) ? 1 : 0, c->stream);
-        for (int k = 0; k < 5; ++k)
-            if (outs[k])
-                MHS_CUDA(cudaMemcpy2DAsync(outs[k], g.nx * sizeof(double), c->fld[k], g.px * sizeof(double),
-                                           g.nx * sizeof(double), size_t(g.ny) * g.nz, cudaMemcpyDefault,
-                                           c->stream));
+    if (r.phi) {
+        const size_t rows = size_t(g.ny) * g.nz;
+        if (is_device_ptr(r.phi))
+            launch_pack(c->h3.d[0].u, r.phi, g.nx, g.px, rows, c->stream);
+        else
+            MHS_CUDA(cudaMemcpy2DAsync(r.phi, g.nx * sizeof(double), c->h3.d[0].u, g.px * sizeof(double),
+                                       g.nx * sizeof(double), rows, cudaMemcpyDeviceToHost, c->stream));
     }
+    double* const outs[5] = {r.Bx, r.By, r.Bz, r.p, r.rho};
+    if (r.Bx || r.By || r.Bz || r.p || r.rho) recover_fields(c, outs);
     if (!q->done_ev) MHS_CUDA(cudaEventCreateWithFlags(&q->done_ev, cudaEventDisableTiming));
     MHS_CUDA(cudaEventRecord(q->done_ev, c->stream));
 }

@@ -910,14 +910,79 @@ mhs_status batch_solve(mhs_ctx** hs, int n, double tol, int mode, mhs_solve_info
     return worst;
 }
 
-void ensure_field_buffers(mhs_ctx* c) {
-    if (c->fld[0]) return;
-    for (int q = 0; q < 5; ++q) c->fld[q] = static_cast<double*>(dev_alloc(c, c->h3.g[0].n * sizeof(double)));
+bool is_device_ptr(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-void ensure_post_buffers(mhs_ctx* c) {
-    if (c->post[0]) return;
-    for (int q = 0; q < 5; ++q) c->post[q] = static_cast<double*>(dev_alloc(c, c->h3.g[0].n * sizeof(double)));
+static size_t dense_bytes(const mhs_ctx* c) { return size_t(c->nx) * c->ny * c->nz * sizeof(double); }
+
+// Where the kernels write five dense result arrays: the caller's array when
+// it is device memory, overlaps none of the others and is needed by nobody
+// else, the handle's own (allocated on first use) otherwise.
+static void result_targets(mhs_ctx* c, double* const outs[5], double* own[5], const bool need[5], double* to[5]) {
+    const uintptr_t bytes = dense_bytes(c);
+    bool apart = true;
+    for (int q = 0; q < 5; ++q)
+        for (int r = 0; r < q; ++r)
+            if (outs[q] && outs[r]) {
+                const uintptr_t a = reinterpret_cast<uintptr_t>(outs[q]), b = reinterpret_cast<uintptr_t>(outs[r]);
+                apart = apart && (a + bytes <= b || b + bytes <= a);
+            }
+    for (int q = 0; q < 5; ++q) {
+        to[q] = nullptr;
+        if (!outs[q] && !need[q]) continue;
+        if (outs[q] && apart && is_device_ptr(outs[q])) {
+            to[q] = outs[q];
+            continue;
+        }
+        if (!own[q]) own[q] = static_cast<double*>(dev_alloc(c, dense_bytes(c)));
+        to[q] = own[q];
+    }
+}
+
+// the handle's arrays to the callers' (host memory, or overlapping device arrays)
+static void deliver(mhs_ctx* c, double* const outs[5], double* const from[5]) {
+    for (int q = 0; q < 5; ++q)
+        if (outs[q] && outs[q] != from[q])
+            MHS_CUDA(cudaMemcpyAsync(outs[q], from[q], dense_bytes(c), cudaMemcpyDefault, c->stream));
+}
+
+// B, p and rho of the resident P into outs (NULL entries skipped); B always
+// has a place, as rho, currents and field lines read it (to, five entries)
+static void fields_to(mhs_ctx* c, double* const outs[5], double* to[5]) {
+    const bool need[5] = {true, true, true, false, false};
+    result_targets(c, outs, c->fld, need, to);
+    const double nodes = double(c->nx) * c->ny * c->nz;
+    TimedScope t(c->timer, MHS_KT_FIELDS, 48.0 * nodes, 60.0 * nodes, c->stream);
+    launch_fields(c->h3.g[0], c->alpha, c->prof, c->h3.d[0].u, to[0], to[1], to[2], to[3], to[4],
+                  (c->opts.flags & MHS_FLAG_BZ_MIMETIC) ? 1 : 0, c->stream);
+}
+
+void recover_fields(mhs_ctx* c, double* const outs[5]) {
+    double* to[5];
+    fields_to(c, outs, to);
+    deliver(c, outs, to);
+}
+
+void recover_b(mhs_ctx* c) {
+    double* none[5] = {};
+    double* to[5];
+    fields_to(c, none, to);
+}
+
+void recover_current(mhs_ctx* c, double* const outs[5]) {
+    recover_b(c);
+    const bool need[5] = {};
+    double* to[5];
+    result_targets(c, outs, c->post, need, to);
+    launch_current(c->h3.g[0], c->atm.mu0, c->fld[0], c->fld[1], c->fld[2], to[0], to[1], to[2], to[3], to[4],
+                   c->stream);
+    deliver(c, outs, to);
 }
 
 void ensure_staging(mhs_ctx* c) {
@@ -967,7 +1032,8 @@ size_t handle_bytes_estimate(int nx, int ny, int nz, double Lx, double Ly, doubl
 // recovery allocates.
 size_t handle_bytes_held(const mhs_ctx* c) {
     size_t b = c->dev_bytes;
-    if (!c->fld[0]) b += 5 * round_up(c->h3.g[0].n * sizeof(double), 256);
+    for (const double* f : c->fld)
+        if (!f) b += round_up(dense_bytes(c), 256);
     return b;
 }
 

@@ -58,8 +58,13 @@ void vcycle(mhs_ctx* c, Hierarchy& H, int l);
 template <typename T>
 void smooth_hook(mhs_ctx* c, Hierarchy& H, int l);   // one sweep as the V-cycle runs it
 double read_norm2(mhs_ctx* c, int slot);
-void ensure_field_buffers(mhs_ctx* c);
-void ensure_post_buffers(mhs_ctx* c);
+bool is_device_ptr(const void* p);
+// field recovery of the resident P into dense host or device arrays (B_x, B_y, B_z, p, rho; NULL
+// entries skipped), ordered on c->stream; recover_b: B alone, into the handle's c->fld
+void recover_fields(mhs_ctx* c, double* const outs[5]);
+void recover_b(mhs_ctx* c);
+// j_x, j_y, j_z, |j|, |B| likewise, from B recovered into c->fld
+void recover_current(mhs_ctx* c, double* const outs[5]);
 // separable solver (kernels_sep.cu)
 bool sep_level_ok(const Geom& g);   // sine transforms fast (nx - 1, ny - 1 powers of two) or short (nx, ny <= 66)
 template <typename T>

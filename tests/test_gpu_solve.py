@@ -532,3 +532,38 @@ def test_captured_solves_cached_per_option_set(M):
             assert np.array_equal(pa, pb), o
             assert ia["cycles_3d"] == ib["cycles_3d"] and ia["rel_res_3d"] == ib["rel_res_3d"], o
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(35, 43, 21), (33, 9, 5), (67, 11, 37), (5, 5, 5)])
+def test_fields_destinations(M, shape):
+    """B, p and rho written straight into device arrays, copied to host arrays,
+    asked for one at a time and asked for into overlapping device arrays are
+    the same values, and the oracle's to 1e-11 of each field's largest value
+    (tiles of 32 x 8 columns and chunks of planes with ragged ends)."""
+    import torch
+    nx, ny, nz = shape
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=0.7, Lz=0.4, alpha=0.3, xi_kind=1, xi_a=0.5, xi_kappa=1.0)
+    h = M.mhs_create(nx, ny, nz, 1.0, 0.7, 0.4, 0.3, M.xi_params(M.MHS_XI_EXP, 0.5, 1.0))
+    M.mhs_set_stream(h, torch.cuda.current_stream())
+    M.mhs_set_lower_bz(h, S.magnetogram_random(nx, ny, 1.0, 0.7, seed=4))
+    M.mhs_solve(h, 1e-11, M.MHS_FP64)
+    phi = np.zeros((nz, ny, nx))
+    M.mhs_get_phi(h, phi)
+    dev = [torch.full((nz, ny, nx), -1.0, dtype=torch.float64, device="cuda") for _ in range(5)]
+    M.mhs_fields(h, *dev)
+    host = [np.zeros((nz, ny, nx)) for _ in range(5)]
+    M.mhs_fields(h, *host)
+    want = oracle.fields(pr, phi)
+    for q, key in enumerate(("Bx", "By", "Bz", "p", "rho")):
+        assert np.array_equal(dev[q].cpu().numpy(), host[q]), key
+        assert np.abs(host[q] - want[key]).max() <= 1e-11 * np.abs(want[key]).max(), key
+        one = [None] * 5
+        one[q] = torch.zeros((nz, ny, nx), dtype=torch.float64, device="cuda")
+        M.mhs_fields(h, *one)
+        assert torch.equal(one[q], dev[q]), key
+    # arrays that overlap: delivered in order, the later one over the earlier
+    n = nx * ny * nz
+    pool = torch.zeros(n + n // 2, dtype=torch.float64, device="cuda")
+    M.mhs_fields(h, pool[:n], None, None, None, pool[n // 2:n // 2 + n])
+    assert torch.equal(pool[n // 2:n // 2 + n], dev[4].flatten()) and torch.equal(pool[:n // 2], dev[0].flatten()[:n // 2])
+    M.mhs_destroy(h)
