@@ -124,6 +124,7 @@ struct Hierarchy {
     DFState df;                           // finest-level double-float state (mixed mode)
     // TMA plane maps of the FP32 arrays u, t, f per level (3D levels; see kernels_tma.cu)
     std::vector<CUtensorMap> tm_u, tm_t, tm_f;   // index 2 l + (tiles of 16 rows)
+    std::vector<CUtensorMap> tp_u, tp_t, tp_f;   // per level: boxes of the paired sweeps (kernels_pair.cu)
     int nlev() const { return int(g.size()); }
 };
 
@@ -406,6 +407,12 @@ void launch_trace(int nx, int ny, int nz, double Lx, double Ly, double Lz, size_
 void make_plane_map(CUtensorMap* map, const Geom& g, const float* base, int rows);
 void launch_sweep_tma(const Geom& g, int rows, const CUtensorMap& tm_in, const CUtensorMap& tm_f,
                       const PlaneCoef<float>* coef, float* uout, int* err, cudaStream_t st);
+
+// ---- two red-black sweeps in one pass, FP32 3D levels (kernels_pair.cu) ----
+bool pair_level(const Geom& g);   // the levels whose pairs of sweeps run it
+void make_pair_map(CUtensorMap* map, const Geom& g, const float* base);
+void launch_pair_sweep(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap& tm_f,
+                       const PlaneCoef<float>* coef, float* uout, int* err, cudaStream_t st);
 
 // ---- control and sub-cycle (kernels_ctl.cu) ----
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st);

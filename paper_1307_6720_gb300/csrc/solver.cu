@@ -114,6 +114,14 @@ static void build_hierarchy(mhs_ctx* c, Hierarchy& H, int dim) {
                 make_plane_map(&H.tm_t[2 * l + r], H.g[l], H.s[l].t, 8 << r);
                 make_plane_map(&H.tm_f[2 * l + r], H.g[l], H.s[l].f, 8 << r);
             }
+        H.tp_u.resize(H.g.size());
+        H.tp_t.resize(H.g.size());
+        H.tp_f.resize(H.g.size());
+        for (size_t l = 0; l < H.g.size(); ++l) {
+            make_pair_map(&H.tp_u[l], H.g[l], H.s[l].u);
+            make_pair_map(&H.tp_t[l], H.g[l], H.s[l].t);
+            make_pair_map(&H.tp_f[l], H.g[l], H.s[l].f);
+        }
     }
     const Geom& g0 = H.g[0];
     H.df.hi = static_cast<float*>(dev_alloc(c, g0.n * sizeof(float)));
@@ -297,6 +305,47 @@ static void smooth_n(mhs_ctx* c, Hierarchy& H, int l, const T* f, int n, bool fi
     if (fused && (n & 1)) MHS_CUDA(cudaMemcpyAsync(A.u, A.t, g.n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
 }
 
+// Passes of two sweeps (kernels_pair.cu) that a V-cycle runs on level l
+// before and after its coarse-grid correction: FP32 3D levels large enough,
+// red-black smoothing.  A pass moves the iterate from u to its twin t or
+// back, so their sum is even and the cycle ends in u; sweeps left over run in
+// place.
+struct PairPasses {
+    int pre = 0, post = 0;
+};
+template <typename T>
+static PairPasses pair_passes(const mhs_ctx* c, const Hierarchy& H, int l) {
+    PairPasses p;
+    if (sizeof(T) == 8 || H.dim != 3 || use_zline(c) || (c->opts.flags & MHS_FLAG_NO_TMA) || !pair_level(H.g[l]))
+        return p;
+    p.pre = c->opts.nu1 / 2;
+    p.post = c->opts.nu2 / 2;
+    if ((p.pre + p.post) & 1) --(p.post > 0 ? p.post : p.pre);
+    return p;
+}
+
+// n sweeps of level l in a V-cycle, `passes` pairs of them out of place;
+// in_t: the iterate is in the twin (both ways)
+template <typename T>
+static void smooth_level(mhs_ctx* c, Hierarchy& H, int l, const T* f, int n, int passes, bool paired, bool& in_t,
+                         bool fine, double bytes, double flops) {
+    if (!paired) {
+        smooth_n<T>(c, H, l, f, n, fine, bytes, flops);
+        return;
+    }
+    LevelArrays<float>& A = H.s[l];
+    for (int q = 0; q < passes; ++q) {
+        TimedScope t(c->timer, MHS_KT_SMOOTH32, bytes, 2.0 * flops, c->stream, fine);
+        launch_pair_sweep(H.g[l], in_t ? H.tp_t[l] : H.tp_u[l], H.tp_f[l], A.coef, in_t ? A.u : A.t, c->flag + 1,
+                          c->stream);
+        in_t = !in_t;
+    }
+    for (int q = 2 * passes; q < n; ++q) {
+        TimedScope t(c->timer, MHS_KT_SMOOTH32, bytes, flops, c->stream, fine);
+        launch_smooth<float>(H.g[l], H.dim, A.coef, in_t ? A.t : A.u, A.f, c->stream, c->opts.tile);
+    }
+}
+
 // Per-level accounting and right-hand side of the V-cycle's operations on
 // level l: f vanishes on the finest FP64 interior level (the Dirichlet data
 // sits in u); algorithmic flops per node: the update u = f/d - ax(E+W) -
@@ -325,10 +374,10 @@ struct LevelOps {
 // the coarse-grid correction of level l from its residual: restriction of
 // the residual in A.r (unless the fused pass of FP32 levels has already
 // restricted it; red: A.r is a residual taken on red nodes only), the coarser
-// cycle, interpolation added to u
+// cycle, interpolation added to u (or to its twin, where the iterate then is)
 template <typename T>
 static void coarse_correction(mhs_ctx* c, Hierarchy& H, int l, const LevelOps<T>& o, bool restricted,
-                              bool red = false) {
+                              bool red = false, bool in_t = false) {
     cudaStream_t st = c->stream;
     const bool dbl = sizeof(T) == 8;
     LevelArrays<T>& A = arrays<T>(H, l);
@@ -342,7 +391,7 @@ static void coarse_correction(mhs_ctx* c, Hierarchy& H, int l, const LevelOps<T>
     vcycle<T>(c, H, l + 1);
     {
         TimedScope t(c->timer, dbl ? MHS_KT_PROLONG64 : MHS_KT_PROLONG32, (2 * N + Nc) * s, 4.0 * N, st, o.fine);
-        launch_prolong<T>(H.g[l + 1], H.g[l], H.dim, C.u, A.u, st);
+        launch_prolong<T>(H.g[l + 1], H.g[l], H.dim, C.u, in_t ? A.t : A.u, st);
     }
 }
 
@@ -376,7 +425,10 @@ void vcycle(mhs_ctx* c, Hierarchy& H, int l) {
     const bool dbl = sizeof(T) == 8;
     const LevelOps<T> o(c, H, l);
     const double sweep_bytes = o.N * (2 * o.s + o.fs);
-    smooth_n<T>(c, H, l, o.f, c->opts.nu1, o.fine, sweep_bytes, o.N * o.upd_flops);
+    const PairPasses pp = pair_passes<T>(c, H, l);
+    const bool paired = pp.pre + pp.post > 0;
+    bool in_t = false;
+    smooth_level<T>(c, H, l, o.f, c->opts.nu1, pp.pre, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops);
     if (!dbl) {
         // FP32 levels (bandwidth-bound): residual and restriction in one pass, the residual not
         // stored (u and f read, the coarse right-hand side and iterate written; flops of the
@@ -385,15 +437,15 @@ void vcycle(mhs_ctx* c, Hierarchy& H, int l) {
         const double Nc = double(H.g[l + 1].interior());
         TimedScope t(c->timer, MHS_KT_RESID32, o.N * (o.s + o.fs) + 2 * Nc * o.s,
                      o.N * o.res_flops + Nc * (H.dim == 3 ? 54.0 : 18.0), st, o.fine);
-        launch_resid_restrict<T>(g, H.g[l + 1], H.dim, A.coef, A.u, o.f, C.f, C.u, st);
+        launch_resid_restrict<T>(g, H.g[l + 1], H.dim, A.coef, in_t ? A.t : A.u, o.f, C.f, C.u, st);
     } else {
         // FP64 levels (bound by the FP64 pipe, which the fused pass would not relieve): the
         // residual on red nodes after the sweep, then the restriction
         TimedScope t(c->timer, MHS_KT_RESID64, sweep_bytes, o.N * o.res_flops, st, o.fine);
         launch_residual<T>(g, H.dim, A.coef, A.u, o.f, A.r, nullptr, 0, st, red_residual_level(c, H));
     }
-    coarse_correction<T>(c, H, l, o, !dbl, dbl && red_residual_level(c, H));
-    smooth_n<T>(c, H, l, o.f, c->opts.nu2, o.fine, sweep_bytes, o.N * o.upd_flops);
+    coarse_correction<T>(c, H, l, o, !dbl, dbl && red_residual_level(c, H), in_t);
+    smooth_level<T>(c, H, l, o.f, c->opts.nu2, pp.post, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops);
 }
 
 // FP64 cycles of the finest level with the convergence test after the

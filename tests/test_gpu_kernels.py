@@ -627,3 +627,25 @@ def test_dense_transform_tiles(M, shape, prec):
     want = exact.separable_solve3d(_level_problem(M, h, pr, 3, 0), np.zeros((ny, nx)), f)
     assert _rel(got, want) < (1e-12 if prec == 0 else 2e-5)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (4, 2), (3, 3), (2, 1)])
+@pytest.mark.parametrize("shape", [(129, 129, 65), (193, 97, 49), (249, 129, 33), (129, 33, 257)])
+def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
+    """FP32 V-cycles whose pairs of sweeps run as one out-of-place pass (tiles
+    in x, y and z with ragged ends, boundary values that are not zero, odd
+    sweeps left over) equal the cycles run colour by colour bit for bit."""
+    nx, ny, nz = shape
+    pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
+    rng = np.random.default_rng(nx + nz)
+    u, f = rng.standard_normal((2, nz, ny, nx)).astype(np.float32).astype(np.float64)
+    got = []
+    for flags in (0, M.MHS_FLAG_NO_TMA):
+        M.mhs_set_options(h, nu1=nu[0], nu2=nu[1], flags=flags, fused_min=1 << 30)
+        M.mhs_level_write(h, 3, 0, M.MHS_FIELD_U, 1, u)
+        M.mhs_level_write(h, 3, 0, M.MHS_FIELD_F, 1, f)
+        M.mhs_level_op(h, 3, 0, M.MHS_OP_VCYCLE, 1)
+        got.append(_read(M, h, 3, 0, M.MHS_FIELD_U, 1))
+    assert np.array_equal(got[0], got[1])
+    assert not np.array_equal(got[0], u)
+    M.mhs_destroy(h)
