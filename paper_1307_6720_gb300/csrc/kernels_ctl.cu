@@ -16,8 +16,9 @@ __global__ void bnorm_kernel(const double* __restrict__ partial, int n, SolveCtl
 }
 
 __global__ void check_kernel(const double* __restrict__ partial, int n, SolveCtl* ctl, int first,
-                             cudaGraphConditionalHandle handle, int use_handle) {
+                             cudaGraphConditionalHandle handle, int use_handle, int flips) {
     const int cont = check_body(partial, n, ctl, first);
+    if (threadIdx.x == 0 && flips) ctl->flip ^= 1;
     if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, cont);
 }
 
@@ -35,8 +36,8 @@ void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st) 
 }
 
 void launch_check(const double* partial, int n, SolveCtl* ctl, int first, cudaGraphConditionalHandle handle,
-                  int use_handle, cudaStream_t st) {
-    check_kernel<<<1, 1024, 0, st>>>(partial, n, ctl, first, handle, use_handle);
+                  int use_handle, cudaStream_t st, bool flips) {
+    check_kernel<<<1, 1024, 0, st>>>(partial, n, ctl, first, handle, use_handle, flips ? 1 : 0);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
 }

@@ -200,6 +200,17 @@ __global__ void g_df_residual_kernel(const GItem* items, int n, int gate) {
     GBlock k;
     if (!locate(items, n, gate, -1, -1, k)) return;
     const GItem& it = *k.it;
+    if (D3 && use_df_quads(it.g)) {
+        auto run = [&](auto march) {
+            march(it.g, static_cast<const PlaneCoefDF*>(it.coef), nullptr, static_cast<const float*>(it.p[0]),
+                  static_cast<const float*>(it.p[1]), nullptr, nullptr, static_cast<const float*>(it.p[2]),
+                  static_cast<const float*>(it.p[3]), static_cast<float*>(it.p[4]), static_cast<double*>(it.p[5]), k.b,
+                  k.gd);
+        };
+        if (it.p[2] && it.p[3]) run([](auto&&... a) { df_march_body<false, false>(a...); });
+        else run([](auto&&... a) { df_march_body<false, true>(a...); });
+        return;
+    }
     df_residual_body<D3>(it.g, static_cast<const PlaneCoefDF*>(it.coef), static_cast<const float*>(it.p[0]),
                          static_cast<const float*>(it.p[1]), static_cast<const float*>(it.p[2]),
                          static_cast<const float*>(it.p[3]), static_cast<float*>(it.p[4]),
@@ -380,7 +391,8 @@ void glaunch_df_copy_plane(const GTable& t, cudaStream_t st) {
 
 void glaunch_df_residual(const GTable& t, int d3, int gate, cudaStream_t st) {
     if (!t.n) return;
-    if (d3) g_df_residual_kernel<true><<<t.blocks, kDF, 0, st>>>(t.items, t.n, gate);
+    // the block shape of the quad form; narrow items leave its last rows of threads idle
+    if (d3) g_df_residual_kernel<true><<<t.blocks, dim3(DQ_X, DQ_ROWS), 0, st>>>(t.items, t.n, gate);
     else g_df_residual_kernel<false><<<t.blocks, kDF, 0, st>>>(t.items, t.n, gate);
     after_launch();
 }

@@ -90,6 +90,10 @@ struct PlaneCoefDF {
 
 // Finest-level state of mixed mode: the outer iterate P = hi + lo and the
 // right-hand side f = fh + fl as double-float pairs (FP32 words).
+// The solo solve corrects the iterate out of place, together with the next
+// residual, between (hi, lo) and a second pair held in the level's FP64
+// residual array, which mixed mode does not use; SolveCtl::flip says which
+// pair is current (0: hi, lo).
 struct DFState {
     float *hi = nullptr, *lo = nullptr, *fh = nullptr, *fl = nullptr;
     PlaneCoefDF* coef = nullptr;
@@ -139,6 +143,7 @@ struct SolveCtl {
     int cycles;
     int status;        // MHS_OK or MHS_ERR_NONFINITE
     int cont;          // 1 while another cycle is needed
+    int flip;          // mixed mode: which of the two double-float iterates is current (see DFState)
     int bodies;        // cycles run by a while body (the full-multigrid cycle of the prologue is not one)
 };
 
@@ -205,7 +210,11 @@ struct TimedScope {
     int rec;
     TimedScope(KernelTimer& timer, int k, double b, double f, cudaStream_t s, bool finest = false)
         : t(timer), st(s), rec(timer.begin(k, b, f, s, finest)) {}
-    ~TimedScope() { t.end(rec, st); }
+    ~TimedScope() { stop(); }
+    void stop() {   // ends the record before the scope does
+        t.end(rec, st);
+        rec = -1;
+    }
 };
 
 }  // namespace mhs
@@ -416,8 +425,9 @@ void launch_pair_sweep(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap
 
 // ---- control and sub-cycle (kernels_ctl.cu) ----
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st);
+// flips: the launch before it moved the double-float iterate to the other pair
 void launch_check(const double* partial, int n, SolveCtl* ctl, int first, cudaGraphConditionalHandle handle,
-                  int use_handle, cudaStream_t st);
+                  int use_handle, cudaStream_t st, bool flips = false);
 size_t subcycle_smem_limit();
 // rows of 32 threads of the sub-cycle CTA of a hierarchy cut at a level with
 // `interior` interior nodes: small coarse problems pay mostly for block-wide
@@ -435,11 +445,21 @@ void launch_df_split(const Geom& g, int dim, const double* f, float* hi, float* 
 int launch_df_residual(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* hi, const float* lo,
                        const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st);
 // (hi, lo) += e at interior nodes
+// the two double-float iterates and which is current (DFState); flip == nullptr: the first
+struct DFPair {
+    float *hi[2], *lo[2];
+    const int* flip;
+};
 void launch_df_correct(const Geom& g, int dim, const float* e, float* hi, float* lo, cudaStream_t st);
+// the lower boundary, and 3D levels wide enough for the pass: correction and residual in one launch
+bool df_step_available(const Geom& g, int dim);
+// current pair + e into the other pair (faces copied), and its residual as launch_df_residual's
+int launch_df_step(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* e, const DFPair& p, const float* fh,
+                   const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st);
 // P = hi + lo (double) at every node
-void launch_df_to_double(const Geom& g, const float* hi, const float* lo, double* P, cudaStream_t st);
+void launch_df_to_double(const Geom& g, const DFPair& p, double* P, cudaStream_t st);
 // plane k = 0 of a 3D double-float pair from a 2D pair
-void launch_df_copy_plane(const Geom& g2, const float* hi2, const float* lo2, const Geom& g3, float* hi3, float* lo3,
+void launch_df_copy_plane(const Geom& g2, const DFPair& p2, const Geom& g3, float* hi3, float* lo3,
                           cudaStream_t st);
 
 // ---- fields (kernels_fields.cu) ----

@@ -605,6 +605,32 @@ static int residual_partials(mhs_ctx* c, Hierarchy& H, int mode, bool red = fals
                                    c->stream, red);
 }
 
+static DFPair df_pair(mhs_ctx* c, Hierarchy& H) {
+    const size_t n = H.g[0].n;
+    float* second = reinterpret_cast<float*>(H.d[0].r);   // n doubles: two arrays of n words
+    return DFPair{{H.df.hi, second}, {H.df.lo, second + n}, &c->ctl[H.dim == 3 ? 1 : 0].flip};
+}
+
+// mixed mode: the correction added to the double-float iterate and the
+// residual of the result, as residual_partials forms it; returns the partials' count
+static int correct_and_residual(mhs_ctx* c, Hierarchy& H, bool& flips) {
+    const Geom& g = H.g[0];
+    flips = df_step_available(g, H.dim);
+    if (!flips) {
+        TimedScope t(c->timer, MHS_KT_CORRECT, double(g.interior()) * 20.0, double(g.interior()) * 8.0, c->stream,
+                     H.dim == 3);
+        launch_df_correct(g, H.dim, H.s[0].u, H.df.hi, H.df.lo, c->stream);
+        t.stop();
+        return residual_partials(c, H, MHS_MIXED);
+    }
+    const bool fz = H.dim == 3 && c->f_zero_finest;
+    const double N = double(g.interior());
+    TimedScope t(c->timer, MHS_KT_RESID_MIXED, N * (12.0 + 8.0 + (fz ? 0.0 : 8.0) + 4.0), N * 80.0, c->stream,
+                 H.dim == 3);
+    return launch_df_step(g, H.dim, H.df.coef, H.s[0].u, df_pair(c, H), fz ? nullptr : H.df.fh,
+                          fz ? nullptr : H.df.fl, H.s[0].f, c->ns.partial, c->ns.max_blocks, c->stream);
+}
+
 static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
     mhs_ctx* c = e.c;
     const Geom& g = H.g[0];
@@ -617,10 +643,12 @@ static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
         } else {
             for (int q = 0; q < c->opts.inner_cycles; ++q) vcycle<float>(c, H, 0);
         }
-        TimedScope t(c->timer, MHS_KT_CORRECT, double(g.interior()) * 20.0, double(g.interior()) * 8.0, c->stream,
-                     H.dim == 3);
-        launch_df_correct(g, H.dim, H.s[0].u, H.df.hi, H.df.lo, c->stream);
-    } else if ((c->opts.flags & MHS_FLAG_SEPARABLE) && sep_fp64_available(c)) {
+        bool flips;
+        const int nb = correct_and_residual(c, H, flips);
+        launch_check(c->ns.partial, nb, ctl, 0, e.hnd, e.graph ? 1 : 0, c->stream, flips);
+        return;
+    }
+    if ((c->opts.flags & MHS_FLAG_SEPARABLE) && sep_fp64_available(c)) {
         // direct solve of the correction from the residual of the latest check
         const double N = double(g.interior());
         TimedScope t(c->timer, MHS_KT_SEPARABLE, N * 8.0 * 3.0, 0.0, c->stream, H.dim == 3);
@@ -630,7 +658,7 @@ static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
     } else {
         vcycle<double>(c, H, 0);
     }
-    const int nb = residual_partials(c, H, e.mode, e.mode == MHS_FP64 && red_residual_cycle(c, H));
+    const int nb = residual_partials(c, H, e.mode, red_residual_cycle(c, H));
     launch_check(c->ns.partial, nb, ctl, 0, e.hnd, e.graph ? 1 : 0, c->stream);
 }
 
@@ -648,13 +676,13 @@ static void fmg_cycle(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
     if (e.mode == MHS_MIXED) {
         MHS_CUDA(cudaMemsetAsync(H.s[0].u, 0, g.n * sizeof(float), c->stream));
         fmg<float>(c, H, H.s[0].f);
-        TimedScope t(c->timer, MHS_KT_CORRECT, double(g.interior()) * 20.0, double(g.interior()) * 8.0, c->stream,
-                     H.dim == 3);
-        launch_df_correct(g, H.dim, H.s[0].u, H.df.hi, H.df.lo, c->stream);
-    } else {
-        fmg<double>(c, H, H.d[0].r);
+        bool flips;
+        const int nb = correct_and_residual(c, H, flips);
+        launch_check(c->ns.partial, nb, ctl, 2, e.hnd, e.graph ? 1 : 0, c->stream, flips);
+        return;
     }
-    const int nb = residual_partials(c, H, e.mode, e.mode == MHS_FP64 && red_residual_fmg(c, H));
+    fmg<double>(c, H, H.d[0].r);
+    const int nb = residual_partials(c, H, e.mode, red_residual_fmg(c, H));
     launch_check(c->ns.partial, nb, ctl, 2, e.hnd, e.graph ? 1 : 0, c->stream);
 }
 
@@ -703,7 +731,7 @@ static void prologue_3d(const Enq& e) {
             // split of its FP64 solution when that problem ran in FP64 cycles
             if (lower_mode(c, e.mode) != e.mode)
                 launch_df_split(c->h2.g[0], 2, c->h2.d[0].u, c->h2.df.hi, c->h2.df.lo, c->stream);
-            launch_df_copy_plane(c->h2.g[0], c->h2.df.hi, c->h2.df.lo, g, H.df.hi, H.df.lo, c->stream);
+            launch_df_copy_plane(c->h2.g[0], df_pair(c, c->h2), g, H.df.hi, H.df.lo, c->stream);
             if (!c->f_zero_finest) launch_df_split(g, 3, H.d[0].f, H.df.fh, H.df.fl, c->stream);
         }
         // twins of the levels swept out of place: u's boundary faces (level 0: the Dirichlet data)
@@ -724,7 +752,7 @@ static void prologue_3d(const Enq& e) {
 static void epilogue(const Enq& e, Hierarchy& H) {
     if (e.mode != MHS_MIXED) return;
     TimedScope t(e.c->timer, MHS_KT_OTHER, 0.0, 0.0, e.c->stream);
-    launch_df_to_double(H.g[0], H.df.hi, H.df.lo, H.d[0].u, e.c->stream);
+    launch_df_to_double(H.g[0], df_pair(e.c, H), H.d[0].u, e.c->stream);
 }
 
 // Append a while node to the graph being captured on c->stream whose body

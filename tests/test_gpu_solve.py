@@ -567,3 +567,34 @@ def test_fields_destinations(M, shape):
     M.mhs_fields(h, pool[:n], None, None, None, pool[n // 2:n // 2 + n])
     assert torch.equal(pool[n // 2:n // 2 + n], dev[4].flatten()) and torch.equal(pool[:n // 2], dev[0].flatten()[:n // 2])
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(97, 33, 17), (95, 33, 17), (107, 19, 11), (261, 13, 9), (129, 9, 33)])
+def test_mixed_step_on_wide_levels(M, shape):
+    """Mixed mode on grids around the width from which correction and residual
+    run as one pass over quads (ragged quads, one and several tiles along x):
+    the solution meets the mixed bar against the exact one, and a group, which
+    corrects in place and takes the residual by itself, is bitwise equal."""
+    import torch
+    nx, ny, nz = shape
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=(ny - 1) / (nx - 1), Lz=(nz - 1) / (nx - 1), alpha=0.3, xi_kind=1, xi_a=0.5,
+                   xi_kappa=1.0)
+    bz = S.magnetogram_random(nx, ny, 1.0, pr["Ly"], seed=nx)
+    h = M.mhs_create(nx, ny, nz, pr["Lx"], pr["Ly"], pr["Lz"], pr["alpha"], _xi(M, pr))
+    M.mhs_set_stream(h, torch.cuda.current_stream())
+    M.mhs_set_lower_bz(h, bz)
+    info = M.mhs_solve(h, 1e-11, M.MHS_MIXED)
+    P = np.zeros((nz, ny, nx))
+    M.mhs_get_phi(h, P)
+    assert rel(P, exact.exact_solution(pr, bz)) < 1e-8, info
+    h2 = M.mhs_create(17, 17, 17, 1.0, 1.0, 1.0, 0.2)
+    M.mhs_set_lower_bz(h2, S.magnetogram_random(17, 17, seed=1))
+    g = M.mhs_group_create([h, h2], M.MHS_MIXED, part_bytes=(1 << 64) - 1)
+    infos, sts = M.mhs_group_solve(g, 2, 1e-11)
+    got = np.zeros((nz, ny, nx))
+    M.mhs_get_phi(h, got)
+    assert sts == [0, 0] and np.array_equal(got, P)
+    assert infos[0]["rel_res_3d"] == info["rel_res_3d"] and infos[0]["cycles_3d"] == info["cycles_3d"]
+    M.mhs_group_destroy(g)
+    M.mhs_destroy(h2)
+    M.mhs_destroy(h)
