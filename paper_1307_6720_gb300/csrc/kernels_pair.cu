@@ -77,6 +77,11 @@ struct PairTile {
     bool last;              // this thread owns that quad
 };
 
+// Planes in registers: [slot][row][p] holds the quad's nodes p and p + 2, the
+// pair that one colour updates, so that every operation of an update is one
+// packed FP32 instruction and a published pair is a register pair.
+typedef float2 PairRegs[6][2][2];
+
 // The values outside the thread that an update of colour COL of the plane in
 // register slot S reads: per row the pair the neighbouring row published and
 // the x neighbour outside the quad (west of node 0 or east of node 3).  All
@@ -86,15 +91,15 @@ struct PairOuter {
     float x[2];
 };
 template <int NW, int S, int COL>
-__device__ __forceinline__ void pair_gather(PairOuter& o, const float (&U)[6][2][4], const PairTile& t,
-                                            const float2* pub, const float* east) {
+__device__ __forceinline__ void pair_gather(PairOuter& o, const PairRegs& U, const PairTile& t, const float2* pub,
+                                            const float* east) {
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         o.y[r] = pub[r == 0 ? t.lo : t.hi];
         if (((r + S + COL) & 1) == 0) {
-            o.x[r] = __shfl_up_sync(0xffffffffu, U[S][r][3], 1);
+            o.x[r] = __shfl_up_sync(0xffffffffu, U[S][r][1].y, 1);
         } else {
-            o.x[r] = __shfl_down_sync(0xffffffffu, U[S][r][0], 1);
+            o.x[r] = __shfl_down_sync(0xffffffffu, U[S][r][0].x, 1);
             if (t.east && t.last) o.x[r] = east[S * 2 * NW + r];
         }
     }
@@ -104,27 +109,25 @@ __device__ __forceinline__ void pair_gather(PairOuter& o, const float (&U)[6][2]
 // are published to `out` unless this is the plane's last update.
 // c = (1/d, -az, -ay, -ax); F holds f/d.
 template <int S, int COL, bool LAST>
-__device__ __forceinline__ void pair_update(float (&U)[6][2][4], const float (&F)[6][2][4], const PairTile& t,
-                                            const float4 c, const PairOuter& o, float2* out) {
-    constexpr int P = S & 1, UP = (S + 1) % 6, DN = (S + 5) % 6;
+__device__ __forceinline__ void pair_update(PairRegs& U, const PairRegs& F, const PairTile& t, const float4 c,
+                                            const PairOuter& o, float2* out) {
+    constexpr int UP = (S + 1) % 6, DN = (S + 5) % 6;
+    const float2 cz = make_float2(c.y, c.y), cy = make_float2(c.z, c.z), cx = make_float2(c.w, c.w);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int s = (r + P + COL) & 1;   // the colour's nodes: s and s + 2
+        const int s = (r + S + COL) & 1;   // the colour's nodes: s and s + 2
         if (t.rk[r]) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int q = s + 2 * h;
-                const float w = q == 0 ? o.x[r] : U[S][r][q == 0 ? 0 : q - 1];
-                const float e = q == 3 ? o.x[r] : U[S][r][q == 3 ? 3 : q + 1];
-                float v = fmaf(c.y, U[UP][r][q] + U[DN][r][q], F[S][r][q]);
-                v = fmaf(c.z, (h ? o.y[r].y : o.y[r].x) + U[S][1 - r][q], v);
-                v = fmaf(c.w, e + w, v);
-                if (q == 0) v = t.k0 ? v : U[S][r][q];
-                U[S][r][q] = v;
-            }
+            // x neighbours: (west, node 1) and (1, 3) of nodes (0, 2); (0, 2) and (node 2, east) of (1, 3)
+            const float2 ew = s == 0 ? __fadd2_rn(U[S][r][1], make_float2(o.x[r], U[S][r][1].x))
+                                     : __fadd2_rn(make_float2(U[S][r][0].y, o.x[r]), U[S][r][0]);
+            float2 v = __ffma2_rn(cz, __fadd2_rn(U[UP][r][s], U[DN][r][s]), F[S][r][s]);
+            v = __ffma2_rn(cy, __fadd2_rn(o.y[r], U[S][1 - r][s]), v);
+            v = __ffma2_rn(cx, ew, v);
+            if (s == 0) v.x = t.k0 ? v.x : U[S][r][0].x;
+            U[S][r][s] = v;
         }
         // a face row publishes its fixed values
-        if (!LAST) out[t.own + r * 32] = make_float2(U[S][r][s], U[S][r][s + 2]);
+        if (!LAST) out[t.own + r * 32] = U[S][r][s];
     }
 }
 
@@ -201,7 +204,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     }
     __syncthreads();
 
-    float U[6][2][4] = {}, F[6][2][4] = {};
+    PairRegs U = {}, F = {};
     float* out = uout + (size_t(x) + size_t(g.px) * size_t(j0) + g.plane * size_t(ka));   // plane ka of the quad
     const float* su = s_u + row * PBW + 4 * lane;
     const float* sf = s_f + row * PBW + 4 * lane;
@@ -224,9 +227,9 @@ __global__ void __launch_bounds__(32 * NW, 1)
             const float* a = su + (S % NS) * S_::SLOT;                                                                \
             _Pragma("unroll") for (int r = 0; r < 2; ++r) {                                                           \
                 const float4 v = *reinterpret_cast<const float4*>(a + r * PBW);                                       \
-                U[S][r][0] = v.x, U[S][r][1] = v.y, U[S][r][2] = v.z, U[S][r][3] = v.w;                               \
-                const int b = (r + S + 1) & 1; /* the row's black nodes: b and b + 2 */                               \
-                pout[t.own + r * 32] = make_float2(U[S][r][b], U[S][r][b + 2]);                                       \
+                U[S][r][0] = make_float2(v.x, v.z), U[S][r][1] = make_float2(v.y, v.w);                                 \
+                const int b = (r + S + 1) & 1; /* the row's black pair */                                          \
+                pout[t.own + r * 32] = U[S][r][b];                                                                    \
                 if (t.east && t.last) se[S * H + r] = a[r * PBW + 4];                                                 \
             }                                                                                                         \
         }                                                                                                             \
@@ -236,7 +239,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
             const float4 c = cp[S - 1];                                                                               \
             _Pragma("unroll") for (int r = 0; r < 2; ++r) {                                                           \
                 const float4 v = *reinterpret_cast<const float4*>(a + r * PBW);                                       \
-                F[Z][r][0] = v.x * c.x, F[Z][r][1] = v.y * c.x, F[Z][r][2] = v.z * c.x, F[Z][r][3] = v.w * c.x;       \
+                F[Z][r][0] = __fmul2_rn(make_float2(v.x, v.z), make_float2(c.x, c.x));                                \
+                F[Z][r][1] = __fmul2_rn(make_float2(v.y, v.w), make_float2(c.x, c.x));                                \
             }                                                                                                         \
             pair_update<Z, 0, false>(U, F, t, c, o0, pout + S_::PUB);                                             \
         }                                                                                                             \
@@ -253,7 +257,8 @@ __global__ void __launch_bounds__(32 * NW, 1)
             _Pragma("unroll") for (int r = 0; r < 2; ++r) {                                                           \
                 if (yok[r]) {                                                                                         \
                     float* o = out + size_t(r) * g.px;                                                                \
-                    *reinterpret_cast<float4*>(o) = make_float4(U[Z][r][0], U[Z][r][1], U[Z][r][2], U[Z][r][3]);      \
+                    *reinterpret_cast<float4*>(o) =                                                                   \
+                        make_float4(U[Z][r][0].x, U[Z][r][1].x, U[Z][r][0].y, U[Z][r][1].y);                          \
                     if (t.east && t.last) o[4] = se[Z * H + r];                                                       \
                 }                                                                                                     \
             }                                                                                                         \
