@@ -14,13 +14,18 @@
 // and the lower-boundary problem (eq. lower_bound) into a division per mode.
 // Every multigrid level is a rediscretisation with the same structure, so
 // the same solver applies on any level.  The sine transforms are fast
-// transforms (kernels_dst.cu) when nx - 1 and ny - 1 are powers of two, else
-// dense products with the (symmetric) sine matrices done as batched GEMMs over
-// the planes; the inverse is the same transform scaled by
-// (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
+// transforms (kernels_dst.cu) on large planes whose nx - 1 and ny - 1 are powers
+// of two, dense products with folded sine matrices, both transforms of a plane
+// in one launch, on planes of at most 128 cells a side (plane_body), and
+// batched GEMMs with the (symmetric) sine matrices otherwise; the inverse is
+// the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
 // relative, which the double-float outer loop of mixed mode then corrects.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
 #include <vector>
 
 #include "device_util.cuh"
@@ -127,6 +132,333 @@ template <typename T>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs<T> g) {
     gemm_body(g, int(blockIdx.x), int(blockIdx.y), int(blockIdx.z));
 }
+
+// Both sine transforms of a plane as dense products with folded matrices.
+//
+// With M elements (M + 1 = N), s_i = x_i + x_{N-i} and d_i = x_i - x_{N-i}, the
+// odd results need only the s_i (and the middle element when N is even), the
+// even ones only the d_i: two matrices of half the side, Ko = ceil(M/2) and
+// Ke = floor(M/2), half the products.  A block takes sp odd and sp even results
+// b of the first transform (along the lines) for all A lines, and transforms
+// those along the lines' index: no other block's data is needed, so a plane is
+// one launch without clusters or exchanges, and every block loads the whole
+// plane (from L2).  The sums run in blocks of eight (one FMA chain each), whose
+// sums are added in order: a rounding error that grows with the number of
+// blocks rather than of terms, no larger than the fast transforms'.
+//
+// Fast transforms need fewer operations, but on the planes of coarse levels
+// they are a chain of short barrier-separated steps.  Per launch, forward or
+// inverse: FP32 65^3 9.6 us (fast transforms 14), 33^3 6.9 (8.3), FP64 17^3 5.9
+// (14); the 65^2 lower-boundary solve in one cluster 22.6 us in FP64 (31); as
+// stages of ragged 49 x 41 planes 14 us instead of two products of 9.5.  Whole
+// mixed solves with fields 1.25 -> 1.17 ms (129^3), FP64 33^3 1.01 -> 0.88 ms.
+// Errors against the exact solution, random and smooth right-hand sides, 17^3
+// to 129 x 129 x 17: FP32 1.0e-7 .. 2.4e-7 (fast transforms 1.0e-7 .. 2.8e-7).
+// FP32: four results per thread share each loaded element (R = 4).  FP64 is
+// bound by its pipe, so one result per thread spreads a plane furthest.
+constexpr int PLANE_T = 256;
+
+// shared memory of plane_body (elements; every part a multiple of four)
+template <typename T>
+struct PlaneLayout {
+    int s1, g, x, total;   // offsets after the matrix of the second transform
+    __host__ __device__ PlaneLayout(int A, int M1, int sp) {
+        const int Ko2 = (A + 1) / 2, Ke2 = A / 2;
+        auto up = [](int n) { return (n + 3) / 4 * 4; };
+        s1 = up(Ko2 * Ko2 + Ke2 * Ke2);
+        g = s1 + up(M1 * sp);
+        x = g + up(A * 2 * sp);
+        total = x + up(M1 * (A | 1));
+    }
+};
+
+// blocked dot products: out[q] = sum over i < K of m(i)[q] x(i)
+template <typename T, int R, typename FX, typename FM>
+__device__ __forceinline__ void plane_dot(int K, FX&& x, FM&& m, T (&tot)[R]) {
+#pragma unroll
+    for (int q = 0; q < R; ++q) tot[q] = T(0);
+    int i = 0;
+    for (; i + 8 <= K; i += 8) {
+        T p[R] = {};
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const T xv = x(i + u);
+            T mv[R];
+            m(i + u, mv);
+#pragma unroll
+            for (int q = 0; q < R; ++q) p[q] = fma(mv[q], xv, p[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) tot[q] += p[q];
+    }
+    if (i < K) {
+        T p[R] = {};
+        for (; i < K; ++i) {
+            const T xv = x(i);
+            T mv[R];
+            m(i, mv);
+#pragma unroll
+            for (int q = 0; q < R; ++q) p[q] = fma(mv[q], xv, p[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) tot[q] += p[q];
+    }
+}
+
+template <int R, typename T>
+__device__ __forceinline__ void plane_ld(const T* p, T (&v)[R]) {
+    if constexpr (R == 4 && sizeof(T) == 4) {
+        const float4 w = *reinterpret_cast<const float4*>(p);
+        v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = p[q];
+    }
+}
+
+template <typename T>
+constexpr int plane_r() { return sizeof(T) == 4 ? 4 : 1; }
+
+// matrix of n elements to shared memory, 16 bytes at a time (both aligned)
+template <typename T>
+__device__ __forceinline__ void plane_matrix(T* dst, const T* __restrict__ src, int n) {
+    constexpr int V = 16 / sizeof(T);
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n / V; e += PLANE_T)
+        reinterpret_cast<uint4*>(dst)[e] = __ldg(reinterpret_cast<const uint4*>(src) + e);
+    for (int e = n / V * V + threadIdx.x; e < n; e += PLANE_T) dst[e] = src[e];
+}
+
+// the block's columns of the first transform's matrix: [Ko1][sp] odd, [Ke1][sp] even results from p0
+template <typename T>
+__device__ __forceinline__ void plane_columns(T* S1, const T* __restrict__ s1, int M1, int sp, int p0) {
+    const int Ko1 = (M1 + 1) / 2, Ke1 = M1 / 2;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < M1 * sp; e += PLANE_T) {
+        const int i = e / sp, p = p0 + (e - i * sp);
+        const bool odd = i < Ko1;
+        S1[e] = p < (odd ? Ko1 : Ke1) ? __ldg(s1 + (odd ? i * Ko1 : Ko1 * Ko1 + (i - Ko1) * Ke1) + p) : T(0);
+    }
+}
+
+// lines a < A of M1 elements ld(a, i), folded: X[i][a] the sums (and the
+// middle element), X[M1 - 1 - i][a] the differences.  A warp takes whole
+// lines, eight at a time, all loads before the stores.
+template <typename T, typename LD>
+__device__ __forceinline__ void plane_fold(T* X, int pA, int A, int M1, LD&& ld) {
+    constexpr int B = 8;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = PLANE_T / 32, Ko1 = (M1 + 1) / 2;
+    for (int i = lane; i < Ko1; i += 32) {
+        const int j = M1 - 1 - i;
+        for (int a0 = w; a0 < A; a0 += B * nw) {
+            T lo[B], hi[B];
+#pragma unroll
+            for (int q = 0; q < B; ++q) {
+                const int a = a0 + q * nw;
+                lo[q] = a < A ? ld(a, i) : T(0);
+                hi[q] = a < A && i != j ? ld(a, j) : T(0);
+            }
+#pragma unroll
+            for (int q = 0; q < B; ++q) {
+                const int a = a0 + q * nw;
+                if (a >= A) continue;
+                X[i * pA + a] = i == j ? lo[q] : lo[q] + hi[q];
+                if (i != j) X[j * pA + a] = lo[q] - hi[q];
+            }
+        }
+    }
+}
+
+// first transform: G[a][parity sp + q] = results p0 + q of line a, from X and S1
+template <typename T>
+__device__ __forceinline__ void plane_first(const T* X, const T* S1, T* G, int A, int M1, int sp) {
+    constexpr int R = plane_r<T>();
+    const int Ko1 = (M1 + 1) / 2, Ke1 = M1 / 2, pA = A | 1, A32 = (A + 31) / 32 * 32, per = sp / R;
+    for (int u = threadIdx.x; u < A32 * 2 * per; u += PLANE_T) {
+        const int a = u % A32, h = u / A32, par = h / per, q0 = (h - par * per) * R;
+        if (a >= A) continue;
+        const T* S = S1 + (par ? Ko1 * sp : 0) + q0;
+        const T* Xa = X + (par ? (M1 - 1) * pA : 0) + a;
+        const int step = par ? -pA : pA;
+        T v[R];
+        plane_dot<T, R>(
+            par ? Ke1 : Ko1, [&](int i) { return Xa[i * step]; }, [&](int i, T(&m)[R]) { plane_ld<R>(S + i * sp, m); },
+            v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) G[a * 2 * sp + par * sp + q0 + q] = v[q];
+    }
+}
+
+// fold along the lines' index: row a the sums, row A - 1 - a the differences
+template <typename T>
+__device__ __forceinline__ void plane_refold(T* G, int A, int sp) {
+    for (int e = threadIdx.x; e < A / 2 * 2 * sp; e += PLANE_T) {
+        const int a = e / (2 * sp), q = e - a * 2 * sp;
+        const T lo = G[a * 2 * sp + q], hi = G[(A - 1 - a) * 2 * sp + q];
+        G[a * 2 * sp + q] = lo + hi;
+        G[(A - 1 - a) * 2 * sp + q] = lo - hi;
+    }
+}
+
+// second transform, of the refolded G along the lines' index: st(b, c, value) for result c of the
+// block's column b (0 .. 2 sp - 1, odd results first)
+template <typename T, typename ST>
+__device__ __forceinline__ void plane_second(const T* G, const T* S2, int A, int sp, ST&& st) {
+    constexpr int R = plane_r<T>();
+    const int Ko2 = (A + 1) / 2, Ke2 = A / 2, C32 = (Ko2 + 31) / 32 * 32, groups = 2 * sp / R;
+    for (int u = threadIdx.x; u < C32 * 2 * groups; u += PLANE_T) {
+        const int c = u % C32, h = u / C32, par = h / groups, b0 = (h - par * groups) * R;
+        const int K = par ? Ke2 : Ko2;
+        if (c >= K) continue;
+        const T* S = S2 + (par ? Ko2 * Ko2 : 0) + c;
+        const T* Gb = G + (par ? (A - 1) * 2 * sp : 0) + b0;
+        const int step = par ? -2 * sp : 2 * sp;
+        T v[R];
+        plane_dot<T, R>(K, [&](int i) { return S[i * K]; }, [&](int i, T(&m)[R]) { plane_ld<R>(Gb + i * step, m); }, v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) st(b0 + q, 2 * c + par, v[q]);
+    }
+}
+
+// block bx: results p0 = sp bx .. of either parity; by: the plane
+template <typename T>
+__device__ __forceinline__ void plane_body(const PlaneArgs<T>& g, int bx, int by) {
+    extern __shared__ __align__(16) unsigned char psep_smem[];
+    const int A = g.A, M1 = g.M1, sp = g.sp;
+    const PlaneLayout<T> L(A, M1, sp);
+    const int Ko1 = (M1 + 1) / 2, Ke1 = M1 / 2, Ko2 = (A + 1) / 2, Ke2 = A / 2;
+    T* S2 = reinterpret_cast<T*>(psep_smem);
+    T *S1 = S2 + L.s1, *G = S2 + L.g, *X = S2 + L.x;
+    const int p0 = bx * sp;
+    const T* in = g.in + by * g.in_plane;
+    plane_matrix(S2, g.s2, Ko2 * Ko2 + Ke2 * Ke2);
+    plane_columns(S1, g.s1, M1, sp, p0);
+    plane_fold(X, A | 1, A, M1, [&](int a, int i) { return in[a * g.in_line + i]; });
+    __syncthreads();
+    plane_first(X, S1, G, A, M1, sp);
+    __syncthreads();
+    plane_refold(G, A, sp);
+    __syncthreads();
+    T* out = g.out + by * g.out_plane;
+    plane_second(G, S2, A, sp, [&](int b, int c, T v) {
+        const int par = b >= sp, p = p0 + b - par * sp;
+        if (p >= (par ? Ke1 : Ko1)) return;
+        T* o = out + (long long)(2 * p + par) * g.out_line + c;
+        *o = dst_result(g.scale, v, g.accumulate != 0, g.accumulate ? *o : T(0));
+    });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(PLANE_T) sep_dense_kernel(PlaneArgs<T> a) {
+    plane_body(a, int(blockIdx.x), int(blockIdx.y));
+}
+
+// elements of the cluster kernel's X, which serves as [nxi][nyi | 1], [nyi][2 sp] and [nxi][2 so]
+template <typename T>
+__host__ __device__ inline size_t dense2d_x(int nxi, int nyi, int sp, int so) {
+    size_t n = size_t(nxi) * (nyi | 1);
+    if (size_t(nyi) * 2 * sp > n) n = size_t(nyi) * 2 * sp;
+    if (size_t(nxi) * 2 * so > n) n = size_t(nxi) * 2 * so;
+    return (n + 3) / 4 * 4;
+}
+
+// The whole solve of a lower-boundary level in one cluster (one CTA per slab
+// of results): x and y transforms of the CTA's x modes, the division by the
+// mode eigenvalues, the y transform back (still the CTA's own modes), one
+// exchange through distributed shared memory, and the x transform back of the
+// CTA's rows.  The operations of the plane stages and the division in their
+// order.  f = forward stage (x lines), b = the way back (y lines).
+template <typename T>
+__global__ void __launch_bounds__(PLANE_T) sep_dense2d_kernel(PlaneArgs<T> f, PlaneArgs<T> b, T cf, T cs,
+                                                              const T* __restrict__ mufast,
+                                                              const T* __restrict__ muslow) {
+    extern __shared__ __align__(16) unsigned char psep_smem[];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = int(cl.block_rank());
+    const int nyi = f.A, nxi = f.M1, sp = f.sp, so = b.sp;
+    const int Kox = (nxi + 1) / 2, Kex = nxi / 2, Koy = (nyi + 1) / 2, Key = nyi / 2;
+    const PlaneLayout<T> L(nyi, nxi, sp);
+    // the matrices of y (S2) and of x (after everything else), whole
+    T* Sy = reinterpret_cast<T*>(psep_smem);
+    T *S1 = Sy + L.s1, *G = Sy + L.g, *X = Sy + L.x, *Sx = X + dense2d_x<T>(nxi, nyi, sp, so);
+    T* C = Sx + (Kox * Kox + Kex * Kex + 3) / 4 * 4;   // [2 sp][nyi]: this CTA's modes, back in y
+    const int p0 = rank * sp;
+    plane_matrix(Sy, f.s2, Koy * Koy + Key * Key);
+    plane_matrix(Sx, f.s1, Kox * Kox + Kex * Kex);
+    plane_columns(S1, f.s1, nxi, sp, p0);
+    plane_fold(X, nyi | 1, nyi, nxi, [&](int a, int i) { return f.in[a * f.in_line + i]; });
+    __syncthreads();
+    plane_first(X, S1, G, nyi, nxi, sp);
+    __syncthreads();
+    plane_refold(G, nyi, sp);
+    __syncthreads();
+    // x mode of column q (past the last one: the results are not used)
+    auto mode = [&](int q) { return q < sp ? 2 * (p0 + q) : 2 * (p0 + q - sp) + 1; };
+    T* H = X;   // [nyi][2 sp]: mode n of column q, divided (X is no longer read)
+    plane_second(G, Sy, nyi, sp, [&](int q, int n, T v) {
+        const int m = mode(q);
+        H[n * 2 * sp + q] = m < nxi ? mode_divide(dst_result(T(1), v, false, T(0)), cf, mufast[n], cs, muslow[m]) : T(0);
+    });
+    __syncthreads();
+    plane_refold(H, nyi, sp);
+    __syncthreads();
+    plane_second(H, Sy, nyi, sp, [&](int q, int j, T v) { C[q * nyi + j] = v; });
+    cl.sync();
+    // rows j of this CTA (so odd and so even indexes), all modes from their owners
+    const int r0 = rank * so, rows = 2 * so;
+    T* Y = X;   // [nxi][2 so]: element m of row column r
+    for (int e = threadIdx.x; e < nxi * rows; e += PLANE_T) {
+        const int r = e / nxi, m = e - r * nxi;
+        const int j = r < so ? 2 * (r0 + r) : 2 * (r0 + r - so) + 1;
+        const int p = m >> 1, owner = p / sp, q = (p - owner * sp) + ((m & 1) ? sp : 0);
+        Y[m * rows + r] = j < nyi ? cl.map_shared_rank(C, owner)[q * nyi + j] : T(0);
+    }
+    cl.sync();   // every remote read done before any CTA of the cluster exits
+    plane_refold(Y, nxi, so);
+    __syncthreads();
+    plane_second(Y, Sx, nxi, so, [&](int r, int i, T v) {
+        const int j = r < so ? 2 * (r0 + r) : 2 * (r0 + r - so) + 1;
+        if (j >= nyi) return;
+        T* o = b.out + (long long)j * b.out_line + i;
+        *o = dst_result(b.scale, v, b.accumulate != 0, b.accumulate ? *o : T(0));
+    });
+}
+
+// shared memory of the cluster kernel: plane_body's, the x matrix and the exchanged modes after it
+template <typename T>
+size_t dense2d_smem(int nxi, int nyi, int sp, int so) {
+    const int Kox = (nxi + 1) / 2, Kex = nxi / 2;
+    return (size_t(PlaneLayout<T>(nyi, nxi, sp).x) + dense2d_x<T>(nxi, nyi, sp, so) +
+            (size_t(Kox) * Kox + size_t(Kex) * Kex + 3) / 4 * 4 + size_t(2) * sp * nyi) *
+           sizeof(T);
+}
+
+// one thread per result of a line (the staged form: one transform per
+// launch): plane_dot's sums on the folded line
+template <typename T>
+__global__ void sep_line_kernel(int lines, int M, const T* in, long long in_plane, long long in_line, T* out,
+                                long long out_plane, long long out_line, long long out_elem,
+                                const T* __restrict__ s, T scale, int accumulate) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y, k = blockIdx.z;
+    if (m >= M || l >= lines) return;
+    const T* x = in + k * in_plane + l * in_line;
+    const int Ko = (M + 1) / 2, Ke = M / 2, par = m & 1, p = m >> 1, K = par ? Ke : Ko;
+    const T* S = s + (par ? Ko * Ko : 0) + p;
+    T v[1];
+    plane_dot<T, 1>(
+        K,
+        [&](int i) {
+            const int j = M - 1 - i;
+            return i == j ? x[i] : par ? x[i] - x[j] : x[i] + x[j];
+        },
+        [&](int i, T(&w)[1]) { w[0] = S[i * K]; }, v);
+    T* o = out + k * out_plane + l * out_line + m * out_elem;
+    *o = dst_result(scale, v[0], accumulate != 0, accumulate ? *o : T(0));
+}
+
+constexpr size_t PLANE_SMEM = 227 * 1024;
+constexpr int PLANE_CELLS = 128;
 
 // Elimination factors of the mode systems of one 3D level, one thread per
 // mode (fast index m, slow index n; the layout of the transformed data),
@@ -366,6 +698,7 @@ __global__ void __launch_bounds__(1024) g_sep_kernel(const GSepItem<T>* items, i
     if constexpr (KIND == SEP_GEMM) gemm_body(it->st.gemm, bx, by, bz);
     else if constexpr (KIND == SEP_SCAN) scan_body(it->st.mode, bx, by);
     else if constexpr (KIND == SEP_THOMAS) thomas_body(it->st.mode, bx, by);
+    else if constexpr (KIND == SEP_PLANE) plane_body(it->st.plane, bx, by);
     else divide_body(it->st.mode, bx, by);
 }
 
@@ -426,6 +759,25 @@ SepStage<T> gemm_stage(const GemmArgs<T>& g, int batch) {
     return s;
 }
 
+// The plane transforms as one stage, both directions: along lines of M1
+// elements first.  Blocks of as many results as leave a block per SM (FP64:
+// down to one odd and one even result, FP32: four of each).
+template <typename T>
+SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes) {
+    SepStage<T> s;
+    s.kind = SEP_PLANE;
+    s.plane = p;
+    s.threads = PLANE_T;
+    const int Ko1 = (p.M1 + 1) / 2, least = sizeof(T) == 4 ? 4 : 1;
+    int sp = 16;
+    while (sp > least && (long long)((Ko1 + sp - 1) / sp) * planes < 152) sp /= 2;
+    while (sp > least && PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T) > PLANE_SMEM) sp /= 2;
+    s.plane.sp = sp;
+    s.smem = PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T);
+    s.grid = dim3((Ko1 + sp - 1) / sp, planes);
+    return s;
+}
+
 // The stages of A e = f on one level, e = out (stored, or added with
 // accumulate), f and out pitched level arrays (interior read / written), t1
 // and t2 dense scratch of the interior size (t2 may be the array of f).
@@ -445,6 +797,35 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
     const T* mux = static_cast<const T*>(tab.mux);
     const T* muy = static_cast<const T*>(tab.muy);
     const T scale = T((2.0 / (g.nx - 1)) * (2.0 / (g.ny - 1)));
+    if (tab.fx) {   // x lines of f -> t1[k][m][n], mode solves, y lines back and x -> out, scaled
+        PlaneArgs<T> p;
+        p.A = nyi;
+        p.M1 = nxi;
+        p.in = f + off;
+        p.in_plane = sA;
+        p.in_line = g.px;
+        p.out = t1;
+        p.out_plane = pl;
+        p.out_line = nyi;
+        p.s1 = static_cast<const T*>(tab.fx);
+        p.s2 = static_cast<const T*>(tab.fy);
+        stages.push_back(plane_stage<T>(p, nzi));
+        stages.push_back(mode_stage<T>(g, dim, coef, tab, nyi, nxi, muy, mux, true, t1));
+        p.A = nxi;
+        p.M1 = nyi;
+        p.in = t1;
+        p.in_plane = pl;
+        p.in_line = nyi;
+        p.out = out + off;
+        p.out_plane = sA;
+        p.out_line = g.px;
+        p.s1 = static_cast<const T*>(tab.fy);
+        p.s2 = static_cast<const T*>(tab.fx);
+        p.scale = scale;
+        p.accumulate = accumulate ? 1 : 0;
+        stages.push_back(plane_stage<T>(p, nzi));
+        return;
+    }
     if (tab.twx) {
         auto dst = [&](const DstArgs<T>& a) {
             SepStage<T> s;
@@ -500,6 +881,16 @@ void launch_stage(const SepStage<T>& s, cudaStream_t st) {
         break;
     }
     case SEP_THOMAS: sep_thomas_kernel<T><<<s.grid, s.threads, 0, st>>>(s.mode); break;
+    case SEP_PLANE: {
+        static bool configured = false;
+        if (!configured) {
+            MHS_CUDA(cudaFuncSetAttribute(sep_dense_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          int(PLANE_SMEM)));
+            configured = true;
+        }
+        sep_dense_kernel<T><<<s.grid, s.threads, s.smem, st>>>(s.plane);
+        break;
+    }
     default: sep_divide_kernel<T><<<s.grid, s.threads, 0, st>>>(s.mode); break;
     }
     count_launches(1);
@@ -525,6 +916,89 @@ void level_solve(mhs_ctx* c, const Geom& g, int dim, const PlaneCoef<T>* coef, c
     for (const SepStage<T>& s : stages) launch_stage<T>(s, c->stream);
 }
 
+// the stages of a level with folded matrices, one transform per launch (same results)
+template <typename T>
+void staged_lines(mhs_ctx* c, const Geom& g, int dim, const SepTables& tab, const SepStage<T>& modes, const T* f, T* t,
+                  T* w, T* out) {
+    const int nxi = g.nx - 2, nyi = g.ny - 2, nzi = dim == 3 ? g.nz - 2 : 1;
+    const long long pl = (long long)nxi * nyi;
+    const long long off = dim == 3 ? (long long)g.plane + g.px + 1 : (long long)g.px + 1;
+    const long long sA = dim == 3 ? (long long)g.plane : 0;
+    const T *sx = static_cast<const T*>(tab.fx), *sy = static_cast<const T*>(tab.fy);
+    auto pass = [&](int lines, int M, const T* in, long long ip, long long il, T* o, long long op, long long ol,
+                    long long oe, const T* s, T scale) {
+        sep_line_kernel<T><<<dim3((M + 63) / 64, lines, nzi), 64, 0, c->stream>>>(lines, M, in, ip, il, o, op, ol, oe, s,
+                                                                                  scale, 0);
+        count_launches(1);
+        MHS_CUDA(cudaGetLastError());
+    };
+    pass(nyi, nxi, f + off, sA, g.px, w, pl, 1, nyi, sx, T(1));        // x lines -> w[k][m][j]
+    pass(nxi, nyi, w, pl, nyi, t, pl, nyi, 1, sy, T(1));               // y lines -> t[k][m][n]
+    launch_stage<T>(modes, c->stream);
+    pass(nxi, nyi, t, pl, nyi, w, pl, 1, nxi, sy, T(1));               // back along y -> w[k][j][m]
+    pass(nyi, nxi, w, pl, nxi, out + off, sA, g.px, 1, sx, T((2.0 / (g.nx - 1)) * (2.0 / (g.ny - 1))));
+}
+
+// a lower-boundary level with folded matrices in one cluster; false when no
+// cluster of the kernel fits (nothing launched)
+template <typename T>
+bool dense2d_solve(const std::vector<SepStage<T>>& st, cudaStream_t stream) {
+    PlaneArgs<T> f = st[0].plane, b = st[2].plane;
+    const ModeArgs<T>& m = st[1].mode;
+    const int Kox = (f.M1 + 1) / 2, Koy = (f.A + 1) / 2, r = plane_r<T>();
+    const void* fn = reinterpret_cast<const void*>(&sep_dense2d_kernel<T>);
+    static std::mutex mu;
+    static std::map<std::pair<int, int>, int> known;   // cluster size of (nxi, nyi), 0: none
+    auto slab = [&](int K, int c) { return ((K + c - 1) / c + r - 1) / r * r; };
+    int c = 0;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = known.find({f.M1, f.A});
+        if (it != known.end()) {
+            c = it->second;
+        } else {
+            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PLANE_SMEM)) == cudaSuccess &&
+                cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+                for (int n = 16; n >= 1 && !c; n /= 2) {
+                    const size_t smem = dense2d_smem<T>(f.M1, f.A, slab(Kox, n), slab(Koy, n));
+                    if (smem > PLANE_SMEM) break;
+                    if (n > 1 && (n / 2) * r >= std::max(Kox, Koy)) continue;   // fewer CTAs suffice
+                    cudaLaunchConfig_t cfg{};
+                    cudaLaunchAttribute attr{};
+                    attr.id = cudaLaunchAttributeClusterDimension;
+                    attr.val.clusterDim.x = n;
+                    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+                    cfg.gridDim = dim3(n, 1, 1);
+                    cfg.blockDim = dim3(PLANE_T, 1, 1);
+                    cfg.dynamicSmemBytes = smem;
+                    cfg.attrs = &attr;
+                    cfg.numAttrs = 1;
+                    int clusters = 0;
+                    if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) c = n;
+                }
+            (void)cudaGetLastError();
+            known[{f.M1, f.A}] = c;
+        }
+    }
+    if (c == 0) return false;
+    f.sp = slab(Kox, c);
+    b.sp = slab(Koy, c);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = c;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(c, 1, 1);
+    cfg.blockDim = dim3(PLANE_T, 1, 1);
+    cfg.dynamicSmemBytes = dense2d_smem<T>(f.M1, f.A, f.sp, b.sp);
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    MHS_CUDA(cudaLaunchKernelEx(&cfg, sep_dense2d_kernel<T>, f, b, m.cf, m.cs, m.mufast, m.muslow));
+    count_launches(1);
+    return true;
+}
+
 template <typename T>
 LevelArrays<T>& arrays_of(Hierarchy& H, int l);
 template <>
@@ -539,7 +1013,7 @@ template <typename T>
 void compute_pivots(mhs_ctx* c, Hierarchy& H, int l, SepTables& t) {
     const Geom& g = H.g[l];
     if (H.dim != 3 || !t.inv) return;
-    const bool ytrans = t.twx != nullptr;
+    const bool ytrans = t.twx != nullptr || t.fx != nullptr;
     const int nxi = g.nx - 2, nyi = g.ny - 2;
     const int nfast = ytrans ? nyi : nxi, nslow = ytrans ? nxi : nyi;
     const int threads = nfast <= 64 ? 64 : 128;
@@ -561,6 +1035,19 @@ const SepTables& tables(Hierarchy& H, int l) {
 
 bool sep_level_ok(const Geom& g) {
     return (pow2(g.nx - 1) && pow2(g.ny - 1)) || (g.nx <= 66 && g.ny <= 66);
+}
+
+// The levels whose planes are transformed by plane_body: at most 128 cells a
+// side, and in FP64 those whose dense products take the FP64 pipe less time
+// than the fast transforms' chain of steps (one plane, or short lines), or
+// that have no fast transform.
+template <typename T>
+static bool dense_planes(const Geom& g, int dim) {
+    const int big = std::max(g.nx, g.ny) - 1, least = sizeof(T) == 4 ? 4 : 1;
+    if (big > PLANE_CELLS || PlaneLayout<T>(g.ny - 2, g.nx - 2, least).total * sizeof(T) > PLANE_SMEM ||
+        PlaneLayout<T>(g.nx - 2, g.ny - 2, least).total * sizeof(T) > PLANE_SMEM)
+        return false;
+    return sizeof(T) == 4 || big <= (dim == 2 ? 64 : 32) || !(pow2(g.nx - 1) && pow2(g.ny - 1));
 }
 
 // Mode eigenvalues, and twiddles or sine matrices, of level l in T, built once
@@ -602,9 +1089,23 @@ void sep_tables(mhs_ctx* c, Hierarchy& H, int l) {
             }
         return s;
     };
+    // folded: element (i, p) of the odd results' matrix is S[2p][i], of the even ones' S[2p+1][i]
+    auto folded = [&](int n) {
+        const int M = n - 2, Ko = (M + 1) / 2, Ke = M / 2;
+        const std::vector<T> S = sine(n);
+        std::vector<T> s(size_t(Ko) * Ko + size_t(Ke) * Ke);
+        for (int i = 0; i < Ko; ++i)
+            for (int p = 0; p < Ko; ++p) s[size_t(i) * Ko + p] = S[size_t(2 * p) * M + i];
+        for (int i = 0; i < Ke; ++i)
+            for (int p = 0; p < Ke; ++p) s[size_t(Ko) * Ko + size_t(i) * Ke + p] = S[size_t(2 * p + 1) * M + i];
+        return s;
+    };
     t.mux = upload(mu(g.nx));
     t.muy = upload(mu(g.ny));
-    if (pow2(g.nx - 1) && pow2(g.ny - 1)) {
+    if (dense_planes<T>(g, H.dim)) {
+        t.fx = upload(folded(g.nx));
+        t.fy = upload(folded(g.ny));
+    } else if (pow2(g.nx - 1) && pow2(g.ny - 1)) {
         size_t tb = 0;
         t.twx = make_twiddles<T>(g.nx - 1, &tb);
         c->allocations.push_back(t.twx);
@@ -646,6 +1147,17 @@ void sep_exact(mhs_ctx* c, Hierarchy& H, int l) {
                                              static_cast<const T*>(tab.mux), true, A.t);
         if (plane_level_solve<T>(g, H.dim, tab, A.f, A.t, A.u, false, &ms, c->stream)) return;
     }
+    if (tab.fx) {
+        std::vector<SepStage<T>> st;
+        plan_level<T>(g, H.dim, A.coef, tab, A.f, A.t, A.r, A.u, false, st);
+        if (c->opts.flags & MHS_FLAG_STAGED_TRANSFORMS) {
+            staged_lines<T>(c, g, H.dim, tab, st[1], A.f, A.t, A.r, A.u);
+            return;
+        }
+        if (H.dim == 2 && dense2d_solve<T>(st, c->stream)) return;
+        for (const SepStage<T>& q : st) launch_stage<T>(q, c->stream);
+        return;
+    }
     level_solve<T>(c, g, H.dim, A.coef, tab, A.f, A.r, A.t, A.u, false);
 }
 
@@ -673,6 +1185,16 @@ void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st)
         break;
     }
     case SEP_THOMAS: g_sep_kernel<T, SEP_THOMAS><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate); break;
+    case SEP_PLANE: {
+        static bool configured = false;
+        if (!configured) {
+            MHS_CUDA(cudaFuncSetAttribute(g_sep_kernel<T, SEP_PLANE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          int(PLANE_SMEM)));
+            configured = true;
+        }
+        g_sep_kernel<T, SEP_PLANE><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);
+        break;
+    }
     default: g_sep_kernel<T, SEP_DIVIDE><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate); break;
     }
     count_launches(1);

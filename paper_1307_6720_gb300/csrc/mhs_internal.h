@@ -111,6 +111,7 @@ struct SepTables {
     void *mux = nullptr, *muy = nullptr;
     void *twx = nullptr, *twy = nullptr;
     void *sx = nullptr, *sy = nullptr;
+    void *fx = nullptr, *fy = nullptr;   // folded sine matrices of the plane transforms (kernels_sep.cu)
     void *inv = nullptr, *sup = nullptr;
     bool ready = false;
 };
@@ -372,7 +373,22 @@ struct ModeArgs {
     const T* muslow = nullptr;
     T cf = T(0), cs = T(0);
 };
-enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4 };
+// both sine transforms of every plane: lines a = 0 .. A-1 of M1 elements, then
+// for each result b along the A lines; element i of line a of plane k at
+// in + k in_plane + a in_line + i, result c of b at out + k out_plane + b out_line + c
+template <typename T>
+struct PlaneArgs {
+    int A = 0, M1 = 0, sp = 0;   // sp: results b of either parity per block
+    const T* in = nullptr;
+    long long in_plane = 0, in_line = 0;
+    T* out = nullptr;
+    long long out_plane = 0, out_line = 0;
+    const T* s1 = nullptr;       // folded sine matrices of the two lengths
+    const T* s2 = nullptr;
+    T scale = T(1);
+    int accumulate = 0;
+};
+enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4, SEP_PLANE = 5 };
 // one kernel launch of a separable solve with its launch shape
 template <typename T>
 struct SepStage {
@@ -383,6 +399,7 @@ struct SepStage {
     DstArgs<T> dst;
     GemmArgs<T> gemm;
     ModeArgs<T> mode;
+    PlaneArgs<T> plane;
 };
 // launch shape of a sine-transform stage (sets a.pairs)
 template <typename T>

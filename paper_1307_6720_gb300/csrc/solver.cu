@@ -1093,7 +1093,7 @@ size_t handle_bytes_estimate(int nx, int ny, int nz, double Lx, double Ly, doubl
                 if (dim == 3) b += 2 * round_up(g.interior() * (sizeof(double) + sizeof(float)), q);
                 // mode eigenvalues and twiddles, or sine matrices of short rows, in both precisions
                 b += 4 * round_up(size_t(x + y) * 2 * sizeof(double), q);
-                if (x <= 66 && y <= 66) b += 2 * round_up(size_t(x * x + y * y) * sizeof(double), q);
+                if (x <= 129 && y <= 129) b += 2 * round_up(size_t(x * x + y * y) * sizeof(double), q);
             }
             const bool can = coarsenable(x) && coarsenable(y) && (dim == 2 || coarsenable(z));
             if (!can || l + 1 == MAX_SUB_LEVELS) break;

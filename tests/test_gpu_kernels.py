@@ -649,3 +649,36 @@ def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
     assert np.array_equal(got[0], got[1])
     assert not np.array_equal(got[0], u)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("shape", [(5, 5, 5), (7, 5, 9), (9, 33, 5), (35, 19, 5), (67, 67, 9), (65, 63, 9), (129, 9, 5),
+                                   (129, 129, 5), (127, 67, 5)])
+def test_plane_transforms_of_folded_matrices(M, shape, prec):
+    """The plane transforms with folded sine matrices (one pair of lines up to
+    128 cells, odd and even lengths, ragged slabs of results), 2D and 3D,
+    against the separable direct solution; the staged form, one transform per
+    launch, gives the same bits.  Bounds: those of test_exact_op_parity."""
+    from oracle import exact
+    nx, ny, nz = shape
+    pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
+    for dim in (3, 2):
+        shape_l = (nz, ny, nx) if dim == 3 else (ny, nx)
+        f = np.random.default_rng(nx + dim).standard_normal(shape_l)
+        if prec == 1:
+            f = f.astype(np.float32).astype(np.float64)
+        fast = (nx - 1) & (nx - 2) == 0 and (ny - 1) & (ny - 2) == 0
+        if not (fast or (nx <= 66 and ny <= 66)):
+            continue
+        got = []
+        for flags in (0, M.MHS_FLAG_STAGED_TRANSFORMS):
+            M.mhs_set_options(h, flags=flags)
+            M.mhs_level_write(h, dim, 0, M.MHS_FIELD_U, prec, np.zeros(shape_l))
+            M.mhs_level_write(h, dim, 0, M.MHS_FIELD_F, prec, f)
+            M.mhs_level_op(h, dim, 0, M.MHS_OP_EXACT, prec)
+            got.append(_read(M, h, dim, 0, M.MHS_FIELD_U, prec))
+        prl = _level_problem(M, h, pr, dim, 0)
+        want = exact.separable_solve3d(prl, np.zeros((ny, nx)), f) if dim == 3 else exact.separable_solve2d(prl, -f)
+        assert _rel(got[0], want) < (1e-12 if prec == 0 else 2e-5), dim
+        assert np.array_equal(got[0], got[1]), dim
+    M.mhs_destroy(h)
