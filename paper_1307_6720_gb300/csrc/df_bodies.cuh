@@ -359,12 +359,23 @@ __device__ __forceinline__ void df_split_body(const Geom& g, int d3, const doubl
     }
 }
 
+// a float's double by integer operations (the FP64 pipe, which conversions
+// use, is the bound of df_to_double): exponent rebiased, fraction shifted;
+// zeros, subnormals, infinities and NaN take the conversion
+__device__ __forceinline__ double df_widen(float f) {
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double(int((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), int(u << 29));
+    return a == 0 ? __hiloint2double(int(u), 0) : double(f);
+}
+__device__ __forceinline__ double df_double(float hi, float lo) { return df_widen(hi) + df_widen(lo); }
+
 // P = hi + lo over the whole array (grid-stride over gd.x blocks)
 __device__ __forceinline__ void df_to_double_body(size_t n, const float* __restrict__ hi,
                                                   const float* __restrict__ lo, double* __restrict__ P, dim3 b,
                                                   dim3 gd) {
     for (size_t o = b.x * size_t(blockDim.x) + threadIdx.x; o < n; o += size_t(gd.x) * blockDim.x)
-        P[o] = double(hi[o]) + double(lo[o]);
+        P[o] = df_double(hi[o], lo[o]);
 }
 
 __device__ __forceinline__ void df_copy_plane_body(const Geom& g2, const float* __restrict__ hi2,

@@ -108,8 +108,8 @@ __global__ void __launch_bounds__(DF_TO_DOUBLE_THREADS) df_to_double_kernel(size
     double2* __restrict__ out = reinterpret_cast<double2*>(P);
     for (size_t o = blockIdx.x * size_t(blockDim.x) + threadIdx.x; o < n / 4; o += size_t(gridDim.x) * blockDim.x) {
         const float4 h = hi[o], l = lo[o];
-        out[2 * o] = make_double2(double(h.x) + double(l.x), double(h.y) + double(l.y));
-        out[2 * o + 1] = make_double2(double(h.z) + double(l.z), double(h.w) + double(l.w));
+        out[2 * o] = make_double2(df_double(h.x, l.x), df_double(h.y, l.y));
+        out[2 * o + 1] = make_double2(df_double(h.z, l.z), df_double(h.w, l.w));
     }
 }
 
