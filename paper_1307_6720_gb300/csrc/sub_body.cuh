@@ -105,30 +105,82 @@ __device__ __forceinline__ T sub_off(const SubGeom& g, const PlaneCoef<T>& c, co
     return off;
 }
 
-// one red-black sweep (colour 0 = (i+j+k) even first)
-template <typename T, bool D3>
-__device__ void sub_smooth(const SubSmem<T, D3>& S, int l) {
+// node of work item q of a colour pass (colour 0 = (i+j+k) even), its plane in k; 0: none
+template <bool D3>
+__device__ __forceinline__ int sub_node(const SubGeom& g, int q, int colour, int& k) {
+    const int row = fdiv(q, g.inv_hx);
+    const int t = q - row * g.hx;
+    const int kk = D3 ? fdiv(row, g.inv_nyi) : 0;
+    const int j = 1 + row - kk * g.nyi;
+    k = D3 ? 1 + kk : 0;
+    const int i = 1 + (((1 + j + k) & 1) != colour) + 2 * t;
+    return i > g.nx - 2 ? 0 : i + g.px * (j + g.ny * k);
+}
+
+// n red-black sweeps of a level whose colour passes have at most NI items per
+// thread: the items' places and f / d are formed once, so that a pass is
+// the update u = f/d - ax (E + W) - ay (N + S) - az (U + D) alone
+template <typename T, bool D3, int NI>
+__device__ __forceinline__ void sub_smooth_kept(const SubSmem<T, D3>& S, int l, int n) {
     const SubGeom g = S.g[l];
     T* u = S.a + g.off_u;
     const T* f = S.a + g.off_f;
     const PlaneCoef<T>* cf = S.c + g.off_c;
-    const int nw = g.hx * g.nyi * (D3 ? g.nz - 2 : 1);
+    const int nw = g.hx * g.nyi * (D3 ? g.nz - 2 : 1), nt = SX * blockDim.y;
     const int tid = threadIdx.x + SX * threadIdx.y;
-    for (int colour = 0; colour < 2; ++colour) {
-        for (int q = tid; q < nw; q += SX * blockDim.y) {
-            const int row = fdiv(q, g.inv_hx);
-            const int t = q - row * g.hx;
-            const int kk = D3 ? fdiv(row, g.inv_nyi) : 0;
-            const int j = 1 + row - kk * g.nyi;
-            const int k = D3 ? 1 + kk : 0;
-            const int i = 1 + (((1 + j + k) & 1) != colour) + 2 * t;
-            if (i > g.nx - 2) continue;
-            const PlaneCoef<T> c = cf[k];
-            const int o = i + g.px * (j + g.ny * k);
-            u[o] = (f[o] - sub_off<T, D3>(g, c, u, o)) * c.inv_d;
+    int o[2][NI], kp[2][NI];
+    T fs[2][NI];
+#pragma unroll
+    for (int colour = 0; colour < 2; ++colour)
+#pragma unroll
+        for (int s = 0; s < NI; ++s) {
+            const int q = tid + s * nt;
+            kp[colour][s] = 0;
+            o[colour][s] = q < nw ? sub_node<D3>(g, q, colour, kp[colour][s]) : 0;
+            fs[colour][s] = o[colour][s] ? f[o[colour][s]] * cf[kp[colour][s]].inv_d : T(0);
         }
-        __syncthreads();
-    }
+    for (int sweep = 0; sweep < n; ++sweep)
+#pragma unroll
+        for (int colour = 0; colour < 2; ++colour) {
+#pragma unroll
+            for (int s = 0; s < NI; ++s) {
+                const int at = o[colour][s];
+                if (!at) continue;
+                const PlaneCoef<T>& c = cf[D3 ? kp[colour][s] : 0];
+                T v = fs[colour][s];
+                if (D3) v = fma(-c.az, u[at + g.plane] + u[at - g.plane], v);
+                v = fma(-c.ay, u[at + g.px] + u[at - g.px], v);
+                u[at] = fma(-c.ax, u[at + 1] + u[at - 1], v);
+            }
+            __syncthreads();
+        }
+}
+
+// n red-black sweeps
+template <typename T, bool D3>
+__device__ void sub_smooth(const SubSmem<T, D3>& S, int l, int n) {
+    const SubGeom g = S.g[l];
+    const int nw = g.hx * g.nyi * (D3 ? g.nz - 2 : 1), nt = SX * blockDim.y;
+    if (nw <= nt) return sub_smooth_kept<T, D3, 1>(S, l, n);
+    if (nw <= 3 * nt) return sub_smooth_kept<T, D3, 3>(S, l, n);
+    T* u = S.a + g.off_u;
+    const T* f = S.a + g.off_f;
+    const PlaneCoef<T>* cf = S.c + g.off_c;
+    const int tid = threadIdx.x + SX * threadIdx.y;
+    for (int sweep = 0; sweep < n; ++sweep)
+        for (int colour = 0; colour < 2; ++colour) {
+            for (int q = tid; q < nw; q += nt) {
+                int k;
+                const int o = sub_node<D3>(g, q, colour, k);
+                if (!o) continue;
+                const PlaneCoef<T>& c = cf[k];
+                T v = f[o] * c.inv_d;
+                if (D3) v = fma(-c.az, u[o + g.plane] + u[o - g.plane], v);
+                v = fma(-c.ay, u[o + g.px] + u[o - g.px], v);
+                u[o] = fma(-c.ax, u[o + 1] + u[o - 1], v);
+            }
+            __syncthreads();
+        }
 }
 
 // one zebra z-line sweep (columns with i + j even first): each thread solves
@@ -173,19 +225,21 @@ __device__ void sub_zline(const SubSmem<T, true>& S, int l) {
 }
 
 template <typename T, bool D3>
-__device__ __forceinline__ void sub_relax(const SubSmem<T, D3>& S, int l, int line) {
+__device__ __forceinline__ void sub_relax(const SubSmem<T, D3>& S, int l, int line, int n) {
     if constexpr (D3) {
         if (line) {
-            sub_zline<T>(S, l);
+            for (int q = 0; q < n; ++q) sub_zline<T>(S, l);
             return;
         }
     }
-    sub_smooth<T, D3>(S, l);
+    sub_smooth<T, D3>(S, l, n);
 }
 
-// f[l+1] = full weighting of (f - A u) on level l; u[l+1] = 0 at interior nodes
+// f[l+1] = full weighting of (f - A u) on level l; u[l+1] = 0 at interior nodes.
+// red: right after a red-black sweep, whose black nodes' residual is zero to
+// rounding: only the centre and the neighbours with two offsets count
 template <typename T, bool D3>
-__device__ void sub_restrict_residual(const SubSmem<T, D3>& S, int l) {
+__device__ void sub_restrict_residual(const SubSmem<T, D3>& S, int l, bool red) {
     const SubGeom gf = S.g[l], gc = S.g[l + 1];
     const T* u = S.a + gf.off_u;
     const T* f = S.a + gf.off_f;
@@ -199,7 +253,33 @@ __device__ void sub_restrict_residual(const SubSmem<T, D3>& S, int l) {
         const int KK = D3 ? fdiv(row, gc.inv_nyi) : 0;
         const int J = 1 + row - KK * gc.nyi;
         const int K = D3 ? 1 + KK : 0;
-        {
+        if (red) {
+            auto res = [&](int o, const PlaneCoef<T>& c) {
+                T v = f[o];
+                if (D3) v = fma(-c.cz, u[o + gf.plane] + u[o - gf.plane], v);
+                v = fma(-c.cy, u[o + gf.px] + u[o - gf.px], v);
+                v = fma(-c.cx, u[o + 1] + u[o - 1], v);
+                return fma(-c.d, u[o], v);
+            };
+            const int k = D3 ? 2 * K : 0, o = 2 * I + gf.px * (2 * J + gf.ny * k), py = gf.px;
+            const PlaneCoef<T>& c = cf[k];
+            T sum = (res(o - py - 1, c) + res(o - py + 1, c)) + (res(o + py - 1, c) + res(o + py + 1, c));
+            T acc;
+            if (D3) {
+#pragma unroll
+                for (int s = -1; s <= 1; s += 2) {
+                    const PlaneCoef<T>& cs = cf[k + s];
+                    const int os = o + s * gf.plane;
+                    sum += (res(os - 1, cs) + res(os + 1, cs)) + (res(os - py, cs) + res(os + py, cs));
+                }
+                acc = fma(T(0.125), res(o, c), T(1.0 / 32.0) * sum);
+            } else {
+                acc = fma(T(0.25), res(o, c), T(1.0 / 16.0) * sum);
+            }
+            const int oc = I + gc.px * (J + gc.ny * K);
+            fc[oc] = acc;
+            uc[oc] = T(0);
+        } else {
             T acc = T(0);
             for (int c3 = (D3 ? -1 : 0); c3 <= (D3 ? 1 : 0); ++c3) {
                 const int k = D3 ? 2 * K + c3 : 0;
@@ -283,7 +363,7 @@ __device__ void sub_coarsest(const SubSmem<T, D3>& S, int l, int line) {
     const SubGeom g = S.g[l];
     const int nint = (g.nx - 2) * (g.ny - 2) * (D3 ? g.nz - 2 : 1);
     if (nint == 1) {
-        sub_relax<T, D3>(S, l, line);
+        sub_relax<T, D3>(S, l, line, 1);
         return;
     }
     const double tol = sizeof(T) == 8 ? 1e-10 : 1e-5;
@@ -296,13 +376,11 @@ __device__ void sub_coarsest(const SubSmem<T, D3>& S, int l, int line) {
         s_done = fn == 0.0;
     }
     __syncthreads();
-    for (int sweep = 0; sweep < 2000 && !s_done; ++sweep) {
-        sub_relax<T, D3>(S, l, line);
-        if ((sweep & 3) == 3) {
-            const double rr = sub_norm2<T, D3>(S, l, true);
-            if (tid == 0) s_done = rr <= tol * tol * s_fn;
-            __syncthreads();
-        }
+    for (int sweep = 0; sweep < 2000 && !s_done; sweep += 4) {
+        sub_relax<T, D3>(S, l, line, 4);
+        const double rr = sub_norm2<T, D3>(S, l, true);
+        if (tid == 0) s_done = rr <= tol * tol * s_fn;
+        __syncthreads();
     }
 }
 
@@ -346,13 +424,13 @@ __device__ __forceinline__ void subcycle_body(const SubParams<T>& p) {
     __syncthreads();
     const SubSmem<T, D3> S{sa, sc, sg};
     for (int l = 0; l < p.nlev - 1; ++l) {
-        for (int q = 0; q < p.nu1; ++q) sub_relax<T, D3>(S, l, p.line);
-        sub_restrict_residual<T, D3>(S, l);
+        sub_relax<T, D3>(S, l, p.line, p.nu1);
+        sub_restrict_residual<T, D3>(S, l, p.nu1 >= 1 && !(D3 && p.line));
     }
     sub_coarsest<T, D3>(S, p.nlev - 1, p.line);
     for (int l = p.nlev - 2; l >= 0; --l) {
         sub_prolong<T, D3>(S, l);
-        for (int q = 0; q < p.nu2; ++q) sub_relax<T, D3>(S, l, p.line);
+        sub_relax<T, D3>(S, l, p.line, p.nu2);
     }
     const SubGeom g0 = sg[0];
     const T* u0 = sa + g0.off_u;
