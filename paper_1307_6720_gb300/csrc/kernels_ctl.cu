@@ -15,13 +15,6 @@ __global__ void bnorm_kernel(const double* __restrict__ partial, int n, SolveCtl
     bnorm_body(partial, n, ctl);
 }
 
-__global__ void check_kernel(const double* __restrict__ partial, int n, SolveCtl* ctl, int first,
-                             cudaGraphConditionalHandle handle, int use_handle, int flips) {
-    const int cont = check_body(partial, n, ctl, first);
-    if (threadIdx.x == 0 && flips) ctl->flip ^= 1;
-    if (threadIdx.x == 0 && use_handle) cudaGraphSetConditional(handle, cont);
-}
-
 template <typename T, bool D3>
 __global__ void __launch_bounds__(SX * SY) subcycle_kernel(const SubParams<T> p) {
     subcycle_body<T, D3>(p);
@@ -30,14 +23,7 @@ __global__ void __launch_bounds__(SX * SY) subcycle_kernel(const SubParams<T> p)
 }  // namespace
 
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st) {
-    bnorm_kernel<<<1, 1024, 0, st>>>(partial, n, ctl);
-    count_launches(1);
-    MHS_CUDA(cudaGetLastError());
-}
-
-void launch_check(const double* partial, int n, SolveCtl* ctl, int first, cudaGraphConditionalHandle handle,
-                  int use_handle, cudaStream_t st, bool flips) {
-    check_kernel<<<1, 1024, 0, st>>>(partial, n, ctl, first, handle, use_handle, flips ? 1 : 0);
+    bnorm_kernel<<<1, CHECK_THREADS, 0, st>>>(partial, n, ctl);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
 }

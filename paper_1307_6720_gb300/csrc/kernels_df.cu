@@ -8,6 +8,7 @@
 // to FP32, the right-hand side of the FP32 V-cycles.
 #include <algorithm>
 
+#include "check.cuh"
 #include "device_util.cuh"
 #include "df_bodies.cuh"
 #include "mhs_internal.h"
@@ -19,9 +20,10 @@ namespace {
 template <bool D3>
 __global__ void df_residual_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __restrict__ hi,
                                    const float* __restrict__ lo, const float* __restrict__ fh,
-                                   const float* __restrict__ fl, float* __restrict__ r32,
-                                   double* __restrict__ partial) {
+                                   const float* __restrict__ fl, float* __restrict__ r32, double* partial,
+                                   CheckArgs ck) {
     df_residual_body<D3>(g, cdf, hi, lo, fh, fl, r32, partial, blockIdx, gridDim);
+    check_last_block(ck, partial);
 }
 
 __global__ void df_correct_kernel(Geom g, int d3, const float* __restrict__ e, float* __restrict__ hi,
@@ -32,9 +34,10 @@ __global__ void df_correct_kernel(Geom g, int d3, const float* __restrict__ e, f
 template <bool FZ>
 __global__ void __launch_bounds__(32 * DQ_ROWS, 2)
 df_march_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __restrict__ hi, const float* __restrict__ lo,
-                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32,
-                double* __restrict__ partial) {
+                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32, double* partial,
+                CheckArgs ck) {
     df_march_body<false, FZ>(g, cdf, nullptr, hi, lo, nullptr, nullptr, fh, fl, r32, partial, blockIdx, gridDim);
+    check_last_block(ck, partial);
 }
 
 // One step of defect correction in one pass: the current pair plus e into
@@ -45,19 +48,20 @@ df_march_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __rest
 template <bool FZ>
 __global__ void __launch_bounds__(32 * DQ_ROWS, 2)
 df_step3_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __restrict__ e, DFPair pr,
-                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32,
-                double* __restrict__ partial) {
+                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32, double* partial,
+                CheckArgs ck) {
     const bool flip = *pr.flip != 0;
     df_march_body<true, FZ>(g, cdf, e, flip ? pr.hi[1] : pr.hi[0], flip ? pr.lo[1] : pr.lo[0], flip ? pr.hi[0] : pr.hi[1],
                         flip ? pr.lo[0] : pr.lo[1], fh, fl, r32, partial, blockIdx, gridDim);
+    check_last_block(ck, partial);
 }
 
 // The same on the lower-boundary plane: every thread corrects its node and
 // the four neighbours it reads.
 __global__ void __launch_bounds__(DF_BX * DF_BY)
 df_step2_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __restrict__ e, DFPair pr,
-                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32,
-                double* __restrict__ partial) {
+                const float* __restrict__ fh, const float* __restrict__ fl, float* __restrict__ r32, double* partial,
+                CheckArgs ck) {
     const bool flip = *pr.flip != 0;
     const float* __restrict__ hi = flip ? pr.hi[1] : pr.hi[0];
     const float* __restrict__ lo = flip ? pr.lo[1] : pr.lo[0];
@@ -93,6 +97,7 @@ df_step2_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, const float* __rest
     }
     const double s = block_sum(double(acc));
     if (threadIdx.x == 0 && threadIdx.y == 0) partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = s;
+    check_last_block(ck, partial);
 }
 
 __global__ void df_split_kernel(Geom g, int d3, const double* __restrict__ f, float* __restrict__ hi,
@@ -149,14 +154,15 @@ void launch_df_split(const Geom& g, int dim, const double* f, float* hi, float* 
 }
 
 int launch_df_residual(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* hi, const float* lo,
-                       const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st) {
+                       const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st,
+                       const CheckArgs& ck) {
     const int d3 = dim == 3;
     const dim3 grid = df_residual_grid(g, d3, max_blocks);
     if (d3 && use_df_quads(g))
-        (fh && fl ? df_march_kernel<false> : df_march_kernel<true>)<<<grid, dim3(DQ_X, DQ_ROWS), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial);
+        (fh && fl ? df_march_kernel<false> : df_march_kernel<true>)<<<grid, dim3(DQ_X, DQ_ROWS), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial, ck);
     else if (d3)
-        df_residual_kernel<true><<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial);
-    else df_residual_kernel<false><<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial);
+        df_residual_kernel<true><<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial, ck);
+    else df_residual_kernel<false><<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, hi, lo, fh, fl, r32, partial, ck);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
     return int(grid.x * grid.y * grid.z);
@@ -165,12 +171,12 @@ int launch_df_residual(const Geom& g, int dim, const PlaneCoefDF* cdf, const flo
 bool df_step_available(const Geom& g, int dim) { return dim == 2 || use_df_quads(g); }
 
 int launch_df_step(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* e, const DFPair& p, const float* fh,
-                   const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st) {
+                   const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st, const CheckArgs& ck) {
     const dim3 grid = df_residual_grid(g, dim == 3, max_blocks);
     if (dim == 3)
         (fh && fl ? df_step3_kernel<false> : df_step3_kernel<true>)<<<grid, dim3(DQ_X, DQ_ROWS), 0, st>>>(
-            g, cdf, e, p, fh, fl, r32, partial);
-    else df_step2_kernel<<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, e, p, fh, fl, r32, partial);
+            g, cdf, e, p, fh, fl, r32, partial, ck);
+    else df_step2_kernel<<<grid, dim3(DF_BX, DF_BY), 0, st>>>(g, cdf, e, p, fh, fl, r32, partial, ck);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
     return int(grid.x * grid.y * grid.z);

@@ -411,13 +411,13 @@ void glaunch_df_to_double(const GTable& t, cudaStream_t st) {
 
 void glaunch_bnorm(const GTable& t, cudaStream_t st) {
     if (!t.n) return;
-    g_bnorm_kernel<<<t.blocks, 1024, 0, st>>>(t.items, t.n);
+    g_bnorm_kernel<<<t.blocks, CHECK_THREADS, 0, st>>>(t.items, t.n);
     after_launch();
 }
 
 void glaunch_check(const GTable& t, int first, int gate, cudaStream_t st) {
     if (!t.n) return;
-    g_check_kernel<<<t.blocks, 1024, 0, st>>>(t.items, t.n, first, gate);
+    g_check_kernel<<<t.blocks, CHECK_THREADS, 0, st>>>(t.items, t.n, first, gate);
     after_launch();
 }
 

@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "check.cuh"
 #include "device_util.cuh"
 #include "line_body.cuh"
 #include "mg_bodies.cuh"
@@ -208,14 +209,16 @@ __global__ void residual_v4_kernel(Geom g, const PlaneCoef<float>* __restrict__ 
 
 template <typename T, bool D3, bool NORM>
 __global__ void residual_kernel(Geom g, const PlaneCoef<T>* __restrict__ coef, const T* __restrict__ u,
-                                const T* __restrict__ f, T* __restrict__ r, double* __restrict__ partial) {
+                                const T* __restrict__ f, T* __restrict__ r, double* partial, CheckArgs ck) {
     residual_body<T, D3, NORM>(g, coef, u, f, r, partial, blockIdx, gridDim);
+    if (NORM) check_last_block(ck, partial);
 }
 
 template <typename T, bool D3, bool NORM>
 __global__ void residual_red_kernel(Geom g, const PlaneCoef<T>* __restrict__ coef, const T* __restrict__ u,
-                                    const T* __restrict__ f, T* __restrict__ r, double* __restrict__ partial) {
+                                    const T* __restrict__ f, T* __restrict__ r, double* partial, CheckArgs ck) {
     residual_red_body<T, D3, NORM>(g, coef, u, f, r, partial, blockIdx, gridDim);
+    if (NORM) check_last_block(ck, partial);
 }
 
 template <typename T, bool D3>
@@ -443,16 +446,16 @@ void launch_smooth(const Geom& g, int dim, const PlaneCoef<T>* coef, T* u, const
 
 template <typename T>
 int launch_residual(const Geom& g, int dim, const PlaneCoef<T>* coef, const T* u, const T* f, T* r, double* partial,
-                    int max_blocks, cudaStream_t st, bool red) {
+                    int max_blocks, cudaStream_t st, bool red, const CheckArgs& ck) {
     const int d3 = dim == 3;
     if (red) {   // right after a red-black sweep: red nodes computed, black nodes 0
         const dim3 grid = residual_red_grid(g, d3, partial != nullptr, max_blocks);
         if (partial) {
-            if (d3) residual_red_kernel<T, true, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
-            else residual_red_kernel<T, false, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
+            if (d3) residual_red_kernel<T, true, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
+            else residual_red_kernel<T, false, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
         } else {
-            if (d3) residual_red_kernel<T, true, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
-            else residual_red_kernel<T, false, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
+            if (d3) residual_red_kernel<T, true, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
+            else residual_red_kernel<T, false, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
         }
         count_launches(1);
         MHS_CUDA(cudaGetLastError());
@@ -470,11 +473,11 @@ int launch_residual(const Geom& g, int dim, const PlaneCoef<T>* coef, const T* u
     }
     const dim3 grid = residual_grid(g, d3, partial != nullptr, max_blocks);
     if (partial) {
-        if (d3) residual_kernel<T, true, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
-        else residual_kernel<T, false, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
+        if (d3) residual_kernel<T, true, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
+        else residual_kernel<T, false, true><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
     } else {
-        if (d3) residual_kernel<T, true, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
-        else residual_kernel<T, false, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial);
+        if (d3) residual_kernel<T, true, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
+        else residual_kernel<T, false, false><<<grid, dim3(BX, BY), 0, st>>>(g, coef, u, f, r, partial, ck);
     }
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
@@ -589,7 +592,7 @@ int launch_lift_norm(const Geom& g3, const PlaneCoef<double>* coef, const double
     template void launch_fill<T>(T*, size_t, T, cudaStream_t);                                                 \
     template void launch_smooth<T>(const Geom&, int, const PlaneCoef<T>*, T*, const T*, cudaStream_t, int);    \
     template int launch_residual<T>(const Geom&, int, const PlaneCoef<T>*, const T*, const T*, T*, double*,    \
-                                    int, cudaStream_t, bool);                                                  \
+                                    int, cudaStream_t, bool, const CheckArgs&);                                \
     template void launch_restrict<T>(const Geom&, const Geom&, int, const T*, T*, T*, cudaStream_t, bool);           \
     template void launch_resid_restrict<T>(const Geom&, const Geom&, int, const PlaneCoef<T>*, const T*, const T*, \
                                            T*, T*, cudaStream_t);                                                 \

@@ -148,6 +148,17 @@ struct SolveCtl {
     int bodies;        // cycles run by a while body (the full-multigrid cycle of the prologue is not one)
 };
 
+// The convergence test at the end of a launch that forms norm partials
+// (check.cuh); ctl == nullptr: none.
+struct CheckArgs {
+    SolveCtl* ctl = nullptr;
+    unsigned* ticket = nullptr;   // 0 between launches
+    int first = 0;                // see check_body
+    int flips = 0;                // the launch moved the double-float iterate to the other pair
+    int use_handle = 0;
+    cudaGraphConditionalHandle handle = 0;
+};
+
 // One level of a multigrid sub-hierarchy solved inside a single CTA.
 template <typename T>
 struct SubLevel {
@@ -294,7 +305,8 @@ void launch_smooth(const Geom& g, int dim, const PlaneCoef<T>* coef, T* u, const
 // are stored as 0 and only the red nodes are computed (half the work)
 template <typename T>
 int launch_residual(const Geom& g, int dim, const PlaneCoef<T>* coef, const T* u, const T* f, T* r,
-                    double* partial, int max_blocks, cudaStream_t st, bool red = false);
+                    double* partial, int max_blocks, cudaStream_t st, bool red = false,
+                    const CheckArgs& ck = CheckArgs());
 // finish partial sums into *out (fixed order)
 void launch_norm_finish(const double* partial, int n, double* out, cudaStream_t st);
 template <typename T>
@@ -442,9 +454,6 @@ void launch_pair_sweep(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap
 
 // ---- control and sub-cycle (kernels_ctl.cu) ----
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st);
-// flips: the launch before it moved the double-float iterate to the other pair
-void launch_check(const double* partial, int n, SolveCtl* ctl, int first, cudaGraphConditionalHandle handle,
-                  int use_handle, cudaStream_t st, bool flips = false);
 size_t subcycle_smem_limit();
 // rows of 32 threads of the sub-cycle CTA of a hierarchy cut at a level with
 // `interior` interior nodes: small coarse problems pay mostly for block-wide
@@ -460,7 +469,8 @@ void launch_df_coef(const Geom& g, const PlaneCoef<double>* coef, PlaneCoefDF* c
 void launch_df_split(const Geom& g, int dim, const double* f, float* hi, float* lo, cudaStream_t st);
 // r32 = fh + fl - A (hi + lo) rounded to FP32, with per-block partial sums of r32^2; returns the partial count
 int launch_df_residual(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* hi, const float* lo,
-                       const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st);
+                       const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st,
+                       const CheckArgs& ck = CheckArgs());
 // (hi, lo) += e at interior nodes
 // the two double-float iterates and which is current (DFState); flip == nullptr: the first
 struct DFPair {
@@ -472,7 +482,8 @@ void launch_df_correct(const Geom& g, int dim, const float* e, float* hi, float*
 bool df_step_available(const Geom& g, int dim);
 // current pair + e into the other pair (faces copied), and its residual as launch_df_residual's
 int launch_df_step(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* e, const DFPair& p, const float* fh,
-                   const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st);
+                   const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st,
+                   const CheckArgs& ck = CheckArgs());
 // P = hi + lo (double) at every node
 void launch_df_to_double(const Geom& g, const DFPair& p, double* P, cudaStream_t st);
 // plane k = 0 of a 3D double-float pair from a 2D pair

@@ -564,7 +564,7 @@ double read_norm2(mhs_ctx* c, int slot) {
 //
 // One solve = lower-boundary prologue, while(cond) {lower-boundary cycle},
 // interior prologue, while(cond) {interior cycle}.  The convergence test is
-// check_kernel on the device; in graph mode it drives the conditional while
+// the last block of a residual launch (check.cuh); in graph mode it drives the conditional while
 // nodes, in eager mode the host reads the control block after each check.
 
 struct Enq {
@@ -584,7 +584,7 @@ static int lower_mode(const mhs_ctx* c, int mode) {
 
 // residual of the current iterate (FP64, or FP64 rounded into the FP32
 // right-hand side in mixed mode) with norm partials; returns their count
-static int residual_partials(mhs_ctx* c, Hierarchy& H, int mode, bool red = false) {
+static int residual_partials(mhs_ctx* c, Hierarchy& H, int mode, bool red = false, const CheckArgs& ck = CheckArgs()) {
     const Geom& g = H.g[0];
     LevelArrays<double>& A = H.d[0];
     const double N = double(g.interior());
@@ -598,11 +598,22 @@ static int residual_partials(mhs_ctx* c, Hierarchy& H, int mode, bool red = fals
         TimedScope t(c->timer, MHS_KT_RESID_MIXED, N * (8.0 + (fz ? 0.0 : 8.0) + 4.0), N * 70.0, c->stream,
                      H.dim == 3);
         return launch_df_residual(g, H.dim, H.df.coef, H.df.hi, H.df.lo, fz ? nullptr : H.df.fh,
-                                  fz ? nullptr : H.df.fl, H.s[0].f, c->ns.partial, c->ns.max_blocks, c->stream);
+                                  fz ? nullptr : H.df.fl, H.s[0].f, c->ns.partial, c->ns.max_blocks, c->stream, ck);
     }
     TimedScope t(c->timer, MHS_KT_RESID64, N * (16.0 + fb), N * fl * (red ? 0.5 : 1.0), c->stream, H.dim == 3);
     return launch_residual<double>(g, H.dim, A.coef, A.u, fz ? nullptr : A.f, A.r, c->ns.partial, c->ns.max_blocks,
-                                   c->stream, red);
+                                   c->stream, red, ck);
+}
+
+// the convergence test that ends a solve's residual launch
+static CheckArgs check_args(const Enq& e, SolveCtl* ctl, int first) {
+    CheckArgs ck;
+    ck.ctl = ctl;
+    ck.ticket = reinterpret_cast<unsigned*>(e.c->flag + 2);
+    ck.first = first;
+    ck.use_handle = e.graph ? 1 : 0;
+    ck.handle = e.hnd;
+    return ck;
 }
 
 static DFPair df_pair(mhs_ctx* c, Hierarchy& H) {
@@ -612,23 +623,24 @@ static DFPair df_pair(mhs_ctx* c, Hierarchy& H) {
 }
 
 // mixed mode: the correction added to the double-float iterate and the
-// residual of the result, as residual_partials forms it; returns the partials' count
-static int correct_and_residual(mhs_ctx* c, Hierarchy& H, bool& flips) {
+// residual of the result, as residual_partials forms it, with the convergence test
+static void correct_and_residual(mhs_ctx* c, Hierarchy& H, CheckArgs ck) {
     const Geom& g = H.g[0];
-    flips = df_step_available(g, H.dim);
-    if (!flips) {
+    if (!df_step_available(g, H.dim)) {
         TimedScope t(c->timer, MHS_KT_CORRECT, double(g.interior()) * 20.0, double(g.interior()) * 8.0, c->stream,
                      H.dim == 3);
         launch_df_correct(g, H.dim, H.s[0].u, H.df.hi, H.df.lo, c->stream);
         t.stop();
-        return residual_partials(c, H, MHS_MIXED);
+        residual_partials(c, H, MHS_MIXED, false, ck);
+        return;
     }
+    ck.flips = 1;
     const bool fz = H.dim == 3 && c->f_zero_finest;
     const double N = double(g.interior());
     TimedScope t(c->timer, MHS_KT_RESID_MIXED, N * (12.0 + 8.0 + (fz ? 0.0 : 8.0) + 4.0), N * 80.0, c->stream,
                  H.dim == 3);
-    return launch_df_step(g, H.dim, H.df.coef, H.s[0].u, df_pair(c, H), fz ? nullptr : H.df.fh,
-                          fz ? nullptr : H.df.fl, H.s[0].f, c->ns.partial, c->ns.max_blocks, c->stream);
+    launch_df_step(g, H.dim, H.df.coef, H.s[0].u, df_pair(c, H), fz ? nullptr : H.df.fh, fz ? nullptr : H.df.fl,
+                   H.s[0].f, c->ns.partial, c->ns.max_blocks, c->stream, ck);
 }
 
 static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
@@ -643,9 +655,7 @@ static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
         } else {
             for (int q = 0; q < c->opts.inner_cycles; ++q) vcycle<float>(c, H, 0);
         }
-        bool flips;
-        const int nb = correct_and_residual(c, H, flips);
-        launch_check(c->ns.partial, nb, ctl, 0, e.hnd, e.graph ? 1 : 0, c->stream, flips);
+        correct_and_residual(c, H, check_args(e, ctl, 0));
         return;
     }
     if ((c->opts.flags & MHS_FLAG_SEPARABLE) && sep_fp64_available(c)) {
@@ -658,8 +668,7 @@ static void cycle_body(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
     } else {
         vcycle<double>(c, H, 0);
     }
-    const int nb = residual_partials(c, H, e.mode, red_residual_cycle(c, H));
-    launch_check(c->ns.partial, nb, ctl, 0, e.hnd, e.graph ? 1 : 0, c->stream);
+    residual_partials(c, H, e.mode, red_residual_cycle(c, H), check_args(e, ctl, 0));
 }
 
 // First cycle of a solve by full multigrid (skipped with MHS_FLAG_NO_FMG):
@@ -676,14 +685,11 @@ static void fmg_cycle(const Enq& e, Hierarchy& H, SolveCtl* ctl) {
     if (e.mode == MHS_MIXED) {
         MHS_CUDA(cudaMemsetAsync(H.s[0].u, 0, g.n * sizeof(float), c->stream));
         fmg<float>(c, H, H.s[0].f);
-        bool flips;
-        const int nb = correct_and_residual(c, H, flips);
-        launch_check(c->ns.partial, nb, ctl, 2, e.hnd, e.graph ? 1 : 0, c->stream, flips);
+        correct_and_residual(c, H, check_args(e, ctl, 2));
         return;
     }
     fmg<double>(c, H, H.d[0].r);
-    const int nb = residual_partials(c, H, e.mode, red_residual_fmg(c, H));
-    launch_check(c->ns.partial, nb, ctl, 2, e.hnd, e.graph ? 1 : 0, c->stream);
+    residual_partials(c, H, e.mode, red_residual_fmg(c, H), check_args(e, ctl, 2));
 }
 
 static void prologue_2d(const Enq& e) {
@@ -700,9 +706,7 @@ static void prologue_2d(const Enq& e) {
             launch_df_split(g, 2, H.d[0].f, H.df.fh, H.df.fl, c->stream);
         }
         // with u = 0 the residual is the right-hand side: its norm is ||b||
-        const int nb = residual_partials(c, H, e.mode);
-        launch_bnorm(c->ns.partial, nb, c->ctl + 0, c->stream);
-        launch_check(c->ns.partial, nb, c->ctl + 0, 1, e.hnd, e.graph ? 1 : 0, c->stream);
+        residual_partials(c, H, e.mode, false, check_args(e, c->ctl + 0, 3));
     }
     // the first cycle's kernels are timed under their own kinds
     fmg_cycle(e, H, c->ctl + 0);
@@ -741,8 +745,7 @@ static void prologue_3d(const Enq& e) {
         }
         const int nl = launch_lift_norm(g, H.d[0].coef, H.d[0].u, c->ns.partial, c->stream);
         launch_bnorm(c->ns.partial, nl, c->ctl + 1, c->stream);
-        const int nb = residual_partials(c, H, e.mode);
-        launch_check(c->ns.partial, nb, c->ctl + 1, 1, e.hnd, e.graph ? 1 : 0, c->stream);
+        residual_partials(c, H, e.mode, false, check_args(e, c->ctl + 1, 1));
     }
     fmg_cycle(e, H, c->ctl + 1);
 }

@@ -2,9 +2,7 @@
 // bodies shared by the solver's own kernels (kernels_ctl.cu) and the
 // grouped launches over many instances (kernels_group.cu).
 //
-// check_body finishes a residual norm in a fixed summation order, forms the
-// relative residual ||b - A u|| / ||b|| (the stopping test of a multigrid
-// solve) and counts cycles.
+// (bnorm_body and check_body, the norms' finish: check.cuh)
 //
 // subcycle_body runs a complete V(nu1,nu2)-cycle over the coarse levels of
 // a hierarchy (from a cut-off level down to the coarsest) inside one CTA,
@@ -17,52 +15,11 @@
 
 #include <cmath>
 
+#include "check.cuh"
 #include "device_util.cuh"
 #include "mhs_internal.h"
 
 namespace mhs {
-
-// ||b|| of a solve from its norm partials; resets the control block
-__device__ __forceinline__ void bnorm_body(const double* __restrict__ partial, int n, SolveCtl* ctl) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) s += partial[b];
-    s = block_sum(s);
-    if (threadIdx.x == 0) {
-        ctl->bnorm = sqrt(s);
-        ctl->cycles = 0;
-        ctl->status = MHS_OK;
-        ctl->cont = 0;
-        ctl->bodies = 0;
-    }
-}
-
-// Convergence test after a cycle: finishes the residual norm in a fixed
-// order, updates the control block and returns (in thread 0) whether
-// another cycle is needed.  first = 1: the initial test; first = 2: after
-// the full-multigrid cycle of the prologue, which counts as a cycle only if
-// the initial test asked for one; first = 0: after a cycle.
-__device__ __forceinline__ int check_body(const double* __restrict__ partial, int n, SolveCtl* ctl, int first) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) s += partial[b];
-    s = block_sum(s);
-    int cont = 0;
-    if (threadIdx.x == 0) {
-        const double rn = sqrt(s);
-        const double b = ctl->bnorm;
-        const double rel = b > 0.0 ? rn / b : 0.0;
-        if (first == 0 || (first == 2 && ctl->cont)) ctl->cycles += 1;
-        if (first == 0) ctl->bodies += 1;
-        ctl->rel = rel;
-        if (first == 1) ctl->rel0 = rel;
-        cont = (b > 0.0 && rel >= ctl->tol && ctl->cycles < ctl->max_cycles) ? 1 : 0;
-        if (!isfinite(rn)) {
-            ctl->status = MHS_ERR_NONFINITE;
-            cont = 0;
-        }
-        ctl->cont = cont;
-    }
-    return cont;
-}
 
 // ---------------------------------------------------------------------------
 // one-CTA sub-cycle
