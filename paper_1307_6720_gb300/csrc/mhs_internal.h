@@ -452,6 +452,12 @@ void make_pair_map(CUtensorMap* map, const Geom& g, const float* base);
 void launch_pair_sweep(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap& tm_f,
                        const PlaneCoef<float>* coef, float* uout, int* err, cudaStream_t st);
 
+// the same on a lower-boundary level (kernels_pair2d.cu); gc, uc: the interpolation of the
+// coarse iterate added to u first (nullptr: none)
+template <typename T>
+void launch_lower_pair(const Geom& g, const PlaneCoef<T>* coef, const T* u, const T* f, T* out, const Geom* gc,
+                       const T* uc, cudaStream_t st);
+
 // ---- control and sub-cycle (kernels_ctl.cu) ----
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st);
 size_t subcycle_smem_limit();

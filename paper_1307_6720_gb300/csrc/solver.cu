@@ -305,18 +305,19 @@ static void smooth_n(mhs_ctx* c, Hierarchy& H, int l, const T* f, int n, bool fi
     if (fused && (n & 1)) MHS_CUDA(cudaMemcpyAsync(A.u, A.t, g.n * sizeof(T), cudaMemcpyDeviceToDevice, c->stream));
 }
 
-// Passes of two sweeps (kernels_pair.cu) that a V-cycle runs on level l
-// before and after its coarse-grid correction: FP32 3D levels large enough,
-// red-black smoothing.  A pass moves the iterate from u to its twin t or
-// back, so their sum is even and the cycle ends in u; sweeps left over run in
-// place.
+// Passes of two sweeps (kernels_pair.cu, kernels_pair2d.cu) that a V-cycle
+// runs on level l before and after its coarse-grid correction: lower-boundary
+// levels, and FP32 3D levels large enough with red-black smoothing.  A pass
+// moves the iterate from u to its twin t or back, so their sum is even and
+// the cycle ends in u; sweeps left over run in place.  On lower-boundary
+// levels the first pass after the correction interpolates it too.
 struct PairPasses {
     int pre = 0, post = 0;
 };
 template <typename T>
 static PairPasses pair_passes(const mhs_ctx* c, const Hierarchy& H, int l) {
     PairPasses p;
-    if (sizeof(T) == 8 || H.dim != 3 || use_zline(c) || (c->opts.flags & MHS_FLAG_NO_TMA) || !pair_level(H.g[l]))
+    if (H.dim == 3 && (sizeof(T) == 8 || use_zline(c) || (c->opts.flags & MHS_FLAG_NO_TMA) || !pair_level(H.g[l])))
         return p;
     p.pre = c->opts.nu1 / 2;
     p.post = c->opts.nu2 / 2;
@@ -325,24 +326,31 @@ static PairPasses pair_passes(const mhs_ctx* c, const Hierarchy& H, int l) {
 }
 
 // n sweeps of level l in a V-cycle, `passes` pairs of them out of place;
-// in_t: the iterate is in the twin (both ways)
+// in_t: the iterate is in the twin (both ways); correct: the first pass adds
+// the interpolation of the coarser level's iterate
 template <typename T>
 static void smooth_level(mhs_ctx* c, Hierarchy& H, int l, const T* f, int n, int passes, bool paired, bool& in_t,
-                         bool fine, double bytes, double flops) {
+                         bool fine, double bytes, double flops, bool correct = false) {
     if (!paired) {
         smooth_n<T>(c, H, l, f, n, fine, bytes, flops);
         return;
     }
-    LevelArrays<float>& A = H.s[l];
+    LevelArrays<T>& A = arrays<T>(H, l);
+    const int kind = sizeof(T) == 8 ? MHS_KT_SMOOTH64 : MHS_KT_SMOOTH32;
     for (int q = 0; q < passes; ++q) {
-        TimedScope t(c->timer, MHS_KT_SMOOTH32, bytes, 2.0 * flops, c->stream, fine);
-        launch_pair_sweep(H.g[l], in_t ? H.tp_t[l] : H.tp_u[l], H.tp_f[l], A.coef, in_t ? A.u : A.t, c->flag + 1,
-                          c->stream);
+        TimedScope t(c->timer, kind, bytes, 2.0 * flops, c->stream, fine);
+        if (H.dim == 2)
+            launch_lower_pair<T>(H.g[l], A.coef, in_t ? A.t : A.u, f, in_t ? A.u : A.t,
+                                 correct && q == 0 ? &H.g[l + 1] : nullptr, correct ? arrays<T>(H, l + 1).u : nullptr,
+                                 c->stream);
+        else
+            launch_pair_sweep(H.g[l], in_t ? H.tp_t[l] : H.tp_u[l], H.tp_f[l], H.s[l].coef,
+                              in_t ? H.s[l].u : H.s[l].t, c->flag + 1, c->stream);
         in_t = !in_t;
     }
     for (int q = 2 * passes; q < n; ++q) {
-        TimedScope t(c->timer, MHS_KT_SMOOTH32, bytes, flops, c->stream, fine);
-        launch_smooth<float>(H.g[l], H.dim, A.coef, in_t ? A.t : A.u, A.f, c->stream, c->opts.tile);
+        TimedScope t(c->timer, kind, bytes, flops, c->stream, fine);
+        launch_smooth<T>(H.g[l], H.dim, A.coef, in_t ? A.t : A.u, f, c->stream, c->opts.tile);
     }
 }
 
@@ -374,10 +382,11 @@ struct LevelOps {
 // the coarse-grid correction of level l from its residual: restriction of
 // the residual in A.r (unless the fused pass of FP32 levels has already
 // restricted it; red: A.r is a residual taken on red nodes only), the coarser
-// cycle, interpolation added to u (or to its twin, where the iterate then is)
+// cycle, interpolation added to u (or to its twin, where the iterate then is;
+// deferred: left to the smoothing that follows)
 template <typename T>
 static void coarse_correction(mhs_ctx* c, Hierarchy& H, int l, const LevelOps<T>& o, bool restricted,
-                              bool red = false, bool in_t = false) {
+                              bool red = false, bool in_t = false, bool deferred = false) {
     cudaStream_t st = c->stream;
     const bool dbl = sizeof(T) == 8;
     LevelArrays<T>& A = arrays<T>(H, l);
@@ -389,7 +398,7 @@ static void coarse_correction(mhs_ctx* c, Hierarchy& H, int l, const LevelOps<T>
         launch_restrict<T>(H.g[l], H.g[l + 1], H.dim, A.r, C.f, C.u, st, red);
     }
     vcycle<T>(c, H, l + 1);
-    {
+    if (!deferred) {
         TimedScope t(c->timer, dbl ? MHS_KT_PROLONG64 : MHS_KT_PROLONG32, (2 * N + Nc) * s, 4.0 * N, st, o.fine);
         launch_prolong<T>(H.g[l + 1], H.g[l], H.dim, C.u, in_t ? A.t : A.u, st);
     }
@@ -442,10 +451,11 @@ void vcycle(mhs_ctx* c, Hierarchy& H, int l) {
         // FP64 levels (bound by the FP64 pipe, which the fused pass would not relieve): the
         // residual on red nodes after the sweep, then the restriction
         TimedScope t(c->timer, MHS_KT_RESID64, sweep_bytes, o.N * o.res_flops, st, o.fine);
-        launch_residual<T>(g, H.dim, A.coef, A.u, o.f, A.r, nullptr, 0, st, red_residual_level(c, H));
+        launch_residual<T>(g, H.dim, A.coef, in_t ? A.t : A.u, o.f, A.r, nullptr, 0, st, red_residual_level(c, H));
     }
-    coarse_correction<T>(c, H, l, o, !dbl, dbl && red_residual_level(c, H), in_t);
-    smooth_level<T>(c, H, l, o.f, c->opts.nu2, pp.post, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops);
+    const bool deferred = H.dim == 2 && pp.post > 0;
+    coarse_correction<T>(c, H, l, o, !dbl, dbl && red_residual_level(c, H), in_t, deferred);
+    smooth_level<T>(c, H, l, o.f, c->opts.nu2, pp.post, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops, deferred);
 }
 
 // FP64 cycles of the finest level with the convergence test after the
@@ -484,9 +494,13 @@ bool red_residual_rotated(const mhs_ctx* c, const Hierarchy& H) {
 static void vcycle_rotated(mhs_ctx* c, Hierarchy& H) {
     const LevelOps<double> o(c, H, 0);
     const double sweep_bytes = o.N * (2 * o.s + o.fs);
-    coarse_correction<double>(c, H, 0, o, false, red_residual_rotated(c, H));
-    smooth_n<double>(c, H, 0, o.f, c->opts.nu2, o.fine, sweep_bytes, o.N * o.upd_flops);
-    smooth_n<double>(c, H, 0, o.f, c->opts.nu1, o.fine, sweep_bytes, o.N * o.upd_flops);
+    const PairPasses pp = pair_passes<double>(c, H, 0);
+    const bool paired = pp.pre + pp.post > 0, deferred = pp.post > 0;
+    bool in_t = false;
+    coarse_correction<double>(c, H, 0, o, false, red_residual_rotated(c, H), false, deferred);
+    smooth_level<double>(c, H, 0, o.f, c->opts.nu2, pp.post, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops,
+                         deferred);
+    smooth_level<double>(c, H, 0, o.f, c->opts.nu1, pp.pre, paired, in_t, o.fine, sweep_bytes, o.N * o.upd_flops);
 }
 
 // Levels whose red-black sweeps run out of place (u and its twin t taking

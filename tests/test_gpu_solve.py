@@ -598,3 +598,31 @@ def test_mixed_step_on_wide_levels(M, shape):
     M.mhs_group_destroy(g)
     M.mhs_destroy(h2)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("shape", [(67, 35, 5), (145, 81, 9), (129, 65, 5), (49, 113, 9)])
+def test_lower_boundary_pairs_equal_colour_passes(M, shape, mode):
+    """Lower-boundary levels smoothed in passes of two sweeps with the
+    interpolation inside (tiles of 16 x 16 nodes, ragged ends): the solution is
+    bitwise that of a group, which runs the colour passes and the
+    interpolation as launches of their own; V(2,2), V(1,1) and V(2,3)."""
+    nx, ny, nz = shape
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=(ny - 1) / (nx - 1), Lz=(nz - 1) / (nx - 1), alpha=0.3, xi_kind=1, xi_a=0.5,
+                   xi_kappa=1.0)
+    h = M.mhs_create(nx, ny, nz, pr["Lx"], pr["Ly"], pr["Lz"], pr["alpha"], _xi(M, pr))
+    M.mhs_set_lower_bz(h, S.magnetogram_random(nx, ny, 1.0, pr["Ly"], seed=nx))
+    h2 = M.mhs_create(17, 17, 17, 1.0, 1.0, 1.0, 0.2)
+    M.mhs_set_lower_bz(h2, S.magnetogram_random(17, 17, seed=1))
+    for nu in ((2, 2), (1, 1), (2, 3)):
+        M.mhs_set_options(h, nu1=nu[0], nu2=nu[1])
+        M.mhs_solve(h, 1e-10, mode)
+        P, Q = np.zeros((nz, ny, nx)), np.zeros((nz, ny, nx))
+        M.mhs_get_phi(h, P)
+        g = M.mhs_group_create([h, h2], mode, part_bytes=(1 << 64) - 1)
+        M.mhs_group_solve(g, 2, 1e-10)
+        M.mhs_get_phi(h, Q)
+        assert np.array_equal(P, Q), nu
+        M.mhs_group_destroy(g)
+    M.mhs_destroy(h2)
+    M.mhs_destroy(h)
