@@ -788,7 +788,7 @@ SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes) {
 // sum_j Sy[n][j] t1[k][j][m], mode solves, and back the same way.
 template <typename T>
 void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTables& tab, const T* f, T* t1, T* t2,
-                T* out, bool accumulate, std::vector<SepStage<T>>& stages) {
+                T* out, bool accumulate, std::vector<SepStage<T>>& stages, bool split = false) {
     const int nxi = g.nx - 2, nyi = g.ny - 2, nzi = dim == 3 ? g.nz - 2 : 1;
     if (nxi < 1 || nyi < 1 || nzi < 1) return;
     const long long pl = (long long)nxi * nyi;
@@ -829,9 +829,14 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
     if (tab.twx) {
         auto dst = [&](const DstArgs<T>& a) {
             SepStage<T> s;
-            s.kind = SEP_DST;
             s.dst = a;
-            dst_shape<T>(s.dst, s.grid, s.threads, s.smem);
+            if (split && tab.gx && tab.gy) {
+                s.kind = SEP_SPLIT;
+                s.digits = a.tw == tab.twx && a.L == g.nx - 1 ? tab.gx : tab.gy;
+            } else {
+                s.kind = SEP_DST;
+                dst_shape<T>(s.dst, s.grid, s.threads, s.smem);
+            }
             stages.push_back(s);
         };
         const int Lx = g.nx - 1, Ly = g.ny - 1;
@@ -869,6 +874,9 @@ template <typename T>
 void launch_stage(const SepStage<T>& s, cudaStream_t st) {
     switch (s.kind) {
     case SEP_DST: launch_dst_stage<T>(s, st); return;
+    case SEP_SPLIT:
+        if constexpr (sizeof(T) == 8) launch_dst_split(s.dst, s.digits, st);
+        return;
     case SEP_GEMM: gemm_kernel<T><<<s.grid, s.threads, 0, st>>>(s.gemm); break;
     case SEP_SCAN: {
         static bool configured = false;   // per template instance
@@ -910,9 +918,9 @@ namespace {
 
 template <typename T>
 void level_solve(mhs_ctx* c, const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTables& tab, const T* f,
-                 T* t1, T* t2, T* out, bool accumulate) {
+                 T* t1, T* t2, T* out, bool accumulate, bool split = false) {
     std::vector<SepStage<T>> stages;
-    plan_level<T>(g, dim, coef, tab, f, t1, t2, out, accumulate, stages);
+    plan_level<T>(g, dim, coef, tab, f, t1, t2, out, accumulate, stages, split);
     for (const SepStage<T>& s : stages) launch_stage<T>(s, c->stream);
 }
 
@@ -1113,6 +1121,21 @@ void sep_tables(mhs_ctx* c, Hierarchy& H, int l) {
         t.twy = make_twiddles<T>(g.ny - 1, &tb);
         c->allocations.push_back(t.twy);
         c->dev_bytes += round_up(tb, 256);
+        // the direct solves of the finest level (the lower boundary's lines are as long as the volume's)
+        if (sizeof(T) == 8 && l == 0 && split_length(g.nx - 1) && split_length(g.ny - 1)) {
+            const std::vector<SepTables>& twin = tables_of<T>(H.dim == 2 ? c->h3 : c->h2);
+            const SepTables o = twin.empty() ? SepTables{} : twin[0];
+            auto digits = [&](int n, void* have) {
+                if (have) return have;
+                size_t bytes = 0;
+                void* p = make_split_table(n, &bytes);
+                c->allocations.push_back(p);
+                c->dev_bytes += round_up(bytes, 256);
+                return p;
+            };
+            t.gx = digits(g.nx - 1, o.gx);
+            t.gy = digits(g.ny - 1, o.gy ? o.gy : g.ny == g.nx ? t.gx : nullptr);
+        }
     } else {
         t.sx = upload(sine(g.nx));
         t.sy = upload(sine(g.ny));
@@ -1218,7 +1241,7 @@ bool sep_fp64_available(const mhs_ctx* c) { return sep_level_ok(c->h3.g[0]); }
 // latest check (in A.r, consumed), the level's twin t as scratch.
 void sep_correct64(mhs_ctx* c, Hierarchy& H) {
     LevelArrays<double>& A = H.d[0];
-    level_solve<double>(c, H.g[0], H.dim, A.coef, tables<double>(H, 0), A.r, A.t, A.r, A.u, true);
+    level_solve<double>(c, H.g[0], H.dim, A.coef, tables<double>(H, 0), A.r, A.t, A.r, A.u, true, true);
 }
 
 template void sep_tables<double>(mhs_ctx*, Hierarchy&, int);

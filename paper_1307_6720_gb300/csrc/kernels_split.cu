@@ -1,0 +1,301 @@
+// FP64 sine transforms of long lines on the tensor cores, by exact splitting.
+//
+// The FP64 pipe (two lanes per clock and SM) is the bound of the fast
+// transforms: 26 FP64 instructions per element at 257 nodes.  Here a line is a
+// dense product with the folded sine matrices (half the side: the sums of
+// mirrored elements give the odd results, the differences the even ones) in
+// fixed point, formed from exact small integer products (Ozaki, Ogita, Oishi
+// and Rump, Numer. Algorithms 59, 2012):
+//
+// - the folded elements become integers of up to 2^55 relative to their line's
+//   largest exponent, x = sum_i a_i 256^(6-i), seven digits in [-128, 127] (the
+//   first up to 128); likewise the matrix entries, scaled by 2^55;
+// - digits are exact in FP16, a product of two is at most 2^14, and a sum of up
+//   to 7 x 128 of them stays below 2^24, so FP32 accumulation is exact; the
+//   products with i + j = d share the accumulator of order d, d <= 7 (34
+//   products of digit matrices; those left out lie below 2^-59 of the line's
+//   largest element each);
+// - the eight integers of a result are put together in 64 bits, rounded once
+//   and written as a double, all by integer instructions (conversions between
+//   64-bit integers and doubles run at the FP64 pipe's rate: 650 us a pass);
+//   what is left to the FP64 pipe is the folding and the scaling of the last pass.
+//
+// mma.sync (m16n8k16) rather than tcgen05: the eight accumulators of a result
+// meet in one thread and the digits are made in the fragments' layout.  Two
+// warps share the digits of 16 lines of one parity in shared memory (29 KB at
+// 256 cells), each forms half of their results, two column tiles at a time, so
+// that three blocks (12 warps) fit an SM; the matrices' digits stream from L2
+// in fragment order, one tile ahead.  Four tiles per warp with two warps' worth
+// of registers and lines of its own ran at two warps per scheduler: 550 us.
+//
+// One pass over 255^3, in place of 733 us of the fast transform: 374 us to 420 us
+// (strided stores), tensor pipe 67 % busy; the rest is the digits and putting
+// results together (2.7 other instructions per product).  Over one plane of
+// 255^2, where the results are spread over blocks: 17.5 us, was 27 us.
+//
+// Against the exact solution of the discrete equations, one direct step
+// (four transforms in each problem), fast transforms -> these, 2-norm:
+// 129^3 lower boundary 2.4e-15 -> 0.8e-15, volume 1.89e-14 -> 1.84e-14 (the
+// tridiagonal solves'); 257 x 129 x 17 3.3e-15 -> 1.0e-15 and 4.7e-15 -> 2.4e-15;
+// 257 x 257 x 33 6.0e-15 -> 1.4e-15 and 8.7e-15 -> 4.9e-15, its residual
+// 4.5e-14 -> 2.6e-15.  Lines with an infinity or NaN become NaN.
+#include <cuda_fp16.h>
+
+#include <cmath>
+#include <vector>
+
+#include "device_util.cuh"
+#include "dst_body.cuh"
+#include "mhs_internal.h"
+#include "solver.h"
+
+namespace mhs {
+
+namespace {
+
+constexpr int DIG = 7;               // digits
+constexpr int ORDERS = 8;            // of products of digits that are kept
+constexpr int STEP = DIG * 128 + 4;   // words of a k step's digits of 16 lines (four more than they fill: lanes on other banks)
+constexpr int SW = 4;                // warps of a block, two to 16 lines
+constexpr int TILES = 2;             // column tiles of 8 results that a warp forms at a time
+constexpr long long BIAS = 0x80808080808080LL;   // 128 in every digit
+
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint4& a, const uint2& b) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+}
+
+// biased exponent (subnormals as exponent 1)
+__device__ __forceinline__ int expo(double x) {
+    const int e = (__double2hiint(x) >> 20) & 0x7ff;
+    return e ? e : 1;
+}
+
+// x 2^(1077 - emax) rounded to an integer (|.| <= 2^55 for exponents up to emax)
+__device__ __forceinline__ long long fixed(double x, int emax) {
+    const unsigned hi = unsigned(__double2hiint(x)), ex = (hi >> 20) & 0x7ffu;
+    const unsigned long long m =
+        static_cast<unsigned long long>(__double_as_longlong(x) & 0xfffffffffffffLL) | (ex ? 0x10000000000000ull : 0ull);
+    const int sh = emax - int(ex ? ex : 1u);
+    const long long q = static_cast<long long>(sh > 60 ? 0ull : ((m << 2) + ((1ull << sh) >> 1)) >> sh);
+    return (hi >> 31) ? -q : q;
+}
+
+// v 2^k as a double, rounded to nearest (ties away)
+__device__ __forceinline__ double widened(long long v, int k) {
+    const unsigned long long m0 = v < 0 ? 0ull - static_cast<unsigned long long>(v) : static_cast<unsigned long long>(v);
+    if (m0 == 0) return 0.0;
+    const int lz = __clzll(static_cast<long long>(m0));
+    const unsigned long long m = (m0 << lz) >> 1;                 // leading bit 62
+    const unsigned long long r = (m + (1ull << 9)) >> 10;         // 53 bits, or 2^53 after a carry
+    const int e = 1023 + k + 63 - lz;                              // exponent field of the leading bit
+    if (e < 1 || e > 2045) return scalbn(double(v), k);           // near the ends of the range
+    const unsigned long long bits = (static_cast<unsigned long long>(e - 1) << 52) + r;   // the leading bit (and a carry) add to it
+    return __longlong_as_double(static_cast<long long>(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+// lines of N - 1 elements, N = 32 KS; tab: the matrices' digits in fragment
+// order [parity][column tile][k step][digit][lane]
+template <int KS>
+__global__ void __launch_bounds__(32 * SW, 3) dst_split_kernel(DstArgs<double> a, const uint2* __restrict__ tab) {
+    constexpr int Ko = 16 * KS, N = 2 * Ko;
+    constexpr int NG = Ko / 16 / TILES;   // groups of tiles of a warp
+    constexpr int EP = Ko / 32;   // folded elements of a lane
+    extern __shared__ __align__(16) unsigned char split_smem[];
+    __shared__ int s_e[SW / 2][16];
+    const int lane = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1, w = threadIdx.x >> 6;
+    unsigned* A = reinterpret_cast<unsigned*>(split_smem) + w * (KS * STEP);
+    const long long total = (long long)a.lines * a.planes, first = ((long long)blockIdx.x * (SW / 2) + w) * 16;
+    const int g = lane >> 2, t4 = lane & 3;
+    // the two lines whose results this thread holds
+    long long base[2];
+    bool live[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const long long gl = first + g + 8 * h;
+        live[h] = gl < total;
+        const long long pl = live[h] ? gl / a.lines : 0, l = live[h] ? gl - pl * a.lines : 0;
+        base[h] = pl * a.out_plane + l * a.out_line;
+    }
+    // all results, or (few lines, gridDim.y = 2 NG) one group of each warp
+    const bool one = gridDim.y > 1;
+    const int par0 = one ? blockIdx.y & 1 : 0, par1 = one ? par0 : 1;
+    const int ng0 = one ? (blockIdx.y >> 1) * 2 + half : half * NG, ng1 = one ? ng0 + 1 : ng0 + NG;
+    for (int par = par0; par <= par1; ++par) {
+        // digits of the folded lines, each line loaded while the one before is worked on
+        auto load_line = [&](int r, double(&lo)[EP], double(&hi)[EP]) {
+            const long long gl = first + r;
+            const bool on = gl < total;
+            const long long pl = on ? gl / a.lines : 0;
+            const double* x = a.in + pl * a.in_plane + (on ? gl - pl * a.lines : 0) * a.in_line;
+#pragma unroll
+            for (int u = 0; u < EP; ++u) {
+                const int i = lane * EP + u, j = N - 2 - i;
+                lo[u] = on ? x[i] : 0.0;
+                // (the middle element is its own mirror: it counts once, in the sums)
+                hi[u] = !on ? 0.0 : j != i ? x[j] : par ? lo[u] : 0.0;
+            }
+        };
+        double lo[EP], hi[EP];
+        load_line(8 * half, lo, hi);
+#pragma unroll 1
+        for (int r = 8 * half; r < 8 * half + 8; ++r) {
+            double f[EP];
+            int e = 1;
+#pragma unroll
+            for (int u = 0; u < EP; ++u) {
+                f[u] = par ? lo[u] - hi[u] : lo[u] + hi[u];
+                e = max(e, expo(f[u]));
+            }
+            if (r < 8 * half + 7) load_line(r + 1, lo, hi);
+            e = int(__reduce_max_sync(0xffffffffu, unsigned(e)));
+            unsigned long long q[EP];
+#pragma unroll
+            for (int u = 0; u < EP; ++u) q[u] = static_cast<unsigned long long>(fixed(f[u], e) + BIAS);
+            if (lane == 0) s_e[w][r] = e;
+            const __half2 off = __halves2half2(__ushort_as_half(0xe480), __ushort_as_half(0xe480));   // -1152
+#pragma unroll
+            for (int u = 0; u < EP; u += 2) {
+                const int k = lane * EP + u, ks = k >> 4, kk = k & 15;
+                const int word = ks * STEP + (((r & 7) * 4 + ((kk & 7) >> 1)) << 2) + (r >> 3) + 2 * (kk >> 3);
+#pragma unroll
+                for (int s = 0; s < DIG; ++s) {
+                    const int b = DIG - 1 - s;   // byte of digit s
+                    const unsigned u0 = b < 4 ? unsigned(q[u]) : unsigned(q[u] >> 32);
+                    const unsigned u1 = b < 4 ? unsigned(q[u + 1]) : unsigned(q[u + 1] >> 32);
+                    // 1024 + byte, twice (the first digit may be 128: nine bits)
+                    const unsigned h = s == 0 ? __byte_perm(u0, u1, 0x7632) | 0x64006400u
+                                              : __byte_perm(__byte_perm(u0, u1, (b & 3) | ((4 + (b & 3)) << 4)), 0x64646464u, 0x4140);
+                    const __half2 d = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
+                    A[word + s * 128] = *reinterpret_cast<const unsigned*>(&d);
+                }
+            }
+        }
+        __syncthreads();
+        for (int ng = ng0; ng < ng1; ++ng) {
+            float acc[TILES][ORDERS][4];
+#pragma unroll
+            for (int n = 0; n < TILES; ++n)
+#pragma unroll
+                for (int d = 0; d < ORDERS; ++d)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) acc[n][d][c] = 0.f;
+            // column tile n of k step ks, its digits loaded one tile ahead
+            const uint2* bt = tab + (size_t(par) * (Ko / 8) + ng * TILES) * KS * DIG * 32 + lane;
+            auto load_b = [&](uint2(&v)[DIG], int ks, int n) {
+#pragma unroll
+                for (int s = 0; s < DIG; ++s) v[s] = __ldg(bt + ((n * KS + ks) * DIG + s) * 32);
+            };
+            uint2 bn[DIG];
+            load_b(bn, 0, 0);
+#pragma unroll 1
+            for (int ks = 0; ks < KS; ++ks) {
+                uint4 av[DIG];
+#pragma unroll
+                for (int s = 0; s < DIG; ++s)
+                    av[s] = *reinterpret_cast<const uint4*>(A + ks * STEP + s * 128 + 4 * lane);
+#pragma unroll
+                for (int n = 0; n < TILES; ++n) {
+                    uint2 bv[DIG];
+#pragma unroll
+                    for (int s = 0; s < DIG; ++s) bv[s] = bn[s];
+                    if (n + 1 < TILES) load_b(bn, ks, n + 1);
+                    else if (ks + 1 < KS) load_b(bn, ks + 1, 0);
+#pragma unroll
+                    for (int i = 0; i < DIG; ++i)
+#pragma unroll
+                        for (int j = 0; j < DIG && i + j < ORDERS; ++j) mma16816(acc[n][i + j], av[i], bv[j]);
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < TILES; ++n)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const int h = c >> 1, col = (ng * TILES + n) * 8 + 2 * t4 + (c & 1), m = 2 * col + par;
+                    if (!live[h] || m > N - 2) continue;
+                    auto in = [&](int d) { return static_cast<long long>(__float2int_rn(acc[n][d][c])); };
+                    const long long top = (in(0) << 24) + (in(1) << 16) + (in(2) << 8) + in(3);
+                    const long long low = (in(4) << 16) + (in(5) << 8) + in(6) + (in(7) >> 8);
+                    const int e = s_e[w][g + 8 * h];
+                    // 256^7 2^-55 times 2^(e - 1077) of the elements: 2^(e - 1076)
+                    double v = widened((top << 16) + ((low + 128) >> 8), e - 1076);
+                    if (e == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
+                    double* o = a.out + base[h] + (long long)m * a.out_elem;
+                    *o = a.scale == 1.0 && !a.accumulate ? v : dst_result(a.scale, v, a.accumulate != 0, a.accumulate ? *o : 0.0);
+                }
+        }
+        __syncthreads();
+    }
+}
+
+template <int KS>
+void launch_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
+    static bool attr = false;
+    constexpr int smem = SW / 2 * KS * STEP * 4;
+    if (!attr) {
+        MHS_CUDA(cudaFuncSetAttribute(dst_split_kernel<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        attr = true;
+    }
+    const long long total = (long long)a.lines * a.planes;
+    const unsigned blocks = unsigned((total + 8 * SW - 1) / (8 * SW));
+    // up to a block per SM (4864 lines): a group of results per block, their lines' digits made by each
+    // (255 lines: 17.5 us; the same in eight blocks 130 us)
+    const dim3 grid(blocks, blocks <= 152 ? 2 * KS / TILES : 1);
+    dst_split_kernel<KS><<<grid, 32 * SW, smem, st>>>(a, static_cast<const uint2*>(tab));
+    count_launches(1);
+    MHS_CUDA(cudaGetLastError());
+}
+
+}  // namespace
+
+// 512 cells: the digits of a parity (58 KB for 16 lines) would leave one block per SM; 64: a fast transform of six
+// stages, a sixth of a pass over 128 cells in FP64 work, was left as it is
+bool split_length(int N) { return N == 128 || N == 256; }
+
+// sin(pi q / N) 2^55 as an integer
+static long long sine55(long long q, int N) {
+    return llrintl(sinl(3.14159265358979323846264338327950288L * (long double)q / (long double)N) * 36028797018963968.0L);
+}
+
+// digits of the folded sine matrices of N cells in fragment order (B of
+// m16n8k16: lane (g, t) holds rows 2t, 2t + 1 and 2t + 8, 2t + 9 of column g)
+void* make_split_table(int N, size_t* bytes) {
+    const int Ko = N / 2, KS = Ko / 16;
+    std::vector<uint2> tab(size_t(2) * (Ko / 8) * KS * DIG * 32);
+    std::vector<long long> sines(2 * N);
+    for (int q = 0; q < 2 * N; ++q) sines[q] = sine55(q, N);
+    auto digits = [&](int par, int i, int p) -> unsigned long long {   // of element i of result p, biased
+        const int m = 2 * p + 1 + par;                                  // mode
+        if (m > N - 1 || (par && i >= Ko - 1)) return BIAS;             // padding: zero
+        return static_cast<unsigned long long>(sines[size_t(m) * (i + 1) % (2 * N)] + BIAS);
+    };
+    unsigned short half_of[257];   // a digit (biased by 128; the first may be 128) as FP16
+    for (int q = 0; q <= 256; ++q) half_of[q] = __half_as_ushort(__float2half(float(q - 128)));
+    for (int par = 0; par < 2; ++par)
+        for (int nt = 0; nt < Ko / 8; ++nt)
+            for (int ks = 0; ks < KS; ++ks)
+                for (int l = 0; l < 32; ++l) {
+                    const int g = l >> 2, t = l & 3;
+                    unsigned long long d[4];
+                    for (int r = 0; r < 4; ++r) d[r] = digits(par, ks * 16 + 2 * t + (r & 1) + 8 * (r >> 1), nt * 8 + g);
+                    for (int s = 0; s < DIG; ++s) {
+                        const int sh = 8 * (DIG - 1 - s);
+                        auto digit = [&](int r) { return unsigned(half_of[s ? (d[r] >> sh) & 255 : d[r] >> sh]); };
+                        auto pack = [&](int r) { return digit(r) | (digit(r + 1) << 16); };
+                        tab[(((size_t(par) * (Ko / 8) + nt) * KS + ks) * DIG + s) * 32 + l] = make_uint2(pack(0), pack(2));
+                    }
+                }
+    void* p = nullptr;
+    MHS_CUDA(cudaMalloc(&p, tab.size() * sizeof(uint2)));
+    MHS_CUDA(cudaMemcpy(p, tab.data(), tab.size() * sizeof(uint2), cudaMemcpyHostToDevice));
+    *bytes = tab.size() * sizeof(uint2);
+    return p;
+}
+
+void launch_dst_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
+    if (a.L == 128) launch_split<4>(a, tab, st);
+    else launch_split<8>(a, tab, st);
+}
+
+}  // namespace mhs

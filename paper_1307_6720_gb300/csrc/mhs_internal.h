@@ -111,6 +111,7 @@ struct SepTables {
     void *mux = nullptr, *muy = nullptr;
     void *twx = nullptr, *twy = nullptr;
     void *sx = nullptr, *sy = nullptr;
+    void *gx = nullptr, *gy = nullptr;   // digits of the folded matrices of the split transforms (kernels_split.cu)
     void *fx = nullptr, *fy = nullptr;   // folded sine matrices of the plane transforms (kernels_sep.cu)
     void *inv = nullptr, *sup = nullptr;
     bool ready = false;
@@ -355,6 +356,11 @@ struct DstArgs {
 };
 template <typename T>
 void* make_twiddles(int L, size_t* bytes = nullptr);
+// FP64 lines as exact digit products on the tensor cores (kernels_split.cu): lengths it serves, the
+// digits of a length's matrices, one transform
+bool split_length(int N);
+void* make_split_table(int N, size_t* bytes);
+void launch_dst_split(const DstArgs<double>& a, const void* digits, cudaStream_t st);
 
 // ---- stages of one separable solve (kernels_sep.cu, kernels_dst.cu) ----
 // C_b = scale A_b B_b (+ C_b with accumulate), b < batch, row-major with
@@ -400,7 +406,7 @@ struct PlaneArgs {
     T scale = T(1);
     int accumulate = 0;
 };
-enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4, SEP_PLANE = 5 };
+enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4, SEP_PLANE = 5, SEP_SPLIT = 6 };
 // one kernel launch of a separable solve with its launch shape
 template <typename T>
 struct SepStage {
@@ -412,6 +418,7 @@ struct SepStage {
     GemmArgs<T> gemm;
     ModeArgs<T> mode;
     PlaneArgs<T> plane;
+    const void* digits = nullptr;   // SEP_SPLIT: dst with these
 };
 // launch shape of a sine-transform stage (sets a.pairs)
 template <typename T>

@@ -626,3 +626,37 @@ def test_lower_boundary_pairs_equal_colour_passes(M, shape, mode):
         M.mhs_group_destroy(g)
     M.mhs_destroy(h2)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(129, 129, 9), (129, 257, 33), (257, 129, 17), (257, 257, 17)])
+def test_direct_fp64_steps_on_long_lines(M, shape):
+    """The FP64 direct step with lines of 128 and 256 cells (few lines: results
+    spread over blocks; many lines; a ragged last block): one step is as
+    accurate as the arithmetic allows, and scaling by a power of two scales
+    every bit.  Tolerance: four transforms of 2^-52 each per sqrt(log2 n)
+    stage, and the elimination's nz steps, all in units of 2^-53."""
+    nx, ny, nz = shape
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=(ny - 1) / (nx - 1), Lz=(nz - 1) / (nx - 1), alpha=0.5, xi_kind=1, xi_a=0.5,
+                   xi_kappa=1.0)
+    tol = (4 * 2 * 8 + nz) * 2.0**-53
+    h = M.mhs_create(nx, ny, nz, pr["Lx"], pr["Ly"], pr["Lz"], pr["alpha"], _xi(M, pr))
+    M.mhs_set_options(h, flags=M.MHS_FLAG_SEPARABLE)
+
+    def solve(bz):
+        M.mhs_set_lower_bz(h, bz)
+        info = M.mhs_solve(h, 1e-9, 0)
+        assert info["cycles_3d"] <= 1
+        P = np.zeros((nz, ny, nx))
+        M.mhs_get_phi(h, P)
+        return P
+
+    noise = np.random.default_rng(nx + ny).standard_normal((ny, nx))
+    spot = np.zeros((ny, nx))
+    spot[ny // 3, nx // 5] = 1.0
+    for bz in (noise, spot):
+        P, E = solve(bz), exact.exact_solution(pr, bz)
+        assert np.linalg.norm(P - E) <= tol * np.linalg.norm(E)
+        assert np.linalg.norm(P[0] - E[0]) <= tol * np.linalg.norm(E[0])
+        assert np.array_equal(solve(bz * 2.0**300), P * 2.0**300)
+        assert np.array_equal(solve(bz * 2.0**-300), P * 2.0**-300)
+    M.mhs_destroy(h)
