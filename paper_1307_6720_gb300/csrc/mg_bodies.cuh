@@ -302,9 +302,16 @@ __device__ __forceinline__ void prolong_body(const Geom& gc, const Geom& gf, con
 // coarse iterate is zeroed at the same nodes.  RX = 32 coarse nodes along x
 // (threads 32 x 8, one per coarse node in the last step).  The V-cycles run
 // it on FP32 levels, which are bound by memory traffic; on FP64 levels the
-// FP64 pipe is the bound and the pass saves no FP64 operation.  Blocks of
-// RR_THREADS threads; every thread must call it.
-constexpr int RR_X = 32, RR_Y = 8, RR_THREADS = 256;
+// FP64 pipe is the bound and the pass saves no FP64 operation.
+//
+// A plane's step is two barriers and the latency of its loads.  So each of the
+// 17 x 17 quads of the window belongs to one thread (ten warps; with 256 threads
+// 33 quads took a second round), which keeps its column of planes in registers
+// and loads the next plane's values before the present one is restricted:
+// 513 x 513 x 257 180 us, was 277 us (its traffic takes 85 us), 257^3 52 us, was
+// 65 us; the number of chunks changes little (456 to 1824 blocks: 252 to 178 us).
+// Blocks of RR_THREADS threads; every thread must call it.
+constexpr int RR_X = 32, RR_Y = 8, RR_THREADS = 320;
 
 template <typename T, bool D3>
 __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& gc, const PlaneCoef<T>* __restrict__ coef,
@@ -321,43 +328,44 @@ __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& 
     const int fy0 = 2 * Jb - 1;                            // first window row
     const int x0 = 2 * Ib - 2;                             // first quad column: one node left of the window
     const int I = Ib + tx, J = Jb + ty;
-    const bool node = I <= gc.nx - 2 && J <= gc.ny - 2;
-    // residual of the quad (x0 + 4 q .. + 3, fy0 + y) of fine plane kf into rw (0 off the interior)
-    auto resid_quad = [&](int q, int y, int kf, const PlaneCoef<T>& c) {
-        const int i0 = x0 + 4 * q, j = fy0 + y;
-        T res[4] = {T(0), T(0), T(0), T(0)};
-        if (j <= gf.ny - 2 && i0 <= gf.nx - 2) {
-            const size_t o = at(gf, i0, j, kf);
-            T cc[4], nn[4], ss[4], uu[4], dd[4], ff[4];
-            if constexpr (sizeof(T) == 4) {
-                // the quad lies inside the padded row (px a multiple of four, i0 < nx)
-                auto ld4 = [](const T* ptr, T* out) {
-                    const float4 v = *reinterpret_cast<const float4*>(ptr);
-                    out[0] = v.x, out[1] = v.y, out[2] = v.z, out[3] = v.w;
-                };
-                ld4(u + o, cc);
-                ld4(u + o + gf.px, nn);
-                ld4(u + o - gf.px, ss);
-                if (D3) {
-                    ld4(u + o + gf.plane, uu);
-                    ld4(u + o - gf.plane, dd);
-                }
-                if (f) ld4(f + o, ff);
-            } else {
+    const bool node = ty < RR_Y && I <= gc.nx - 2 && J <= gc.ny - 2;
+    // this thread's quad of the window, (x0 + 4 q .. + 3, fy0 + y): its own column of planes in
+    // registers, the next plane's values loaded while the present one is restricted
+    const int y = tid / NQ, q = tid - y * NQ, i0 = x0 + 4 * q, j = fy0 + y;
+    const bool live = tid < WY * NQ && j <= gf.ny - 2 && i0 <= gf.nx - 2;
+    T dd[4], cc[4], uu[4], nn[4], ss[4], ff[4], west = T(0), east = T(0);
+    auto ld4 = [](const T* ptr, T(&out)[4]) {
+        if constexpr (sizeof(T) == 4) {
+            // the quad lies inside the padded row (px a multiple of four, i0 < nx)
+            const float4 v = *reinterpret_cast<const float4*>(ptr);
+            out[0] = v.x, out[1] = v.y, out[2] = v.z, out[3] = v.w;
+        } else {
 #pragma unroll
-                for (int l = 0; l < 4; ++l) {
-                    cc[l] = u[o + l];
-                    nn[l] = u[o + l + gf.px];
-                    ss[l] = u[o + l - gf.px];
-                    if (D3) {
-                        uu[l] = u[o + l + gf.plane];
-                        dd[l] = u[o + l - gf.plane];
-                    }
-                    if (f) ff[l] = f[o + l];
-                }
-            }
-            const T west = i0 > 0 ? u[o - 1] : T(0);
-            const T east = i0 + 3 <= gf.nx - 2 ? u[o + 4] : T(0);
+            for (int l = 0; l < 4; ++l) out[l] = ptr[l];
+        }
+    };
+    // the rest of plane kf, whose centre quad is there
+    auto load_rest = [&](int kf) {
+        if (!live) return;
+        const size_t o = at(gf, i0, j, kf);
+        if (D3) ld4(u + o + gf.plane, uu);
+        ld4(u + o + gf.px, nn);
+        ld4(u + o - gf.px, ss);
+        if (f) ld4(f + o, ff);
+        west = i0 > 0 ? u[o - 1] : T(0);
+        east = i0 + 3 <= gf.nx - 2 ? u[o + 4] : T(0);
+    };
+    auto load_first = [&](int kf) {
+        if (!live) return;
+        const size_t o = at(gf, i0, j, kf);
+        if (D3) ld4(u + o - gf.plane, dd);
+        ld4(u + o, cc);
+    };
+    // residual of the loaded plane kf into rw (0 off the interior), then the loads of plane kf + 1
+    auto resid_plane = [&](int kf, bool more) {
+        const PlaneCoef<T> c = coef[kf];
+        T res[4] = {T(0), T(0), T(0), T(0)};
+        if (live) {
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 const int i = i0 + l;
@@ -371,23 +379,26 @@ __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& 
                 res[l] = fma(-c.d, cc[l], v);
             }
         }
+        if (tid < WY * NQ) {
 #pragma unroll
-        for (int l = 0; l < 4; ++l) rw[y][4 * q + l] = res[l];
-    };
-    auto resid_plane = [&](int kf) {
-        const PlaneCoef<T> c = coef[kf];
-        for (int e = tid; e < WY * NQ; e += RR_THREADS) {
-            const int y = e / NQ, q = e - y * NQ;
-            resid_quad(q, y, kf, c);
+            for (int l = 0; l < 4; ++l) rw[y][4 * q + l] = res[l];
+        }
+        if (D3 && more) {
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                dd[l] = cc[l];
+                cc[l] = uu[l];
+            }
+            load_rest(kf + 1);
         }
     };
     // full-weighting y-x sum of the window at this thread's coarse node (window node x at rw
     // column x + 1)
     auto plane_sum = [&]() {
         __syncthreads();
-        for (int y = ty; y < WY; y += RR_THREADS / RR_X) {
+        for (int r = ty; r < WY; r += RR_THREADS / RR_X) {
             const int w = 2 * tx + 2;
-            rs[y][tx] = fma(T(2), rw[y][w], rw[y][w - 1] + rw[y][w + 1]);
+            rs[r][tx] = fma(T(2), rw[r][w], rw[r][w - 1] + rw[r][w + 1]);
         }
         __syncthreads();
         const int w = 2 * ty + 1;
@@ -398,13 +409,15 @@ __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& 
         const int per = (nkc + int(gd.z) - 1) / int(gd.z);
         const int K0 = 1 + int(b.z) * per, K1 = min(nkc, K0 + per - 1);
         if (K0 <= K1) {
-            resid_plane(2 * K0 - 1);
+            load_first(2 * K0 - 1);
+            load_rest(2 * K0 - 1);
+            resid_plane(2 * K0 - 1, true);
             T lo = plane_sum();
             for (int K = K0; K <= K1; ++K) {
                 // plane_sum's barriers order these writes of rw after every read of the previous plane
-                resid_plane(2 * K);
+                resid_plane(2 * K, true);
                 const T mid = plane_sum();
-                resid_plane(2 * K + 1);
+                resid_plane(2 * K + 1, K < K1);
                 const T hi = plane_sum();
                 if (node) {
                     fc[at(gc, I, J, K)] = fma(T(2), mid, lo + hi) * T(1.0 / 64.0);
@@ -414,7 +427,9 @@ __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& 
             }
         }
     } else {
-        resid_plane(0);
+        load_first(0);
+        load_rest(0);
+        resid_plane(0, false);
         const T sum = plane_sum();
         if (node) {
             fc[at(gc, I, J, 0)] = sum * T(1.0 / 16.0);
