@@ -16,9 +16,11 @@
 // the same solver applies on any level.  The sine transforms are fast
 // transforms (kernels_dst.cu) on large planes whose nx - 1 and ny - 1 are powers
 // of two, dense products with folded sine matrices, both transforms of a plane
-// in one launch, on planes of at most 128 cells a side (plane_body), and
-// batched GEMMs with the (symmetric) sine matrices otherwise; the inverse is
-// the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
+// in one launch, on planes of at most 128 cells a side (plane_body), exact
+// digit products on the tensor cores in the FP64 direct correction of 128 and
+// 256 cells (kernels_split.cu), and in FP32 batched GEMMs with the (symmetric)
+// sine matrices otherwise (in FP64 such levels are refused, sep_level_ok); the
+// inverse is the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
 // relative, which the double-float outer loop of mixed mode then corrects.
 #include <cooperative_groups.h>
 
@@ -102,19 +104,15 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs<T>& g, int bx, int by, 
     }
 }
 
-// The tile of a product (GemmArgs::tile).  FP64 products are bound by the
-// FP64 pipe, one FMA per output and k whatever the tile, and their rows are
-// short: 16 x 16 tiles waste little at ragged ends and spread a 47 x 39
-// plane over nine SMs instead of one (6.6 against 59 us per product, and 9.4
-// against 59 us for the 23 planes of a 49 x 41 x 25 level).
-// FP32 products take the largest tile that still gives two blocks per SM.
+// The tile of a product (GemmArgs::tile): the largest that still gives two
+// blocks per SM (one plane's product in 64 x 64 tiles ran on a few SMs alone).
+// FP32 only: the FP64 levels without a fast transform are planes of at most 65
+// cells, which plane_body serves.
 constexpr int TK64 = 16, TK32 = 32, TK16 = 64;
 constexpr int GEMM_SMEM = 2 * TK32 * 36;   // the 32 x 32 tiles' two operands, the largest
 static_assert(GEMM_SMEM >= 2 * TK16 * 17 && GEMM_SMEM >= 2 * TK64 * 68, "shared memory of the other tiles");
 
-template <typename T>
 int gemm_tile_size(int M, int N, int batch) {
-    if (sizeof(T) == 8) return 16;
     for (int tb : {64, 32})
         if ((long long)((M + tb - 1) / tb) * ((N + tb - 1) / tb) * batch >= 2 * 152) return tb;
     return 16;
@@ -695,7 +693,7 @@ __global__ void __launch_bounds__(1024) g_sep_kernel(const GSepItem<T>* items, i
     const GSepItem<T>* it = glocate(items, n, gate, fmg_step, lb);
     if (!it) return;
     const int bx = lb % it->gx, by = (lb / it->gx) % it->gy, bz = lb / (it->gx * it->gy);
-    if constexpr (KIND == SEP_GEMM) gemm_body(it->st.gemm, bx, by, bz);
+    if constexpr (KIND == SEP_GEMM && sizeof(T) == 4) gemm_body(it->st.gemm, bx, by, bz);
     else if constexpr (KIND == SEP_SCAN) scan_body(it->st.mode, bx, by);
     else if constexpr (KIND == SEP_THOMAS) thomas_body(it->st.mode, bx, by);
     else if constexpr (KIND == SEP_PLANE) plane_body(it->st.plane, bx, by);
@@ -754,7 +752,7 @@ SepStage<T> gemm_stage(const GemmArgs<T>& g, int batch) {
     s.kind = SEP_GEMM;
     s.gemm = g;
     s.threads = 256;
-    const int tb = s.gemm.tile = gemm_tile_size<T>(g.M, g.N, batch);
+    const int tb = s.gemm.tile = gemm_tile_size(g.M, g.N, batch);
     s.grid = dim3((g.N + tb - 1) / tb, (g.M + tb - 1) / tb, batch);
     return s;
 }
@@ -860,6 +858,7 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
         dst(a);
         return;
     }
+    if (sizeof(T) == 8) throw Error(MHS_ERR_BAD_STATE, "separable solve: no FP64 transforms for this level");
     const T* Sx = static_cast<const T*>(tab.sx);
     const T* Sy = static_cast<const T*>(tab.sy);
     stages.push_back(gemm_stage<T>(GemmArgs<T>{nyi, nxi, nxi, f + off, g.px, sA, Sx, nxi, 0, t1, nxi, pl, T(1), 0}, nzi));
@@ -877,7 +876,9 @@ void launch_stage(const SepStage<T>& s, cudaStream_t st) {
     case SEP_SPLIT:
         if constexpr (sizeof(T) == 8) launch_dst_split(s.dst, s.digits, st);
         return;
-    case SEP_GEMM: gemm_kernel<T><<<s.grid, s.threads, 0, st>>>(s.gemm); break;
+    case SEP_GEMM:
+        if constexpr (sizeof(T) == 4) gemm_kernel<T><<<s.grid, s.threads, 0, st>>>(s.gemm);
+        break;
     case SEP_SCAN: {
         static bool configured = false;   // per template instance
         if (!configured) {
@@ -1196,7 +1197,10 @@ void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st)
     if (t.n == 0) return;
     switch (t.kind) {
     case SEP_DST: glaunch_dst<T>(t, fmg_step, gate, st); return;
-    case SEP_GEMM: g_sep_kernel<T, SEP_GEMM><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate); break;
+    case SEP_GEMM:
+        if constexpr (sizeof(T) == 4)
+            g_sep_kernel<T, SEP_GEMM><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate);
+        break;
     case SEP_SCAN: {
         static bool configured = false;
         if (!configured) {
