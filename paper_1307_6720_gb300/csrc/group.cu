@@ -98,7 +98,7 @@ void upload_exact(GPart* G, GDim& D, std::vector<std::vector<GSepItem<T>>>& by_s
     std::vector<GSepTable<T>>& out = exact_tables<T>(D);
     out.clear();
     for (auto& items : by_stage) {
-        for (int kind = SEP_DST; kind <= SEP_PLANE; ++kind) {
+        for (int kind = SEP_DST; kind <= SEP_SPLIT_PLANE; ++kind) {
             std::vector<GSepItem<T>> v;
             for (const GSepItem<T>& it : items)
                 if (it.st.kind == kind) v.push_back(it);

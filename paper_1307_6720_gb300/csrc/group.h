@@ -93,6 +93,7 @@ struct GSepTable {
 };
 template <typename T>
 void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st);   // kernels_sep.cu
+void glaunch_split_plane(const GSepTable<double>& t, int fmg_step, int gate, cudaStream_t st);   // kernels_split.cu
 template <typename T>
 void glaunch_dst(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st);   // kernels_dst.cu
 

@@ -18,7 +18,8 @@
 // of two, dense products with folded sine matrices, both transforms of a plane
 // in one launch, on planes of at most 128 cells a side (plane_body), exact
 // digit products on the tensor cores in the FP64 direct correction of 128 and
-// 256 cells (kernels_split.cu), and in FP32 batched GEMMs with the (symmetric)
+// 256 cells and on coarse FP64 levels of 64 x 64 cells, where the FP64 pipe
+// bounds the fast transforms (kernels_split.cu), and in FP32 batched GEMMs with the (symmetric)
 // sine matrices otherwise (in FP64 such levels are refused, sep_level_ok); the
 // inverse is the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
 // relative, which the double-float outer loop of mixed mode then corrects.
@@ -786,7 +787,7 @@ SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes) {
 // sum_j Sy[n][j] t1[k][j][m], mode solves, and back the same way.
 template <typename T>
 void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTables& tab, const T* f, T* t1, T* t2,
-                T* out, bool accumulate, std::vector<SepStage<T>>& stages, bool split = false) {
+                T* out, bool accumulate, std::vector<SepStage<T>>& stages, bool split = false, bool lines = false) {
     const int nxi = g.nx - 2, nyi = g.ny - 2, nzi = dim == 3 ? g.nz - 2 : 1;
     if (nxi < 1 || nyi < 1 || nzi < 1) return;
     const long long pl = (long long)nxi * nyi;
@@ -795,7 +796,13 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
     const T* mux = static_cast<const T*>(tab.mux);
     const T* muy = static_cast<const T*>(tab.muy);
     const T scale = T((2.0 / (g.nx - 1)) * (2.0 / (g.ny - 1)));
-    if (tab.fx) {   // x lines of f -> t1[k][m][n], mode solves, y lines back and x -> out, scaled
+    const bool planes = tab.fx || (tab.gp && !lines);
+    auto plane = [&](const PlaneArgs<T>& p) {
+        if constexpr (sizeof(T) == 8)
+            if (tab.gp) return split_plane_stage(p, tab.gp, nzi);
+        return plane_stage<T>(p, nzi);
+    };
+    if (planes) {   // x lines of f -> t1[k][m][n], mode solves, y lines back and x -> out, scaled
         PlaneArgs<T> p;
         p.A = nyi;
         p.M1 = nxi;
@@ -807,7 +814,7 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
         p.out_line = nyi;
         p.s1 = static_cast<const T*>(tab.fx);
         p.s2 = static_cast<const T*>(tab.fy);
-        stages.push_back(plane_stage<T>(p, nzi));
+        stages.push_back(plane(p));
         stages.push_back(mode_stage<T>(g, dim, coef, tab, nyi, nxi, muy, mux, true, t1));
         p.A = nxi;
         p.M1 = nyi;
@@ -821,16 +828,16 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
         p.s2 = static_cast<const T*>(tab.fx);
         p.scale = scale;
         p.accumulate = accumulate ? 1 : 0;
-        stages.push_back(plane_stage<T>(p, nzi));
+        stages.push_back(plane(p));
         return;
     }
-    if (tab.twx) {
+    if (tab.twx || tab.gp) {
         auto dst = [&](const DstArgs<T>& a) {
             SepStage<T> s;
             s.dst = a;
-            if (split && tab.gx && tab.gy) {
+            if (tab.gp || (split && tab.gx && tab.gy)) {
                 s.kind = SEP_SPLIT;
-                s.digits = a.tw == tab.twx && a.L == g.nx - 1 ? tab.gx : tab.gy;
+                s.digits = tab.gp ? tab.gp : a.L == g.nx - 1 ? tab.gx : tab.gy;
             } else {
                 s.kind = SEP_DST;
                 dst_shape<T>(s.dst, s.grid, s.threads, s.smem);
@@ -873,6 +880,9 @@ template <typename T>
 void launch_stage(const SepStage<T>& s, cudaStream_t st) {
     switch (s.kind) {
     case SEP_DST: launch_dst_stage<T>(s, st); return;
+    case SEP_SPLIT_PLANE:
+        if constexpr (sizeof(T) == 8) launch_split_plane(s, st);
+        break;
     case SEP_SPLIT:
         if constexpr (sizeof(T) == 8) launch_dst_split(s.dst, s.digits, st);
         return;
@@ -919,9 +929,9 @@ namespace {
 
 template <typename T>
 void level_solve(mhs_ctx* c, const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTables& tab, const T* f,
-                 T* t1, T* t2, T* out, bool accumulate, bool split = false) {
+                 T* t1, T* t2, T* out, bool accumulate, bool split = false, bool lines = false) {
     std::vector<SepStage<T>> stages;
-    plan_level<T>(g, dim, coef, tab, f, t1, t2, out, accumulate, stages, split);
+    plan_level<T>(g, dim, coef, tab, f, t1, t2, out, accumulate, stages, split, lines);
     for (const SepStage<T>& s : stages) launch_stage<T>(s, c->stream);
 }
 
@@ -1022,7 +1032,7 @@ template <typename T>
 void compute_pivots(mhs_ctx* c, Hierarchy& H, int l, SepTables& t) {
     const Geom& g = H.g[l];
     if (H.dim != 3 || !t.inv) return;
-    const bool ytrans = t.twx != nullptr || t.fx != nullptr;
+    const bool ytrans = t.twx != nullptr || t.fx != nullptr || t.gp != nullptr;
     const int nxi = g.nx - 2, nyi = g.ny - 2;
     const int nfast = ytrans ? nyi : nxi, nslow = ytrans ? nxi : nyi;
     const int threads = nfast <= 64 ? 64 : 128;
@@ -1114,6 +1124,11 @@ void sep_tables(mhs_ctx* c, Hierarchy& H, int l) {
     if (dense_planes<T>(g, H.dim)) {
         t.fx = upload(folded(g.nx));
         t.fy = upload(folded(g.ny));
+    } else if (sizeof(T) == 8 && H.dim == 3 && l > 0 && split_planes(g)) {   // (direct corrections, l = 0, keep the fast form)
+        size_t bytes = 0;
+        t.gp = make_split_table(g.nx - 1, &bytes);
+        c->allocations.push_back(t.gp);
+        c->dev_bytes += round_up(bytes, 256);
     } else if (pow2(g.nx - 1) && pow2(g.ny - 1)) {
         size_t tb = 0;
         t.twx = make_twiddles<T>(g.nx - 1, &tb);
@@ -1182,7 +1197,8 @@ void sep_exact(mhs_ctx* c, Hierarchy& H, int l) {
         for (const SepStage<T>& q : st) launch_stage<T>(q, c->stream);
         return;
     }
-    level_solve<T>(c, g, H.dim, A.coef, tab, A.f, A.r, A.t, A.u, false);
+    level_solve<T>(c, g, H.dim, A.coef, tab, A.f, A.r, A.t, A.u, false, false,
+                   (c->opts.flags & MHS_FLAG_STAGED_TRANSFORMS) != 0);
 }
 
 template <typename T>
@@ -1222,6 +1238,9 @@ void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st)
         g_sep_kernel<T, SEP_PLANE><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);
         break;
     }
+    case SEP_SPLIT_PLANE:
+        if constexpr (sizeof(T) == 8) glaunch_split_plane(t, fmg_step, gate, st);
+        break;
     default: g_sep_kernel<T, SEP_DIVIDE><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate); break;
     }
     count_launches(1);

@@ -46,6 +46,7 @@
 
 #include "device_util.cuh"
 #include "dst_body.cuh"
+#include "group.h"
 #include "mhs_internal.h"
 #include "solver.h"
 
@@ -95,19 +96,96 @@ __device__ __forceinline__ double widened(long long v, int k) {
     return __longlong_as_double(static_cast<long long>(bits | (v < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
+// Digits of the two folded elements f of row r at k, k + 1, relative to 2^(e - 1077)
+__device__ __forceinline__ void put_digits(unsigned* A, int r, int k, double f0, double f1, int e) {
+    const unsigned long long q0 = static_cast<unsigned long long>(fixed(f0, e) + BIAS);
+    const unsigned long long q1 = static_cast<unsigned long long>(fixed(f1, e) + BIAS);
+    const __half2 off = __halves2half2(__ushort_as_half(0xe480), __ushort_as_half(0xe480));   // -1152
+    const int ks = k >> 4, kk = k & 15;
+    unsigned* word = A + ks * STEP + (((r & 7) * 4 + ((kk & 7) >> 1)) << 2) + (r >> 3) + 2 * (kk >> 3);
+#pragma unroll
+    for (int s = 0; s < DIG; ++s) {
+        const int b = DIG - 1 - s;   // byte of digit s
+        const unsigned u0 = b < 4 ? unsigned(q0) : unsigned(q0 >> 32);
+        const unsigned u1 = b < 4 ? unsigned(q1) : unsigned(q1 >> 32);
+        // 1024 + byte, twice (the first digit may be 128: nine bits)
+        const unsigned h = s == 0 ? __byte_perm(u0, u1, 0x7632) | 0x64006400u
+                                  : __byte_perm(__byte_perm(u0, u1, (b & 3) | ((4 + (b & 3)) << 4)), 0x64646464u, 0x4140);
+        const __half2 d = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
+        word[s * 128] = *reinterpret_cast<const unsigned*>(&d);
+    }
+}
+
+// largest exponent of a line held by L lanes
+template <int L>
+__device__ __forceinline__ int line_max(int e) {
+    if constexpr (L == 32) return int(__reduce_max_sync(0xffffffffu, unsigned(e)));
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    return e;
+}
+
+// The digit products of 16 rows with TILES column tiles; bt: the first tile's
+// digits [tile][k step][digit][lane], at this lane, loaded one tile ahead
+template <int KS>
+__device__ __forceinline__ void products(const unsigned* A, const uint2* __restrict__ bt, int lane,
+                                         float (&acc)[TILES][ORDERS][4]) {
+#pragma unroll
+    for (int n = 0; n < TILES; ++n)
+#pragma unroll
+        for (int d = 0; d < ORDERS; ++d)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[n][d][c] = 0.f;
+    auto load_b = [&](uint2(&v)[DIG], int ks, int n) {
+#pragma unroll
+        for (int s = 0; s < DIG; ++s) v[s] = __ldg(bt + ((n * KS + ks) * DIG + s) * 32);
+    };
+    uint2 bn[DIG];
+    load_b(bn, 0, 0);
+#pragma unroll 1
+    for (int ks = 0; ks < KS; ++ks) {
+        uint4 av[DIG];
+#pragma unroll
+        for (int s = 0; s < DIG; ++s) av[s] = *reinterpret_cast<const uint4*>(A + ks * STEP + s * 128 + 4 * lane);
+#pragma unroll
+        for (int n = 0; n < TILES; ++n) {
+            uint2 bv[DIG];
+#pragma unroll
+            for (int s = 0; s < DIG; ++s) bv[s] = bn[s];
+            if (n + 1 < TILES) load_b(bn, ks, n + 1);
+            else if (ks + 1 < KS) load_b(bn, ks + 1, 0);
+#pragma unroll
+            for (int i = 0; i < DIG; ++i)
+#pragma unroll
+                for (int j = 0; j < DIG && i + j < ORDERS; ++j) mma16816(acc[n][i + j], av[i], bv[j]);
+        }
+    }
+}
+
+// result c of a tile's accumulators, of a row with exponent e
+__device__ __forceinline__ double joined(const float (&acc)[ORDERS][4], int c, int e) {
+    auto in = [&](int d) { return static_cast<long long>(__float2int_rn(acc[d][c])); };
+    const long long top = (in(0) << 24) + (in(1) << 16) + (in(2) << 8) + in(3);
+    const long long low = (in(4) << 16) + (in(5) << 8) + in(6) + (in(7) >> 8);
+    // 256^7 2^-55 times 2^(e - 1077) of the elements: 2^(e - 1076)
+    const double v = widened((top << 16) + ((low + 128) >> 8), e - 1076);
+    return e == 2047 ? __longlong_as_double(0x7ff8000000000000LL) : v;
+}
+
 // lines of N - 1 elements, N = 32 KS; tab: the matrices' digits in fragment
 // order [parity][column tile][k step][digit][lane]
 template <int KS>
 __global__ void __launch_bounds__(32 * SW, 3) dst_split_kernel(DstArgs<double> a, const uint2* __restrict__ tab) {
     constexpr int Ko = 16 * KS, N = 2 * Ko;
-    constexpr int NG = Ko / 16 / TILES;   // groups of tiles of a warp
-    constexpr int EP = Ko / 32;   // folded elements of a lane
+    constexpr int NG = Ko / 16 / TILES;              // groups of tiles of a warp
+    constexpr int EP = Ko >= 64 ? Ko / 32 : 2;       // folded elements of a lane
+    constexpr int LL = Ko / EP, RW = 32 / LL;        // lanes of a line, lines of a warp
     extern __shared__ __align__(16) unsigned char split_smem[];
     __shared__ int s_e[SW / 2][16];
     const int lane = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1, w = threadIdx.x >> 6;
     unsigned* A = reinterpret_cast<unsigned*>(split_smem) + w * (KS * STEP);
     const long long total = (long long)a.lines * a.planes, first = ((long long)blockIdx.x * (SW / 2) + w) * 16;
-    const int g = lane >> 2, t4 = lane & 3;
+    const int g = lane >> 2, t4 = lane & 3, li = lane % LL;
     // the two lines whose results this thread holds
     long long base[2];
     bool live[2];
@@ -131,16 +209,17 @@ __global__ void __launch_bounds__(32 * SW, 3) dst_split_kernel(DstArgs<double> a
             const double* x = a.in + pl * a.in_plane + (on ? gl - pl * a.lines : 0) * a.in_line;
 #pragma unroll
             for (int u = 0; u < EP; ++u) {
-                const int i = lane * EP + u, j = N - 2 - i;
+                const int i = li * EP + u, j = N - 2 - i;
                 lo[u] = on ? x[i] : 0.0;
                 // (the middle element is its own mirror: it counts once, in the sums)
                 hi[u] = !on ? 0.0 : j != i ? x[j] : par ? lo[u] : 0.0;
             }
         };
         double lo[EP], hi[EP];
-        load_line(8 * half, lo, hi);
+        const int r0 = 8 * half + lane / LL, r1 = 8 * half + 8;
+        load_line(r0, lo, hi);
 #pragma unroll 1
-        for (int r = 8 * half; r < 8 * half + 8; ++r) {
+        for (int r = r0; r < r1; r += RW) {
             double f[EP];
             int e = 1;
 #pragma unroll
@@ -148,85 +227,117 @@ __global__ void __launch_bounds__(32 * SW, 3) dst_split_kernel(DstArgs<double> a
                 f[u] = par ? lo[u] - hi[u] : lo[u] + hi[u];
                 e = max(e, expo(f[u]));
             }
-            if (r < 8 * half + 7) load_line(r + 1, lo, hi);
-            e = int(__reduce_max_sync(0xffffffffu, unsigned(e)));
-            unsigned long long q[EP];
+            if (r + RW < r1) load_line(r + RW, lo, hi);
+            e = line_max<LL>(e);
+            if (li == 0) s_e[w][r] = e;
 #pragma unroll
-            for (int u = 0; u < EP; ++u) q[u] = static_cast<unsigned long long>(fixed(f[u], e) + BIAS);
-            if (lane == 0) s_e[w][r] = e;
-            const __half2 off = __halves2half2(__ushort_as_half(0xe480), __ushort_as_half(0xe480));   // -1152
-#pragma unroll
-            for (int u = 0; u < EP; u += 2) {
-                const int k = lane * EP + u, ks = k >> 4, kk = k & 15;
-                const int word = ks * STEP + (((r & 7) * 4 + ((kk & 7) >> 1)) << 2) + (r >> 3) + 2 * (kk >> 3);
-#pragma unroll
-                for (int s = 0; s < DIG; ++s) {
-                    const int b = DIG - 1 - s;   // byte of digit s
-                    const unsigned u0 = b < 4 ? unsigned(q[u]) : unsigned(q[u] >> 32);
-                    const unsigned u1 = b < 4 ? unsigned(q[u + 1]) : unsigned(q[u + 1] >> 32);
-                    // 1024 + byte, twice (the first digit may be 128: nine bits)
-                    const unsigned h = s == 0 ? __byte_perm(u0, u1, 0x7632) | 0x64006400u
-                                              : __byte_perm(__byte_perm(u0, u1, (b & 3) | ((4 + (b & 3)) << 4)), 0x64646464u, 0x4140);
-                    const __half2 d = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
-                    A[word + s * 128] = *reinterpret_cast<const unsigned*>(&d);
-                }
-            }
+            for (int u = 0; u < EP; u += 2) put_digits(A, r, li * EP + u, f[u], f[u + 1], e);
         }
         __syncthreads();
         for (int ng = ng0; ng < ng1; ++ng) {
             float acc[TILES][ORDERS][4];
-#pragma unroll
-            for (int n = 0; n < TILES; ++n)
-#pragma unroll
-                for (int d = 0; d < ORDERS; ++d)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[n][d][c] = 0.f;
-            // column tile n of k step ks, its digits loaded one tile ahead
-            const uint2* bt = tab + (size_t(par) * (Ko / 8) + ng * TILES) * KS * DIG * 32 + lane;
-            auto load_b = [&](uint2(&v)[DIG], int ks, int n) {
-#pragma unroll
-                for (int s = 0; s < DIG; ++s) v[s] = __ldg(bt + ((n * KS + ks) * DIG + s) * 32);
-            };
-            uint2 bn[DIG];
-            load_b(bn, 0, 0);
-#pragma unroll 1
-            for (int ks = 0; ks < KS; ++ks) {
-                uint4 av[DIG];
-#pragma unroll
-                for (int s = 0; s < DIG; ++s)
-                    av[s] = *reinterpret_cast<const uint4*>(A + ks * STEP + s * 128 + 4 * lane);
-#pragma unroll
-                for (int n = 0; n < TILES; ++n) {
-                    uint2 bv[DIG];
-#pragma unroll
-                    for (int s = 0; s < DIG; ++s) bv[s] = bn[s];
-                    if (n + 1 < TILES) load_b(bn, ks, n + 1);
-                    else if (ks + 1 < KS) load_b(bn, ks + 1, 0);
-#pragma unroll
-                    for (int i = 0; i < DIG; ++i)
-#pragma unroll
-                        for (int j = 0; j < DIG && i + j < ORDERS; ++j) mma16816(acc[n][i + j], av[i], bv[j]);
-                }
-            }
+            products<KS>(A, tab + (size_t(par) * (Ko / 8) + ng * TILES) * KS * DIG * 32 + lane, lane, acc);
 #pragma unroll
             for (int n = 0; n < TILES; ++n)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int h = c >> 1, col = (ng * TILES + n) * 8 + 2 * t4 + (c & 1), m = 2 * col + par;
                     if (!live[h] || m > N - 2) continue;
-                    auto in = [&](int d) { return static_cast<long long>(__float2int_rn(acc[n][d][c])); };
-                    const long long top = (in(0) << 24) + (in(1) << 16) + (in(2) << 8) + in(3);
-                    const long long low = (in(4) << 16) + (in(5) << 8) + in(6) + (in(7) >> 8);
-                    const int e = s_e[w][g + 8 * h];
-                    // 256^7 2^-55 times 2^(e - 1077) of the elements: 2^(e - 1076)
-                    double v = widened((top << 16) + ((low + 128) >> 8), e - 1076);
-                    if (e == 2047) v = __longlong_as_double(0x7ff8000000000000LL);
+                    const double v = joined(acc[n], c, s_e[w][g + 8 * h]);
                     double* o = a.out + base[h] + (long long)m * a.out_elem;
                     *o = a.scale == 1.0 && !a.accumulate ? v : dst_result(a.scale, v, a.accumulate != 0, a.accumulate ? *o : 0.0);
                 }
         }
         __syncthreads();
     }
+}
+
+// Both transforms of a plane of 63 x 63 values (64 cells; the coarse-grid solves
+// of 129^3 and 257^3 FP64 cycles): along the lines, then across.  Block (par, plane) forms the lines' odd (par = 0) or even
+// results and takes them across by itself, so nothing passes between blocks.
+// Eight warps: two to 16 lines of a parity, each for half of their results
+// (one group of tiles); the second transforms read the first ones' results
+// from shared memory.  63 planes in 126 blocks: 13.5 us, of which the chain of
+// loads, digits, products and sums of one block is all; the fast transforms on
+// clusters of two blocks took 30 us, 67 % of it FP64 pipe.  A 65^3 level's solve
+// 75 -> 42 us, its residual 7e-15 -> 1.6e-15.
+constexpr int SP_CELLS = 64, SP_KS = 2, SP_T = 256;
+
+__device__ __forceinline__ void split_plane_body(const PlaneArgs<double>& a, const uint2* __restrict__ tab, int par,
+                                                 int plane) {
+    constexpr int KS = SP_KS, Ko = 16 * KS, N = SP_CELLS, LD = N + 1;
+    __shared__ __align__(16) unsigned s_A[4][KS * STEP];
+    __shared__ double s_x[Ko][LD];   // results of the first transforms [mode][line]
+    __shared__ int s_e[4][16];
+    const int lane = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1, w = threadIdx.x >> 6;
+    const int g = lane >> 2, t4 = lane & 3, li = lane & 15, sub = lane >> 4;
+    unsigned* A = s_A[w];
+    // the digits of rows r, r + 2, .. of 8 half .. 8 half + 7, two rows at a time, of lines x(r)
+    auto digits = [&](auto&& line, int p) {
+        double lo[4][2], hi[4][2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const double* x = line(8 * half + 2 * q + sub);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = 2 * li + u, j = N - 2 - i;
+                lo[q][u] = x ? x[i] : 0.0;
+                hi[q][u] = !x ? 0.0 : j != i ? x[j] : p ? lo[q][u] : 0.0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = 8 * half + 2 * q + sub;
+            const double f0 = p ? lo[q][0] - hi[q][0] : lo[q][0] + hi[q][0];
+            const double f1 = p ? lo[q][1] - hi[q][1] : lo[q][1] + hi[q][1];
+            const int e = line_max<16>(max(max(1, expo(f0)), expo(f1)));
+            if (li == 0) s_e[w][r] = e;
+            put_digits(A, r, 2 * li, f0, f1, e);
+        }
+    };
+    auto form = [&](int p, float(&acc)[TILES][ORDERS][4]) {
+        products<KS>(A, tab + (size_t(p) * (Ko / 8) + half * TILES) * KS * DIG * 32 + lane, lane, acc);
+    };
+    float acc[TILES][ORDERS][4];
+    const double* in = a.in + plane * a.in_plane;
+    digits([&](int r) { return 16 * w + r < a.A ? in + (16 * w + r) * a.in_line : nullptr; }, par);
+    __syncthreads();
+    form(par, acc);
+#pragma unroll
+    for (int n = 0; n < TILES; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int row = g + 8 * (c >> 1), col = (half * TILES + n) * 8 + 2 * t4 + (c & 1);
+            s_x[col][16 * w + row] = joined(acc[n], c, s_e[w][row]);
+        }
+    __syncthreads();
+    // 32 lines of both parities: warps 0 .. 3 the first 16, 4 .. 7 the others
+    const int p2 = w & 1, l0 = 16 * (w >> 1);
+    digits([&](int r) { return &s_x[l0 + r][0]; }, p2);
+    __syncthreads();
+    form(p2, acc);
+#pragma unroll
+    for (int n = 0; n < TILES; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int row = g + 8 * (c >> 1), m = 2 * (l0 + row) + par;
+            const int col = (half * TILES + n) * 8 + 2 * t4 + (c & 1), q = 2 * col + p2;
+            if (m > N - 2 || q > N - 2) continue;
+            const double v = joined(acc[n], c, s_e[w][row]);
+            double* o = a.out + plane * a.out_plane + m * a.out_line + q;
+            *o = a.scale == 1.0 && !a.accumulate ? v : dst_result(a.scale, v, a.accumulate != 0, a.accumulate ? *o : 0.0);
+        }
+}
+
+__global__ void __launch_bounds__(SP_T) split_plane_kernel(PlaneArgs<double> a, const uint2* __restrict__ tab) {
+    split_plane_body(a, tab, int(blockIdx.x), int(blockIdx.y));
+}
+
+__global__ void __launch_bounds__(SP_T) g_split_plane_kernel(const GSepItem<double>* items, int n, int fmg_step, int gate) {
+    int lb;
+    const GSepItem<double>* it = glocate(items, n, gate, fmg_step, lb);
+    if (!it) return;
+    split_plane_body(it->st.plane, static_cast<const uint2*>(it->st.digits), lb % it->gx, lb / it->gx);
 }
 
 template <int KS>
@@ -249,8 +360,12 @@ void launch_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
 
 }  // namespace
 
-// 512 cells: the digits of a parity (58 KB for 16 lines) would leave one block per SM; 64: a fast transform of six
-// stages, a sixth of a pass over 128 cells in FP64 work, was left as it is
+// coarse FP64 levels: planes of 64 x 64 cells (one parity's digits of a whole plane in one block); the dense plane
+// transforms serve smaller ones
+bool split_planes(const Geom& g) { return g.nx - 1 == SP_CELLS && g.ny - 1 == SP_CELLS; }
+
+// direct corrections.  512 cells: the digits of a parity (58 KB for 16 lines) would leave one block per SM; 64: direct
+// corrections keep the fast transforms (their error, 2.3e-15 to 3.5e-15 at 65 x 65 x 33, is the tridiagonal solves')
 bool split_length(int N) { return N == 128 || N == 256; }
 
 // sin(pi q / N) 2^55 as an integer
@@ -264,7 +379,13 @@ void* make_split_table(int N, size_t* bytes) {
     const int Ko = N / 2, KS = Ko / 16;
     std::vector<uint2> tab(size_t(2) * (Ko / 8) * KS * DIG * 32);
     std::vector<long long> sines(2 * N);
-    for (int q = 0; q < 2 * N; ++q) sines[q] = sine55(q, N);
+    for (int q = 0; q <= N / 2; ++q) {   // one quarter of the period holds them all
+        const long long v = sine55(q, N);
+        sines[q] = sines[N - q] = v;
+        sines[N + q] = -v;
+        sines[(2 * N - q) % (2 * N)] = -v;
+    }
+    sines[0] = sines[N] = 0;
     auto digits = [&](int par, int i, int p) -> unsigned long long {   // of element i of result p, biased
         const int m = 2 * p + 1 + par;                                  // mode
         if (m > N - 1 || (par && i >= Ko - 1)) return BIAS;             // padding: zero
@@ -294,8 +415,27 @@ void* make_split_table(int N, size_t* bytes) {
 }
 
 void launch_dst_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
-    if (a.L == 128) launch_split<4>(a, tab, st);
+    if (a.L == SP_CELLS) launch_split<2>(a, tab, st);
+    else if (a.L == 128) launch_split<4>(a, tab, st);
     else launch_split<8>(a, tab, st);
+}
+
+SepStage<double> split_plane_stage(const PlaneArgs<double>& p, const void* digits, int planes) {
+    SepStage<double> s;
+    s.kind = SEP_SPLIT_PLANE;
+    s.plane = p;
+    s.digits = digits;
+    s.threads = SP_T;
+    s.grid = dim3(2, planes);
+    return s;
+}
+
+void launch_split_plane(const SepStage<double>& s, cudaStream_t st) {
+    split_plane_kernel<<<s.grid, s.threads, 0, st>>>(s.plane, static_cast<const uint2*>(s.digits));
+}
+
+void glaunch_split_plane(const GSepTable<double>& t, int fmg_step, int gate, cudaStream_t st) {
+    g_split_plane_kernel<<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate);
 }
 
 }  // namespace mhs

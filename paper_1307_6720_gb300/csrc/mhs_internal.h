@@ -112,6 +112,7 @@ struct SepTables {
     void *twx = nullptr, *twy = nullptr;
     void *sx = nullptr, *sy = nullptr;
     void *gx = nullptr, *gy = nullptr;   // digits of the folded matrices of the split transforms (kernels_split.cu)
+    void* gp = nullptr;                  // the same of planes of 64 x 64 cells
     void *fx = nullptr, *fy = nullptr;   // folded sine matrices of the plane transforms (kernels_sep.cu)
     void *inv = nullptr, *sup = nullptr;
     bool ready = false;
@@ -406,7 +407,7 @@ struct PlaneArgs {
     T scale = T(1);
     int accumulate = 0;
 };
-enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4, SEP_PLANE = 5, SEP_SPLIT = 6 };
+enum SepKind { SEP_DST = 0, SEP_GEMM = 1, SEP_SCAN = 2, SEP_THOMAS = 3, SEP_DIVIDE = 4, SEP_PLANE = 5, SEP_SPLIT_PLANE = 6, SEP_SPLIT = 7 };
 // one kernel launch of a separable solve with its launch shape
 template <typename T>
 struct SepStage {
@@ -418,8 +419,12 @@ struct SepStage {
     GemmArgs<T> gemm;
     ModeArgs<T> mode;
     PlaneArgs<T> plane;
-    const void* digits = nullptr;   // SEP_SPLIT: dst with these
+    const void* digits = nullptr;   // of SEP_SPLIT (a dst) and SEP_SPLIT_PLANE (a plane)
 };
+// both transforms of FP64 planes of 64 x 64 cells as digit products (kernels_split.cu)
+bool split_planes(const Geom& g);
+SepStage<double> split_plane_stage(const PlaneArgs<double>& p, const void* digits, int planes);
+void launch_split_plane(const SepStage<double>& s, cudaStream_t st);
 // launch shape of a sine-transform stage (sets a.pairs)
 template <typename T>
 void dst_shape(DstArgs<T>& a, dim3& grid, int& threads, size_t& smem);

@@ -682,3 +682,31 @@ def test_plane_transforms_of_folded_matrices(M, shape, prec):
         assert _rel(got[0], want) < (1e-12 if prec == 0 else 2e-5), dim
         assert np.array_equal(got[0], got[1]), dim
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("shape", [(129, 129, 5), (129, 129, 17), (257, 257, 33)])
+def test_coarse_planes_as_digit_products(M, shape):
+    """FP64 coarse levels of 64 x 64 cells (one plane, few, as many as blocks
+    take): the exact solve against the separable direct solution, the staged
+    form bit for bit, and every bit scaled with the right-hand side by powers
+    of two.  Bound: that of test_exact_op_parity."""
+    from oracle import exact
+    nx, ny, nz = shape
+    pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
+    level = {129: 1, 257: 2}[nx]
+    lx, ly, lz = M.mhs_level_shape(h, 3, level)
+    assert (lx, ly) == (65, 65)
+    f = np.random.default_rng(nz).standard_normal((lz, ly, lx))
+    f[:, ly // 2] *= 1e-9   # a line far below the others of its plane
+    got = []
+    for flags, scale in ((0, 1.0), (M.MHS_FLAG_STAGED_TRANSFORMS, 1.0), (0, 2.0**200), (0, 2.0**-200)):
+        M.mhs_set_options(h, flags=flags)
+        M.mhs_level_write(h, 3, level, M.MHS_FIELD_U, 0, np.zeros_like(f))
+        M.mhs_level_write(h, 3, level, M.MHS_FIELD_F, 0, f * scale)
+        M.mhs_level_op(h, 3, level, M.MHS_OP_EXACT, 0)
+        got.append(_read(M, h, 3, level, M.MHS_FIELD_U, 0) / scale)
+    want = exact.separable_solve3d(_level_problem(M, h, pr, 3, level), np.zeros((ly, lx)), f)
+    assert _rel(got[0], want) < 1e-12
+    for other in got[1:]:
+        assert np.array_equal(got[0], other)
+    M.mhs_destroy(h)
