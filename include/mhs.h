@@ -107,8 +107,10 @@ typedef struct {
                             the one-CTA shared-memory sub-cycle [1200] */
     int cut32;           /* same for FP32 levels [4000] */
     int fused_min;       /* FP32 3D levels with at least this many interior nodes use the fused, TMA-staged
-                            red-black sweep (one pass per sweep, HBM-bound); smaller, cache-resident levels use the
-                            two colour passes, which have less latency [12000000] */
+                            red-black sweep (one pass per sweep) for the sweeps that do not run in pairs (two
+                            sweeps per pass: levels of 800,000 nodes and more with nx = 4m + 1); smaller levels use
+                            the two colour passes, which have less latency; results do not depend on it
+                            [12000000] */
     int sep_coarse;      /* coarse-grid solve of the V-cycles: the first level below the finest with at most this
                             many interior nodes, whose sine transforms are fast (nx - 1 and ny - 1 powers of two)
                             or short (nx, ny <= 66), is solved exactly by the separable solver (sine transforms
@@ -153,11 +155,11 @@ typedef struct {
                                    with this flag a mixed solve reaches 1e-12 on 257^3 and 2e-12 on 513 x 513 x 257
                                    nodes.  The lower boundary is a small part of the work (1 / nz of the
                                    unknowns).  Not in groups */
-#define MHS_FLAG_NO_TMA 16      /* FP32 levels sweep with plain global loads instead of TMA-staged planes (same
-                                   results; for comparison) */
+#define MHS_FLAG_NO_TMA 16      /* FP32 levels sweep with plain global loads instead of TMA-staged planes, and one
+                                   sweep at a time (same results; for comparison) */
 #define MHS_FLAG_STAGED_TRANSFORMS 1024 /* separable solves of a level (the exact coarse-grid solves, MHS_OP_EXACT)
                                    launch one kernel per sine-transform pass instead of the per-plane kernels
-                                   on thread-block clusters (same results bit for bit; for comparison) */
+                                   (same results bit for bit; for comparison) */
 #define MHS_FLAG_NO_GRAPH 4     /* launch the solve kernel by kernel with host-side convergence checks instead of
                                    one captured CUDA graph (same kernels, same results; for profilers that cannot
                                    see kernels inside conditional graph nodes) */

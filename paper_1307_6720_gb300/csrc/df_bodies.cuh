@@ -101,10 +101,10 @@ __device__ __forceinline__ void df_residual_body(const Geom& g, const PlaneCoefD
                                                  const float* __restrict__ fh, const float* __restrict__ fl,
                                                  float* __restrict__ r32, double* __restrict__ partial, dim3 b,
                                                  dim3 gd) {
-    const int i = 1 + b.x * DF_BX + threadIdx.x;
-    const int j = 1 + b.y * DF_BY + threadIdx.y;
+    const int i = 1 + b.x * blockDim.x + threadIdx.x;
+    const int j = 1 + b.y * blockDim.y + threadIdx.y;
     float acc = 0.f;
-    if (threadIdx.y < DF_BY && i <= g.nx - 2 && j <= g.ny - 2) {   // (a grouped launch has more rows of threads)
+    if (i <= g.nx - 2 && j <= g.ny - 2) {
         const ptrdiff_t sy = g.px, sz = (ptrdiff_t)g.plane;
         if (D3) {
             const int nzi = g.nz - 2, chunk = (nzi + int(gd.z) - 1) / int(gd.z);

@@ -158,7 +158,7 @@ void build_dim(GPart* G, GDim& D, int dim) {
     std::vector<std::vector<GItem>> pre_pt(L), post_pt(L), pre_ln(L), post_ln(L), res(L), restr(L), resr(L), prol(L),
         fmg_restr(L), fmg_prol(L);
     std::vector<GItem> sub, sub8, subz, subz8, zero_u, lower_rhs, zero_hi, zero_lo, split, copy_u, copy_t, df_copy, lift, bnorm, check1,
-        res_norm0, res_norm, check, fmg_res_norm, fmg_check, zero_e, correct, fmg_zero_e, fmg_correct, to_double;
+        res_norm0, res_norm, res_wide0, res_wide, check, fmg_res_norm, fmg_res_wide, fmg_check, zero_e, correct, fmg_zero_e, fmg_correct, to_double;
     std::vector<SubParams<T>> params;
     std::vector<std::vector<GSepItem<T>>> exact_items;   // per stage of the separable solves
     D.max_nu1 = D.max_nu2 = 0;
@@ -219,7 +219,7 @@ void build_dim(GPart* G, GDim& D, int dim) {
                 rs.ia[3] = (l == 0 && red_residual_rotated(c, H)) ? 1 : 0;    // in a rotated cycle
                 restr[l].push_back(rs);
             } else {   // FP32 levels: the solo V-cycle's fused residual and restriction
-                GItem r = item(q, fat(resid_restrict_grid(gc, d3)), g, ctl);
+                GItem r = item(q, fat(resid_restrict_grid(gc, d3, true)), g, ctl);
                 r.g2 = gc;
                 r.coef = A.coef;
                 r.p[0] = A.u;
@@ -358,8 +358,9 @@ void build_dim(GPart* G, GDim& D, int dim) {
             rn_cyc = rn64(red_residual_cycle(c, H), nb_cyc);
             rn_fmg = rn64(red_residual_fmg(c, H), nb_fmg);
         }
-        res_norm0.push_back(rn);
-        res_norm.push_back(rn_cyc);
+        const bool wide = mixed && d3 && use_df_quads(g0);
+        (wide ? res_wide0 : res_norm0).push_back(rn);
+        (wide ? res_wide : res_norm).push_back(rn_cyc);
         GItem ck = item(q, dim3(1, 1, 1), g0, ctl);
         ck.p[0] = c->ns.partial;
         ck.ia[0] = nb;
@@ -369,7 +370,7 @@ void build_dim(GPart* G, GDim& D, int dim) {
         ck_fmg.ia[0] = nb_fmg;
         check.push_back(ck_cyc);
         if (fmg) {
-            fmg_res_norm.push_back(rn_fmg);
+            (wide ? fmg_res_wide : fmg_res_norm).push_back(rn_fmg);
             fmg_check.push_back(ck_fmg);
         }
         if (dim == 2) {
@@ -493,8 +494,11 @@ void build_dim(GPart* G, GDim& D, int dim) {
     D.check1 = upload(G, check1);
     D.res_norm0 = upload(G, res_norm0);
     D.res_norm = upload(G, res_norm);
+    D.res_wide0 = upload(G, res_wide0);
+    D.res_wide = upload(G, res_wide);
     D.check = upload(G, check);
     D.fmg_res_norm = upload(G, fmg_res_norm);
+    D.fmg_res_wide = upload(G, fmg_res_wide);
     D.fmg_check = upload(G, fmg_check);
     D.zero_e = upload(G, zero_e);
     D.correct = upload(G, correct);
@@ -590,7 +594,7 @@ void gfmg(GPart* G, GDim& D) {
         gvcycle<T>(G, D, s, s, G_ALL);
     }
     if (mixed) glaunch_df_correct(D.fmg_correct, d3, G_ALL, st);
-    if (mixed) glaunch_df_residual(D.fmg_res_norm, d3, G_ALL, st);
+    if (mixed) glaunch_df_residual(D.fmg_res_norm, D.fmg_res_wide, d3, G_ALL, st);
     else glaunch_residual_norm<double>(D.fmg_res_norm, d3, G_ALL, st);
     glaunch_check(D.fmg_check, 2, G_ALL, st);
 }
@@ -608,7 +612,7 @@ void gprologue(GPart* G, GDim& D) {
             glaunch_zero(D.zero_lo, G_ALL, st);
             glaunch_df_split(D.split, 0, st);
         }
-        if (mixed) glaunch_df_residual(D.res_norm0, 0, G_ALL, st);
+        if (mixed) glaunch_df_residual(D.res_norm0, D.res_wide0, 0, G_ALL, st);
         else glaunch_residual_norm<double>(D.res_norm0, 0, G_ALL, st);
         glaunch_bnorm(D.bnorm, st);
     } else {
@@ -622,7 +626,7 @@ void gprologue(GPart* G, GDim& D) {
         }
         glaunch_lift_norm(D.lift, st);
         glaunch_bnorm(D.bnorm, st);
-        if (mixed) glaunch_df_residual(D.res_norm0, 1, G_ALL, st);
+        if (mixed) glaunch_df_residual(D.res_norm0, D.res_wide0, 1, G_ALL, st);
         else glaunch_residual_norm<double>(D.res_norm0, 1, G_ALL, st);
     }
     glaunch_check(D.check1, 1, G_ALL, st);
@@ -639,7 +643,7 @@ void gcycle(GPart* G, GDim& D, SolveCtl* const* ctls, cudaGraphConditionalHandle
     else gvcycle_rotated(G, D, G_ACTIVE);
     if (mixed) {
         glaunch_df_correct(D.correct, d3, G_ACTIVE, st);
-        glaunch_df_residual(D.res_norm, d3, G_ACTIVE, st);
+        glaunch_df_residual(D.res_norm, D.res_wide, d3, G_ACTIVE, st);
     } else {
         glaunch_residual_norm<double>(D.res_norm, d3, G_ACTIVE, st);
     }

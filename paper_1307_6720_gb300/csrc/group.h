@@ -64,7 +64,8 @@ void glaunch_copy_plane(const GTable& t, cudaStream_t st);
 void glaunch_lift_norm(const GTable& t, cudaStream_t st);
 void glaunch_df_split(const GTable& t, int d3, cudaStream_t st);
 void glaunch_df_copy_plane(const GTable& t, cudaStream_t st);
-void glaunch_df_residual(const GTable& t, int d3, int gate, cudaStream_t st);
+// wide: the items of use_df_quads levels
+void glaunch_df_residual(const GTable& t, const GTable& wide, int d3, int gate, cudaStream_t st);
 void glaunch_df_correct(const GTable& t, int d3, int gate, cudaStream_t st);
 void glaunch_df_to_double(const GTable& t, cudaStream_t st);
 void glaunch_bnorm(const GTable& t, cudaStream_t st);
@@ -139,6 +140,7 @@ struct GDim {
     GTable zero_u, lower_rhs, zero_hi, zero_lo, split, copy_u, copy_t, df_copy, lift, bnorm, check1;
     // the first test; cycle end (every instance), and after the full-multigrid cycle (instances using it)
     GTable res_norm0, res_norm, check, fmg_res_norm, fmg_check;
+    GTable res_wide0, res_wide, fmg_res_wide;   // mixed mode: the same on wide levels (use_df_quads)
     // mixed mode
     GTable zero_e, correct, fmg_zero_e, fmg_correct, to_double;
 };

@@ -26,11 +26,12 @@
 // operations in their order: the result equals four colour passes bit for
 // bit.
 //
-// Measured: 513 x 513 x 257 256 us per pair (twice 307 us as fused single
-// sweeps), 257^3 95 us (twice 65), 129^3 19 us.  240 instructions per thread
-// and step of eight nodes; 42 % of the issue slots, 23 % of the stalls at the
-// barrier, 21 % on shared memory; a quarter of the rows and a fifth of the
-// quads (513 nodes: 5 tiles) are halo.
+// Measured: 513 x 513 x 257 243 us per pair (twice 307 us as fused single
+// sweeps), 257^3 85 us (twice 65), 129^3 17 us; its traffic at 513 x 513 x 257
+// takes 119 us.  In scalar FP32 instructions 256, 95 and 19 us (240 per thread
+// and step of eight nodes).  47 % of the issue slots at 129^3; the stalls are
+// shared memory, dependent instructions and the barrier in equal parts; a
+// quarter of the rows and a fifth of the quads (513 nodes: 5 tiles) are halo.
 //
 // TMA rules as in kernels_tma.cu: boxes start at x a multiple of four floats,
 // slots are 128-byte aligned, every mbarrier wait is bounded.

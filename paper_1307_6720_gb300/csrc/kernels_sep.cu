@@ -760,16 +760,19 @@ SepStage<T> gemm_stage(const GemmArgs<T>& g, int batch) {
 
 // The plane transforms as one stage, both directions: along lines of M1
 // elements first.  Blocks of as many results as leave a block per SM (FP64:
-// down to one odd and one even result, FP32: four of each).
+// down to one odd and one even result, FP32: four of each).  Grouped launches
+// have blocks enough of other instances: the fewest per plane (1024 solves of
+// 33^3 42.7 -> 40.0 ms).
 template <typename T>
-SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes) {
+SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes, bool grouped) {
     SepStage<T> s;
     s.kind = SEP_PLANE;
     s.plane = p;
     s.threads = PLANE_T;
     const int Ko1 = (p.M1 + 1) / 2, least = sizeof(T) == 4 ? 4 : 1;
     int sp = 16;
-    while (sp > least && (long long)((Ko1 + sp - 1) / sp) * planes < 152) sp /= 2;
+    if (grouped) while (sp / 2 >= Ko1 && sp > least) sp /= 2;
+    while (!grouped && sp > least && (long long)((Ko1 + sp - 1) / sp) * planes < 152) sp /= 2;
     while (sp > least && PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T) > PLANE_SMEM) sp /= 2;
     s.plane.sp = sp;
     s.smem = PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T);
@@ -787,7 +790,8 @@ SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes) {
 // sum_j Sy[n][j] t1[k][j][m], mode solves, and back the same way.
 template <typename T>
 void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTables& tab, const T* f, T* t1, T* t2,
-                T* out, bool accumulate, std::vector<SepStage<T>>& stages, bool split = false, bool lines = false) {
+                T* out, bool accumulate, std::vector<SepStage<T>>& stages, bool split = false, bool lines = false,
+                bool grouped = false) {
     const int nxi = g.nx - 2, nyi = g.ny - 2, nzi = dim == 3 ? g.nz - 2 : 1;
     if (nxi < 1 || nyi < 1 || nzi < 1) return;
     const long long pl = (long long)nxi * nyi;
@@ -800,7 +804,7 @@ void plan_level(const Geom& g, int dim, const PlaneCoef<T>* coef, const SepTable
     auto plane = [&](const PlaneArgs<T>& p) {
         if constexpr (sizeof(T) == 8)
             if (tab.gp) return split_plane_stage(p, tab.gp, nzi);
-        return plane_stage<T>(p, nzi);
+        return plane_stage<T>(p, nzi, grouped);
     };
     if (planes) {   // x lines of f -> t1[k][m][n], mode solves, y lines back and x -> out, scaled
         PlaneArgs<T> p;
@@ -1205,7 +1209,7 @@ template <typename T>
 void sep_exact_plan(mhs_ctx* c, Hierarchy& H, int l, std::vector<SepStage<T>>& stages) {
     (void)c;
     LevelArrays<T>& A = arrays_of<T>(H, l);
-    plan_level<T>(H.g[l], H.dim, A.coef, tables<T>(H, l), A.f, A.r, A.t, A.u, false, stages);
+    plan_level<T>(H.g[l], H.dim, A.coef, tables<T>(H, l), A.f, A.r, A.t, A.u, false, stages, false, false, true);
 }
 
 template <typename T>

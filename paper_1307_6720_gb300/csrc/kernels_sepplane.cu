@@ -1,7 +1,8 @@
 // Separable solve of one level with the sine transforms of each plane fused
 // into one kernel: the coarse-grid solves of the V-cycles (and any other
 // single-level separable solve whose planes fit the shared memory of a
-// thread-block cluster).
+// thread-block cluster) on levels with fast transforms: those of at most 128
+// cells a side take dense planes (FP64: smaller ones, or digit products).
 //
 // The staged separable solve (kernels_sep.cu) runs one launch per transform
 // pass (x, y, mode solves, inverse y, inverse x) with the transformed data

@@ -443,13 +443,15 @@ __device__ __forceinline__ void resid_restrict_body(const Geom& gf, const Geom& 
 // SM; every chunk recomputes one fine plane of its neighbour, so single planes
 // only while they leave at most four blocks per SM (a march is latency: with
 // chunks of four, 65^3 mixed solves 0.99 against 0.94 ms; with chunks of one,
-// 129^3 1.15 against 1.14 with two)
-inline dim3 resid_restrict_grid(const Geom& gc, int d3) {
+// 129^3 1.15 against 1.14 with two).  Grouped launches have blocks enough of
+// other instances: chunks of four (78 instances of 33^3 32 -> 27 us a launch).
+inline dim3 resid_restrict_grid(const Geom& gc, int d3, bool grouped = false) {
     const int gx = (gc.nx - 2 + RR_X - 1) / RR_X, gy = (gc.ny - 2 + RR_Y - 1) / RR_Y;
     if (!d3) return dim3(gx, gy, 1);
     const int nkc = gc.nz - 2;
     int per = std::max(1, (nkc * gx * gy + 152 * 8 - 1) / (152 * 8));
     if (nkc * gx * gy > 152 * 4) per = std::max(per, 2);
+    if (grouped) per = std::max(per, std::min(4, nkc));
     return dim3(gx, gy, (nkc + per - 1) / per);
 }
 
