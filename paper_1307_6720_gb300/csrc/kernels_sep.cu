@@ -434,12 +434,13 @@ size_t dense2d_smem(int nxi, int nyi, int sp, int so) {
 }
 
 // one thread per result of a line (the staged form: one transform per
-// launch): plane_dot's sums on the folded line
+// launch): plane_dot's sums on the folded line; blocks of 64, a warp's results
+// of one parity
 template <typename T>
 __global__ void sep_line_kernel(int lines, int M, const T* in, long long in_plane, long long in_line, T* out,
                                 long long out_plane, long long out_line, long long out_elem,
                                 const T* __restrict__ s, T scale, int accumulate) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y, k = blockIdx.z;
+    const int m = blockIdx.x * 64 + 2 * (threadIdx.x & 31) + (threadIdx.x >> 5), l = blockIdx.y, k = blockIdx.z;
     if (m >= M || l >= lines) return;
     const T* x = in + k * in_plane + l * in_line;
     const int Ko = (M + 1) / 2, Ke = M / 2, par = m & 1, p = m >> 1, K = par ? Ke : Ko;
