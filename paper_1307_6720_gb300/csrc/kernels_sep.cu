@@ -34,6 +34,7 @@
 #include "device_util.cuh"
 #include "dst_body.cuh"
 #include "group.h"
+#include "launch_rules.h"
 #include "mhs_internal.h"
 #include "solver.h"
 
@@ -760,11 +761,8 @@ SepStage<T> gemm_stage(const GemmArgs<T>& g, int batch) {
 }
 
 // The plane transforms as one stage, both directions: along lines of M1
-// elements first.  Blocks of as many results as leave a block per SM (FP64:
-// down to one odd and one even result, FP32: four of each).  Grouped launches
-// have blocks enough of other instances: eight results of either parity per
-// block (1024 FP32 solves of 33^3 42.7 -> 40.0 ms, 256 in FP64 16.4 -> 13.3 ms;
-// with sixteen, 64 FP64 solves of 65 x 65 x 33 7.75 instead of 7.63 ms).
+// elements first.  Blocks of plane_results results of either parity (FP64:
+// down to one, FP32: four).
 template <typename T>
 SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes, bool grouped) {
     SepStage<T> s;
@@ -772,9 +770,7 @@ SepStage<T> plane_stage(const PlaneArgs<T>& p, int planes, bool grouped) {
     s.plane = p;
     s.threads = PLANE_T;
     const int Ko1 = (p.M1 + 1) / 2, least = sizeof(T) == 4 ? 4 : 1;
-    int sp = grouped ? 8 : 16;
-    if (grouped) while (sp / 2 >= Ko1 && sp > least) sp /= 2;
-    while (!grouped && sp > least && (long long)((Ko1 + sp - 1) / sp) * planes < 152) sp /= 2;
+    int sp = plane_results(Ko1, planes, least, grouped);
     while (sp > least && PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T) > PLANE_SMEM) sp /= 2;
     s.plane.sp = sp;
     s.smem = PlaneLayout<T>(p.A, p.M1, sp).total * sizeof(T);
