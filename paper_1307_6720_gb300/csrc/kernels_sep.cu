@@ -1059,16 +1059,15 @@ bool sep_level_ok(const Geom& g) {
 }
 
 // The levels whose planes are transformed by plane_body: at most 128 cells a
-// side, and in FP64 those whose dense products take the FP64 pipe less time
-// than the fast transforms' chain of steps (one plane, or short lines), or
-// that have no fast transform.
+// side, where there are no fast transforms or they are slower.
 template <typename T>
 static bool dense_planes(const Geom& g, int dim) {
     const int big = std::max(g.nx, g.ny) - 1, least = sizeof(T) == 4 ? 4 : 1;
     if (big > PLANE_CELLS || PlaneLayout<T>(g.ny - 2, g.nx - 2, least).total * sizeof(T) > PLANE_SMEM ||
         PlaneLayout<T>(g.nx - 2, g.ny - 2, least).total * sizeof(T) > PLANE_SMEM)
         return false;
-    return sizeof(T) == 4 || big <= (dim == 2 ? 64 : 32) || !(pow2(g.nx - 1) && pow2(g.ny - 1));
+    return !(pow2(g.nx - 1) && pow2(g.ny - 1)) ||
+           dense_planes_faster(sizeof(T) == 8, dim, g.nx - 1, g.ny - 1, dim == 3 ? g.nz - 2 : 1);
 }
 
 // Mode eigenvalues, and twiddles or sine matrices, of level l in T, built once

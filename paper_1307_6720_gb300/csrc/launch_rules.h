@@ -25,4 +25,42 @@ inline int plane_results(int ko, int planes, int least, bool grouped) {
     return sp;
 }
 
+// Whether a level of cx x cy cells (powers of two, at most 128) and `planes`
+// planes takes the dense plane transforms or the fast ones, by device time of
+// its transforms (us, fast / dense; two launches on 3D levels).
+//
+// A dense plane is O(n) per node but one launch of few steps; the fast ones are
+// a chain of short steps that a wave of planes shares.  So dense loses
+// - in FP64, whose pipe it fills, with 32 cells from about a wave of planes:
+//   33 x 33 nodes 63 planes 29.7 / 25.8, 127 planes 38.6 / 41.7, 511 planes
+//   108 / 136; 33 x 17 nodes 127 planes 28.9 / 27.3, 255 planes 35.4 / 43.6;
+//   33 x 9 nodes 127 planes 26.4 / 21.6, 191 planes 27.3 / 32.4.  17 x 17 nodes
+//   stay ahead (127 planes 26.2 / 17.5, 2047 planes 167 / 128), 65 x 33 lose at
+//   any count (one plane: 25.7 / 13.7);
+// - in FP32 where the short side is far below a warp's 32 lanes, which the long
+//   side's matrix then feeds badly: 129 x 9 nodes 31 planes 14.5 / 14.3, 39 planes
+//   15.0 / 16.1; 129 x 17 nodes 127 planes 25.4 / 24.3, 191 planes 29.4 / 32.7;
+//   65 x 9 nodes 191 planes 15.9 / 14.6, 255 planes 15.9 / 16.2; 65 x 17 nodes
+//   511 planes 28.4 / 27.4, 1023 planes 44.4 / 46.4;
+// - with 128 x 128 cells in FP32 by the count of waves, of four blocks a plane,
+//   20 us each and pass, against two, 37 us each: 31 planes (one wave) 47.5 / 35.9,
+//   63 planes 77.9 / 84.1, 95 planes 151 / 124, 127 planes 152 / 163, 191 planes
+//   226 / 240, 255 planes 300 / 285;
+// - on single FP32 planes of 128 cells, in one cluster either way: 129 x 33 nodes
+//   11.8 / 13.3, 129 x 129 17.4 / 17.9; 65 x 65 12.2 / 10.8.
+inline bool dense_planes_faster(bool fp64, int dim, int cx, int cy, int planes) {
+    const int big = std::max(cx, cy), small = std::min(cx, cy);
+    if (dim == 2) return big <= 64;
+    if (fp64)
+        return big <= 16 || (big == 32 && planes <= RULE_SMS && (long long)(cx - 1) * (cy - 1) * planes <= 100000);
+    if (big <= 32) return true;
+    if (small == 128) {
+        const int dense = (4 * planes + RULE_SMS - 1) / RULE_SMS, fast = (2 * planes + RULE_SMS - 1) / RULE_SMS;
+        return dense == 1 || dense * 20 <= fast * 37;
+    }
+    if (small > 16) return true;
+    if (big == 64) return planes <= (small == 16 ? 512 : 192);
+    return planes <= (small == 16 ? RULE_SMS : 32);
+}
+
 }  // namespace mhs

@@ -710,3 +710,33 @@ def test_coarse_planes_as_digit_products(M, shape):
     for other in got[1:]:
         assert np.array_equal(got[0], other)
     M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("prec,shape", [(0, (33, 33, 97)), (0, (33, 33, 113)), (0, (33, 9, 153)), (0, (33, 9, 161)),
+                                        (1, (129, 9, 33)), (1, (129, 9, 41)), (1, (129, 129, 41)), (1, (65, 9, 193)),
+                                        (1, (65, 9, 257)), (1, (129, 33, 5)), (1, (65, 65, 5))])
+def test_transforms_on_either_side_of_the_plane_counts(M, prec, shape):
+    """Levels just below and above the plane counts where fast transforms take
+    over from dense planes, and lower boundaries of 64 and 128 cells: the
+    separable direct solution, and the staged form bit for bit.  Bounds: those
+    of test_exact_op_parity."""
+    from oracle import exact
+    nx, ny, nz = shape
+    pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
+    for dim in (3, 2):
+        shape_l = (nz, ny, nx) if dim == 3 else (ny, nx)
+        f = np.random.default_rng(nx + nz + dim).standard_normal(shape_l)
+        if prec == 1:
+            f = f.astype(np.float32).astype(np.float64)
+        got = []
+        for flags in (0, M.MHS_FLAG_STAGED_TRANSFORMS):
+            M.mhs_set_options(h, flags=flags)
+            M.mhs_level_write(h, dim, 0, M.MHS_FIELD_U, prec, np.zeros(shape_l))
+            M.mhs_level_write(h, dim, 0, M.MHS_FIELD_F, prec, f)
+            M.mhs_level_op(h, dim, 0, M.MHS_OP_EXACT, prec)
+            got.append(_read(M, h, dim, 0, M.MHS_FIELD_U, prec))
+        prl = _level_problem(M, h, pr, dim, 0)
+        want = exact.separable_solve3d(prl, np.zeros((ny, nx)), f) if dim == 3 else exact.separable_solve2d(prl, -f)
+        assert _rel(got[0], want) < (1e-12 if prec == 0 else 2e-5), dim
+        assert np.array_equal(got[0], got[1]), dim
+    M.mhs_destroy(h)

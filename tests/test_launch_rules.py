@@ -12,6 +12,7 @@ SOURCE = """
 #include "launch_rules.h"
 extern "C" {
 int plane_results(int ko, int planes, int least, int grouped) { return mhs::plane_results(ko, planes, least, grouped != 0); }
+int dense_planes_faster(int fp64, int dim, int cx, int cy, int planes) { return mhs::dense_planes_faster(fp64 != 0, dim, cx, cy, planes); }
 }
 """
 
@@ -39,3 +40,34 @@ def test_plane_blocks_have_no_room_for_twice_their_results(rules, least, grouped
             assert sp == least or sp < 2 * ko, (ko, planes)
             if not grouped and sp > least:
                 assert -(-ko // sp) * planes >= 152 or sp // 2 < least, (ko, planes)
+
+
+# device time (us) of a level's transforms, both directions: precision (0 FP64, 1 FP32), cells, planes (0: the
+# lower boundary), fast, dense
+TRANSFORM_TIMES = [
+    (0, 8, 8, 3, 24.0, 10.0), (0, 8, 8, 511, 44.7, 18.7), (0, 8, 8, 2047, 146.2, 50.5), (0, 16, 16, 255, 27.8, 26.1),
+    (0, 16, 16, 2047, 167.4, 127.7), (0, 32, 32, 3, 27.6, 12.9), (0, 32, 32, 63, 29.7, 25.8), (0, 32, 32, 127, 38.6, 41.7),
+    (0, 32, 32, 255, 57.1, 72.4), (0, 32, 32, 2047, 362.2, 448.9), (0, 16, 32, 127, 28.9, 27.3), (0, 16, 32, 255, 35.4, 43.6),
+    (0, 32, 16, 127, 28.7, 27.1), (0, 32, 16, 255, 35.6, 44.1), (0, 32, 16, 2047, 223.2, 254.7), (0, 32, 8, 127, 26.4, 21.6),
+    (0, 32, 8, 191, 27.3, 32.4), (0, 32, 8, 511, 50.3, 56.8), (0, 8, 32, 255, 27.8, 32.9), (0, 32, 4, 127, 24.6, 19.2),
+    (0, 32, 4, 191, 24.4, 27.7), (0, 16, 8, 2047, 151.8, 80.8), (0, 64, 64, 0, 27.1, 18.2), (0, 64, 32, 0, 25.7, 13.7),
+    (0, 64, 4, 0, 22.1, 11.6),
+    (1, 8, 8, 2047, 42.8, 28.8), (1, 16, 16, 1023, 27.0, 20.5), (1, 32, 32, 2047, 80.6, 66.7), (1, 16, 32, 511, 19.6, 17.4),
+    (1, 32, 8, 511, 15.5, 15.1), (1, 32, 4, 255, 14.1, 11.4), (1, 64, 64, 3, 14.4, 12.2), (1, 64, 64, 1023, 177.2, 113.6),
+    (1, 64, 32, 2047, 139.8, 119.6), (1, 64, 16, 255, 19.9, 18.2), (1, 64, 16, 511, 28.4, 27.4), (1, 64, 16, 1023, 44.4, 46.4),
+    (1, 64, 16, 2047, 82.0, 84.1), (1, 64, 8, 191, 15.9, 14.6), (1, 64, 8, 319, 16.6, 19.0), (1, 8, 64, 511, 19.5, 23.3),
+    (1, 64, 4, 191, 14.3, 13.6), (1, 64, 4, 255, 14.8, 15.5), (1, 128, 64, 3, 16.4, 15.8), (1, 128, 64, 511, 289.6, 153.5),
+    (1, 128, 32, 255, 51.6, 48.5), (1, 128, 32, 1023, 177.8, 154.8), (1, 128, 16, 127, 25.4, 24.3), (1, 128, 16, 191, 29.4, 32.7),
+    (1, 16, 128, 511, 46.0, 62.8), (1, 128, 8, 31, 14.5, 14.3), (1, 128, 8, 39, 15.0, 16.1), (1, 128, 8, 511, 26.9, 52.1),
+    (1, 128, 128, 31, 47.5, 35.9), (1, 128, 128, 39, 77.1, 81.4), (1, 128, 128, 63, 78.5, 84.0), (1, 128, 128, 95, 151.0, 124.1),
+    (1, 128, 128, 127, 151.9, 162.5), (1, 128, 128, 191, 225.6, 240.4), (1, 128, 128, 255, 299.5, 285.1), (1, 64, 64, 0, 12.2, 10.8),
+    (1, 64, 8, 0, 10.7, 9.0), (1, 128, 128, 0, 17.4, 17.9), (1, 128, 64, 0, 13.5, 14.1), (1, 128, 32, 0, 11.8, 13.3),
+    (1, 128, 8, 0, 10.7, 11.9),
+]
+
+
+@pytest.mark.parametrize("prec,cx,cy,planes,fast,dense", TRANSFORM_TIMES)
+def test_transforms_of_a_level_take_the_faster_form(rules, prec, cx, cy, planes, fast, dense):
+    """The rule picks the form that measured faster at every measured size."""
+    pick = rules.dense_planes_faster(1 - prec, 3 if planes else 2, cx, cy, max(planes, 1))
+    assert bool(pick) == (dense < fast)
