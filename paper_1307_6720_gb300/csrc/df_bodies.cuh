@@ -14,9 +14,8 @@
 // contracting or reassociating the transformations.
 #pragma once
 
-#include <algorithm>
-
 #include "device_util.cuh"
+#include "launch_rules.h"
 #include "mhs_internal.h"
 
 namespace mhs {
@@ -309,24 +308,10 @@ __device__ __forceinline__ void df_march_body(const Geom& g, const PlaneCoefDF* 
 }
 
 // blocks of df_march_body: tiles of the quads with interior nodes by eight
-// rows and chunks of planes, the count of chunks with the least waves of
-// resident blocks (two per SM) times planes, three of them start-up; at most
-// max_blocks partials
+// rows, and chunks of planes; at most max_blocks partials
 inline dim3 df_march_grid(const Geom& g, int max_blocks) {
-    const int gx = ((g.nx - 2) / 4 + 1 + DQ_X - 1) / DQ_X, gy = (g.ny - 2 + DQ_Y - 1) / DQ_Y, nzi = g.nz - 2;
-    const long long tiles = (long long)gx * gy, resident = 2 * 152;
-    long long best = 0;
-    int chunks = 1;
-    for (int n = 1; n <= std::max(1, nzi / 4); ++n) {
-        const int per = (nzi + n - 1) / n, m = (nzi + per - 1) / per;
-        if (n > 1 && max_blocks > 0 && tiles * m > max_blocks) break;
-        const long long cost = (tiles * m + resident - 1) / resident * (per + 3);
-        if (n == 1 || cost < best) {
-            best = cost;
-            chunks = m;
-        }
-    }
-    return dim3(gx, gy, chunks);
+    const int gx = ((g.nx - 2) / 4 + 1 + DQ_X - 1) / DQ_X, gy = (g.ny - 2 + DQ_Y - 1) / DQ_Y;
+    return dim3(gx, gy, df_march_chunks((long long)gx * gy, g.nz - 2, max_blocks));
 }
 
 // (hi, lo) += e

@@ -63,4 +63,26 @@ inline bool dense_planes_faster(bool fp64, int dim, int cx, int cy, int planes) 
     return planes <= (small == 16 ? RULE_SMS : 32);
 }
 
+// Chunks of the nzi inner planes of the double-float march (df_march_body) over
+// `tiles` tiles: the count with the least waves of resident blocks (two per
+// SM) times planes, three of them start-up; at most max_blocks blocks (0: any)
+// unless the tiles alone are more.  Down to single planes, or a shallow level
+// is marched by its few tiles (129 x 129 x 9 in one chunk of seven planes: 16
+// blocks; a direct mixed solve 205 us, with single planes 190 us).
+inline int df_march_chunks(long long tiles, int nzi, int max_blocks) {
+    const long long resident = 2 * RULE_SMS;
+    long long best = 0;
+    int chunks = 1;
+    for (int n = 1; n <= nzi; ++n) {
+        const int per = (nzi + n - 1) / n, m = (nzi + per - 1) / per;
+        if (n > 1 && max_blocks > 0 && tiles * m > max_blocks) break;
+        const long long cost = (tiles * m + resident - 1) / resident * (per + 3);
+        if (n == 1 || cost < best) {
+            best = cost;
+            chunks = m;
+        }
+    }
+    return chunks;
+}
+
 }  // namespace mhs

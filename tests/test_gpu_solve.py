@@ -569,7 +569,8 @@ def test_fields_destinations(M, shape):
     M.mhs_destroy(h)
 
 
-@pytest.mark.parametrize("shape", [(97, 33, 17), (95, 33, 17), (107, 19, 11), (261, 13, 9), (129, 9, 33)])
+@pytest.mark.parametrize("shape", [(97, 33, 17), (95, 33, 17), (107, 19, 11), (261, 13, 9), (129, 9, 33), (129, 129, 9),
+                                   (97, 5, 5)])
 def test_mixed_step_on_wide_levels(M, shape):
     """Mixed mode on grids around the width from which correction and residual
     run as one pass over quads (ragged quads, one and several tiles along x):

@@ -13,6 +13,7 @@ SOURCE = """
 extern "C" {
 int plane_results(int ko, int planes, int least, int grouped) { return mhs::plane_results(ko, planes, least, grouped != 0); }
 int dense_planes_faster(int fp64, int dim, int cx, int cy, int planes) { return mhs::dense_planes_faster(fp64 != 0, dim, cx, cy, planes); }
+int df_march_chunks(long long tiles, int nzi, int max_blocks) { return mhs::df_march_chunks(tiles, nzi, max_blocks); }
 }
 """
 
@@ -24,7 +25,9 @@ def rules(tmp_path_factory):
     src.write_text(SOURCE)
     subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(lib)],
                    check=True)
-    return ctypes.CDLL(str(lib))
+    lib = ctypes.CDLL(str(lib))
+    lib.df_march_chunks.argtypes = [ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    return lib
 
 
 @pytest.mark.parametrize("least", [1, 4])
@@ -71,3 +74,22 @@ def test_transforms_of_a_level_take_the_faster_form(rules, prec, cx, cy, planes,
     """The rule picks the form that measured faster at every measured size."""
     pick = rules.dense_planes_faster(1 - prec, 3 if planes else 2, cx, cy, max(planes, 1))
     assert bool(pick) == (dense < fast)
+
+
+def test_double_float_march_fills_the_chip_on_shallow_levels(rules):
+    """Chunks of the double-float march: never empty, never over the limit of
+    partial sums, never slower by the rule's own measure than any other
+    count, and single planes where the tiles are few."""
+    for tiles in (1, 2, 3, 5, 16, 33, 64, 110, 152, 305, 1024):
+        for nzi in (1, 2, 3, 5, 7, 9, 15, 31, 63, 127, 255, 511):
+            n = rules.df_march_chunks(tiles, nzi, 65536)
+            per = -(-nzi // n)
+            assert 1 <= n <= nzi and (n - 1) * per < nzi
+            assert n == 1 or tiles * n <= 65536
+            cost = -(-tiles * n // 304) * (per + 3)
+            for p in range(1, nzi + 1):
+                m = -(-nzi // p)
+                if tiles * m <= 65536:
+                    assert cost <= -(-tiles * m // 304) * (p + 3), (tiles, nzi, n, m)
+    assert rules.df_march_chunks(16, 7, 65536) == 7
+    assert rules.df_march_chunks(300, 200, 700) * 300 <= 700 and rules.df_march_chunks(1000, 200, 700) == 1
