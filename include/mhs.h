@@ -107,10 +107,10 @@ typedef struct {
                             the one-CTA shared-memory sub-cycle [1200] */
     int cut32;           /* same for FP32 levels [4000] */
     int fused_min;       /* FP32 3D levels with at least this many interior nodes use the fused, TMA-staged
-                            red-black sweep (one pass per sweep) for the sweeps that do not run in pairs (two
-                            sweeps per pass: levels of 800,000 nodes and more with nx = 4m + 1); smaller levels use
-                            the two colour passes, which have less latency; results do not depend on it
-                            [12000000] */
+                            red-black sweep (one pass per sweep) when no two sweeps of theirs run as one pass,
+                            which levels of nx = 4m + 1 and some 1.2 million nodes do with nu1, nu2 of two and
+                            more (a sweep left over there runs as colour passes); smaller levels use the two
+                            colour passes, which have less latency; results do not depend on it [12000000] */
     int sep_coarse;      /* coarse-grid solve of the V-cycles: the first level below the finest with at most this
                             many interior nodes, whose sine transforms are fast (nx - 1 and ny - 1 powers of two)
                             or short (nx, ny <= 66), is solved exactly by the separable solver (sine transforms

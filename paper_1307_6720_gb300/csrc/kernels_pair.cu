@@ -37,9 +37,8 @@
 // slots are 128-byte aligned, every mbarrier wait is bounded.
 #include <cuda.h>
 
-#include <algorithm>
-
 #include "device_util.cuh"
+#include "launch_rules.h"
 #include "mhs_internal.h"
 #include "tma_util.cuh"
 
@@ -47,10 +46,10 @@ namespace mhs {
 
 namespace {
 
-constexpr int QUADS = 32;          // quads of a tile (lanes)
+constexpr int QUADS = PAIR_QUADS;  // quads of a tile (lanes)
 constexpr int PBW = 4 * QUADS + 4; // floats per box row: the tile and the quad east of it
 constexpr int NS = 3;              // ring slots (half the unrolled steps, so slots and phases are constants)
-constexpr int MAX_CHUNK = 256;     // most planes of a chunk
+constexpr int MAX_CHUNK = PAIR_CHUNK;
 
 template <int NW>
 struct PairShape {
@@ -295,24 +294,10 @@ void launch_pair(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap& tm_f
         MHS_CUDA(cudaFuncSetAttribute(rb_pair_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::BYTES)));
         attr = true;
     }
-    const int nqi = (g.nx - 2) / 4 + 1;
-    const int gx = nqi <= QUADS ? 1 : (nqi - QUADS + QUADS - 3) / (QUADS - 2) + 1;
-    const int gy = g.ny <= S::H ? 1 : (g.ny - S::H + S::H - 9) / (S::H - 8) + 1;
-    // chunks of an even count of planes; a chunk runs eight planes more than
-    // it stores and starts up for about two: the count of chunks with the
-    // least waves of resident blocks times steps
-    const long long resident = 152, tiles = (long long)gx * gy;
-    long long best = 0;
-    int kchunk = 0;
-    for (int c = std::max(1, (g.nz + MAX_CHUNK - 1) / MAX_CHUNK); c <= std::max(1, g.nz / 4) + 1; ++c) {
-        const int kc = std::min(MAX_CHUNK, ((g.nz + c - 1) / c + 1) / 2 * 2), n = (g.nz + kc - 1) / kc;
-        const long long cost = (tiles * n + resident - 1) / resident * (kc + 10);
-        if (!kchunk || cost < best) {
-            best = cost;
-            kchunk = kc;
-        }
-    }
-    const dim3 grid(gx, gy, (g.nz + kchunk - 1) / kchunk);
+    static_assert(S::H == PAIR_ROWS, "the rows that the rule counts with");
+    const PairShapeOf p = pair_shape(g.nx, g.ny, g.nz);
+    const int kchunk = p.chunk;
+    const dim3 grid(p.gx, p.gy, (g.nz + kchunk - 1) / kchunk);
     rb_pair_kernel<NW><<<grid, 32 * NW, S::BYTES, st>>>(tm_u, tm_f, g, coef, uout, kchunk, err);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
@@ -326,12 +311,7 @@ void make_pair_map(CUtensorMap* map, const Geom& g, const float* base) {
     make_box_map(map, g, base, PBW, PairShape<PAIR_WARPS>::H);
 }
 
-// Pairs from 800,000 interior nodes up: below, four colour passes stay in
-// cache and a march of few planes is all start-up (a 65^3 mixed solve 1.15
-// against 1.04 ms with pairs on its finest level; from 129 x 129 x 65 up the
-// pass is level or ahead: 129^3 solves 1.30 against 1.33 ms, 257^3 5.10
-// against 5.59).  nx = 4m + 1: see PairTile.
-bool pair_level(const Geom& g) { return (g.nx & 3) == 1 && g.interior() >= 800000; }
+bool pair_level(const Geom& g) { return pair_pays(g.nx, g.ny, g.nz); }
 
 void launch_pair_sweep(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap& tm_f,
                        const PlaneCoef<float>* coef, float* uout, int* err, cudaStream_t st) {

@@ -85,4 +85,48 @@ inline int df_march_chunks(long long tiles, int nzi, int max_blocks) {
     return chunks;
 }
 
+// Tiles of the pairs of sweeps (kernels_pair.cu): 32 quads of nodes, of which 30
+// inside a row are stored, by 32 rows, of which all but four at either end are.
+constexpr int PAIR_QUADS = 32, PAIR_ROWS = 32, PAIR_CHUNK = 256;   // (most planes of a chunk)
+struct PairShapeOf {
+    int gx, gy, chunk;   // tiles, planes of a chunk (even)
+    long long steps;     // of the march: waves of one block per SM, times planes and start-up
+};
+// Chunks of an even count of planes; a chunk runs eight planes more than it
+// stores and starts up for about two: the count of chunks with the least steps.
+inline PairShapeOf pair_shape(int nx, int ny, int nz) {
+    PairShapeOf s{};
+    const int quads = (nx - 2) / 4 + 1;
+    s.gx = quads <= PAIR_QUADS ? 1 : (quads - PAIR_QUADS + PAIR_QUADS - 3) / (PAIR_QUADS - 2) + 1;
+    s.gy = ny <= PAIR_ROWS ? 1 : (ny - PAIR_ROWS + PAIR_ROWS - 9) / (PAIR_ROWS - 8) + 1;
+    const long long tiles = (long long)s.gx * s.gy;
+    for (int c = std::max(1, (nz + PAIR_CHUNK - 1) / PAIR_CHUNK); c <= std::max(1, nz / 4) + 1; ++c) {
+        const int kc = std::min(PAIR_CHUNK, ((nz + c - 1) / c + 1) / 2 * 2), n = (nz + kc - 1) / kc;
+        const long long steps = (tiles * n + RULE_SMS - 1) / RULE_SMS * (kc + 10);
+        if (!s.chunk || steps < s.steps) {
+            s.steps = steps;
+            s.chunk = kc;
+        }
+    }
+    return s;
+}
+
+// Levels whose pairs of sweeps run as one pass: those where its march takes less
+// time than four colour passes.  nx = 4m + 1: see PairTile.  A step takes 1.04 us;
+// the colour passes, up to three million nodes, 7.45 us more than the march's start
+// and 5.57 us per million nodes, rows counted in whole warps of 64 nodes (fitted to
+// whole mixed solves of 62 boxes of 0.9 to 2.9 million nodes; the rule is right on
+// every one where the two differ by 0.4 us).  Four passes against one, us more (+)
+// or less (-) for the one: 129^3 -1.4, 113^3 -2.1, 97 x 97 x 193 -4.1; 129 x 129 x 65
+// +1.4, 65 x 65 x 513 +4.1, 33 x 33 x 1025 +6.9, 17 x 33 x 2049 +9.6 (31 of 128
+// columns of its tiles used).  Past three million the passes leave the cache:
+// 257 x 129 x 129 -8.2, 33 x 129 x 1025 -36.  Levels of less than 800,000 nodes keep
+// the passes (65^3 mixed solves 1.04 ms with them, 1.15 ms with pairs).
+inline bool pair_pays(int nx, int ny, int nz) {
+    const long long rows = (long long)(ny - 2) * (nz - 2), nodes = rows * (nx - 2);
+    if ((nx & 3) != 1 || nodes < 800000) return false;
+    const double padded = double((nx - 2 + 63) / 64 * 64) * double(rows);
+    return nodes >= 3000000 || 1.04 * double(pair_shape(nx, ny, nz).steps) < 7.45 + 5.57e-6 * padded;
+}
+
 }  // namespace mhs

@@ -629,26 +629,48 @@ def test_dense_transform_tiles(M, shape, prec):
     M.mhs_destroy(h)
 
 
-@pytest.mark.parametrize("nu", [(2, 2), (4, 2), (3, 3), (2, 1)])
-@pytest.mark.parametrize("shape", [(129, 129, 65), (193, 97, 49), (249, 129, 33), (129, 33, 257)])
-def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
-    """FP32 V-cycles whose pairs of sweeps run as one out-of-place pass (tiles
-    in x, y and z with ragged ends, boundary values that are not zero, odd
-    sweeps left over) equal the cycles run colour by colour bit for bit."""
+def _vcycles_with_and_without_pairs(M, shape, nu):
+    """One FP32 V-cycle from random u (boundary values too) and f by default and
+    colour by colour: the iterates and the launches of each, and the start."""
     nx, ny, nz = shape
     pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
     rng = np.random.default_rng(nx + nz)
     u, f = rng.standard_normal((2, nz, ny, nx)).astype(np.float32).astype(np.float64)
-    got = []
-    for flags in (0, M.MHS_FLAG_NO_TMA):
+    got, launches = [], []
+    for flags in (M.MHS_FLAG_POINT, M.MHS_FLAG_POINT | M.MHS_FLAG_NO_TMA):
         M.mhs_set_options(h, nu1=nu[0], nu2=nu[1], flags=flags, fused_min=1 << 30)
         M.mhs_level_write(h, 3, 0, M.MHS_FIELD_U, 1, u)
         M.mhs_level_write(h, 3, 0, M.MHS_FIELD_F, 1, f)
+        n0 = M.mhs_kernel_launches()
         M.mhs_level_op(h, 3, 0, M.MHS_OP_VCYCLE, 1)
+        launches.append(M.mhs_kernel_launches() - n0)
         got.append(_read(M, h, 3, 0, M.MHS_FIELD_U, 1))
+    M.mhs_destroy(h)
+    return got, launches, u
+
+
+@pytest.mark.parametrize("nu", [(2, 2), (4, 2), (3, 3), (3, 2), (2, 4)])
+@pytest.mark.parametrize("shape", [(129, 129, 97), (249, 161, 49), (193, 97, 129), (129, 33, 1025), (73, 145, 97)])
+def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
+    """FP32 V-cycles whose pairs of sweeps run as one out-of-place pass (tiles
+    in x, y and z with ragged ends, boundary values that are not zero, odd
+    sweeps left over) equal the cycles run colour by colour bit for bit.  A
+    pair is one launch in place of four."""
+    got, launches, u = _vcycles_with_and_without_pairs(M, shape, nu)
+    pairs = nu[0] // 2 + nu[1] // 2
+    assert launches[1] - launches[0] == 3 * (pairs - pairs % 2)
     assert np.array_equal(got[0], got[1])
     assert not np.array_equal(got[0], u)
-    M.mhs_destroy(h)
+
+
+@pytest.mark.parametrize("shape,nu", [((129, 129, 65), (2, 2)), ((33, 129, 257), (2, 2)), ((17, 33, 2049), (2, 2)),
+                                      ((65, 65, 257), (2, 2)), ((129, 129, 97), (2, 1)), ((129, 129, 97), (1, 1))])
+def test_levels_and_counts_without_pairs(M, shape, nu):
+    """Levels on which the pass of two sweeps would be the slower form, and
+    sweep counts without an even number of pairs, run colour passes."""
+    got, launches, u = _vcycles_with_and_without_pairs(M, shape, nu)
+    assert launches[0] == launches[1]
+    assert np.array_equal(got[0], got[1])
 
 
 @pytest.mark.parametrize("prec", [0, 1])

@@ -14,6 +14,11 @@ extern "C" {
 int plane_results(int ko, int planes, int least, int grouped) { return mhs::plane_results(ko, planes, least, grouped != 0); }
 int dense_planes_faster(int fp64, int dim, int cx, int cy, int planes) { return mhs::dense_planes_faster(fp64 != 0, dim, cx, cy, planes); }
 int df_march_chunks(long long tiles, int nzi, int max_blocks) { return mhs::df_march_chunks(tiles, nzi, max_blocks); }
+int pair_pays(int nx, int ny, int nz) { return mhs::pair_pays(nx, ny, nz); }
+void pair_shape(int nx, int ny, int nz, int* out) {
+    const mhs::PairShapeOf s = mhs::pair_shape(nx, ny, nz);
+    out[0] = s.gx, out[1] = s.gy, out[2] = s.chunk;
+}
 }
 """
 
@@ -93,3 +98,44 @@ def test_double_float_march_fills_the_chip_on_shallow_levels(rules):
                     assert cost <= -(-tiles * m // 304) * (p + 3), (tiles, nzi, n, m)
     assert rules.df_march_chunks(16, 7, 65536) == 7
     assert rules.df_march_chunks(300, 200, 700) * 300 <= 700 and rules.df_march_chunks(1000, 200, 700) == 1
+
+
+# nodes of a box, us that a pair of sweeps in one pass takes more than four colour passes
+PAIR_TIMES = [
+    (17, 33, 2049, 9.6), (17, 65, 1025, 2.7), (17, 129, 513, 2.7), (17, 257, 257, 0.6), (17, 513, 129, 2.5), (17, 1025, 65, 2.6),
+    (33, 33, 1025, 6.9), (33, 65, 513, 4.5), (33, 129, 257, 4.4), (33, 257, 129, 2.2), (33, 513, 65, 4.3), (33, 1025, 33, 4.7),
+    (65, 33, 513, 5.8), (65, 65, 257, 3.9), (65, 129, 129, 3.1), (65, 257, 65, 3.7), (129, 33, 257, 1.1), (129, 17, 513, 1.6),
+    (257, 17, 257, 3.4), (513, 17, 129, 4.1), (1025, 17, 65, 3.6), (2049, 17, 33, 3.8), (257, 33, 129, 3.8), (513, 33, 65, 4.1),
+    (1025, 33, 33, 3.8), (2049, 33, 17, 4.2), (4097, 17, 17, 4.2), (129, 65, 129, 2.1), (129, 129, 65, 1.4), (257, 129, 33, 4.6),
+    (257, 65, 65, 3.9), (129, 257, 33, 1.3), (41, 321, 81, 5.4), (49, 193, 113, 2.7), (73, 145, 97, -1.6), (25, 321, 129, 4.5),
+    (33, 1025, 129, -33.4), (33, 129, 1025, -35.8), (129, 129, 97, -1.5), (129, 129, 81, -0.8), (33, 65, 1025, 2.9),
+    (65, 65, 513, 4.1), (65, 129, 257, 4.2), (129, 129, 129, -1.4), (257, 65, 129, 2.0), (17, 257, 513, -1.9), (17, 513, 257, 2.0),
+    (33, 257, 257, 1.1), (513, 17, 257, 2.4), (1025, 17, 129, 2.4), (257, 257, 33, 2.4), (2049, 17, 65, 2.4), (161, 145, 65, -1.2),
+    (113, 113, 113, -2.1), (97, 97, 193, -4.1), (97, 161, 97, -1.5), (193, 161, 97, -2.5), (33, 33, 2049, 13.3), (65, 1025, 33, 4.3),
+    (161, 161, 97, -2.2), (193, 193, 97, -5.1), (257, 129, 129, -8.2), (33, 513, 257, -36.0), (513, 33, 257, -8.1),
+    (65, 257, 257, -18.6),
+]
+
+
+@pytest.mark.parametrize("nx,ny,nz,more", PAIR_TIMES)
+def test_pairs_of_sweeps_run_as_one_pass_where_that_is_faster(rules, nx, ny, nz, more):
+    """The rule is right on every box where the forms differ by more than the
+    repeats do (0.4 us a pair)."""
+    assert bool(rules.pair_pays(nx, ny, nz)) == (more < 0)
+
+
+def test_pair_tiles_cover_the_level(rules):
+    """Tiles of 30 stored quads of 32 (the first and last also their outer one),
+    24 stored rows of 32 (likewise four), chunks of even length: every node of
+    any box is stored by some block, and no block starts past the box."""
+    out = (ctypes.c_int * 3)()
+    for nx in (5, 9, 17, 125, 129, 133, 245, 249, 253, 257, 261, 1025):
+        for ny in (3, 5, 31, 32, 33, 55, 56, 57, 80, 81, 129, 1025):
+            for nz in (3, 5, 9, 17, 33, 255, 256, 257, 258, 1025):
+                rules.pair_shape(nx, ny, nz, out)
+                gx, gy, chunk = out
+                quads = (nx - 2) // 4 + 1
+                assert 32 + 30 * (gx - 1) >= quads and (gx == 1 or 32 + 30 * (gx - 2) < quads)
+                assert 32 + 24 * (gy - 1) >= ny and (gy == 1 or 32 + 24 * (gy - 2) < ny)
+                assert chunk % 2 == 0 and 2 <= chunk <= 256
+    assert not rules.pair_pays(131, 129, 129) and not rules.pair_pays(65, 65, 65)
