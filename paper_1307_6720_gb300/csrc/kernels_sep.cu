@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs<T> g) {
 // FP32: four results per thread share each loaded element (R = 4).  FP64 is
 // bound by its pipe, so one result per thread spreads a plane furthest.
 constexpr int PLANE_T = 256;
+constexpr int PLANE_CELLS = 128;   // most cells of a side
 
 // shared memory of plane_body (elements; every part a multiple of four)
 template <typename T>
@@ -434,32 +435,46 @@ size_t dense2d_smem(int nxi, int nyi, int sp, int so) {
            sizeof(T);
 }
 
-// one thread per result of a line (the staged form: one transform per
-// launch): plane_dot's sums on the folded line; blocks of 64, a warp's results
-// of one parity
+// One transform per launch (the staged form): plane_dot's sums on folded lines.
+// A block folds LINE_Y plane_r lines into shared memory once, then each thread forms one
+// result of plane_r of them, a warp's results of one parity, every element of the
+// matrix loaded for all of them (folding at each result took two loads and an
+// addition per term: staged mixed solves of 129 x 129 x 33 772 us, now 573 us, FP64
+// ones of 65 x 65 x 33 773 and 570 us).  Blocks of 64 x LINE_Y threads.
+constexpr int LINE_Y = 4;
 template <typename T>
-__global__ void sep_line_kernel(int lines, int M, const T* in, long long in_plane, long long in_line, T* out,
-                                long long out_plane, long long out_line, long long out_elem,
-                                const T* __restrict__ s, T scale, int accumulate) {
-    const int m = blockIdx.x * 64 + 2 * (threadIdx.x & 31) + (threadIdx.x >> 5), l = blockIdx.y, k = blockIdx.z;
-    if (m >= M || l >= lines) return;
-    const T* x = in + k * in_plane + l * in_line;
-    const int Ko = (M + 1) / 2, Ke = M / 2, par = m & 1, p = m >> 1, K = par ? Ke : Ko;
+__global__ void __launch_bounds__(64 * LINE_Y)
+sep_line_kernel(int lines, int M, const T* __restrict__ in, long long in_plane, long long in_line, T* __restrict__ out,
+                long long out_plane, long long out_line, long long out_elem, const T* __restrict__ s, T scale,
+                int accumulate) {
+    constexpr int R = plane_r<T>(), LB = LINE_Y * R, LD = LB + R;
+    __shared__ __align__(16) T F[PLANE_CELLS * LD];   // [element][line]: sums, then differences
+    const int Ko = (M + 1) / 2, Ke = M / 2, l0 = blockIdx.y * LB, k = blockIdx.z;
+    const T* x = in + k * in_plane + l0 * in_line;
+    for (int e = threadIdx.x + 64 * threadIdx.y; e < Ko * LB; e += 64 * LINE_Y) {
+        const int q = e / Ko, i = e - q * Ko, j = M - 1 - i;
+        const bool on = l0 + q < lines;
+        const T lo = on ? x[q * in_line + i] : T(0), hi = on && i != j ? x[q * in_line + j] : T(0);
+        F[i * LD + q] = i == j ? lo : lo + hi;
+        if (i != j) F[(Ko + i) * LD + q] = lo - hi;
+    }
+    __syncthreads();
+    const int m = blockIdx.x * 64 + 2 * (threadIdx.x & 31) + (threadIdx.x >> 5), q0 = threadIdx.y * R;
+    if (m >= M || l0 + q0 >= lines) return;
+    const int par = m & 1, p = m >> 1, K = par ? Ke : Ko;
     const T* S = s + (par ? Ko * Ko : 0) + p;
-    T v[1];
-    plane_dot<T, 1>(
-        K,
-        [&](int i) {
-            const int j = M - 1 - i;
-            return i == j ? x[i] : par ? x[i] - x[j] : x[i] + x[j];
-        },
-        [&](int i, T(&w)[1]) { w[0] = S[i * K]; }, v);
-    T* o = out + k * out_plane + l * out_line + m * out_elem;
-    *o = dst_result(scale, v[0], accumulate != 0, accumulate ? *o : T(0));
+    const T* f = F + (par ? Ko * LD : 0) + q0;
+    T v[R];
+    plane_dot<T, R>(K, [&](int i) { return __ldg(S + i * K); }, [&](int i, T(&w)[R]) { plane_ld<R>(f + i * LD, w); }, v);
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        if (l0 + q0 + q >= lines) break;
+        T* o = out + k * out_plane + (l0 + q0 + q) * out_line + m * out_elem;
+        *o = dst_result(scale, v[q], accumulate != 0, accumulate ? *o : T(0));
+    }
 }
 
 constexpr size_t PLANE_SMEM = 227 * 1024;
-constexpr int PLANE_CELLS = 128;
 
 // Elimination factors of the mode systems of one 3D level, one thread per
 // mode (fast index m, slow index n; the layout of the transformed data),
@@ -948,8 +963,9 @@ void staged_lines(mhs_ctx* c, const Geom& g, int dim, const SepTables& tab, cons
     const T *sx = static_cast<const T*>(tab.fx), *sy = static_cast<const T*>(tab.fy);
     auto pass = [&](int lines, int M, const T* in, long long ip, long long il, T* o, long long op, long long ol,
                     long long oe, const T* s, T scale) {
-        sep_line_kernel<T><<<dim3((M + 63) / 64, lines, nzi), 64, 0, c->stream>>>(lines, M, in, ip, il, o, op, ol, oe, s,
-                                                                                  scale, 0);
+        constexpr int LB = LINE_Y * plane_r<T>();
+        sep_line_kernel<T><<<dim3((M + 63) / 64, (lines + LB - 1) / LB, nzi), dim3(64, LINE_Y), 0, c->stream>>>(
+            lines, M, in, ip, il, o, op, ol, oe, s, scale, 0);
         count_launches(1);
         MHS_CUDA(cudaGetLastError());
     };

@@ -675,7 +675,7 @@ def test_levels_and_counts_without_pairs(M, shape, nu):
 
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("shape", [(5, 5, 5), (7, 5, 9), (9, 33, 5), (35, 19, 5), (67, 67, 9), (65, 63, 9), (129, 9, 5),
-                                   (129, 129, 5), (127, 67, 5)])
+                                   (129, 129, 5), (127, 67, 5), (65, 17, 5), (65, 19, 5), (19, 65, 7), (35, 33, 5)])
 def test_plane_transforms_of_folded_matrices(M, shape, prec):
     """The plane transforms with folded sine matrices (one pair of lines up to
     128 cells, odd and even lengths, ragged slabs of results), 2D and 3D,
