@@ -4,6 +4,7 @@
 
 #include "device_util.cuh"
 #include "mhs_internal.h"
+#include "per_device.h"
 #include "solver.h"
 #include "sub_body.cuh"
 
@@ -26,6 +27,20 @@ void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st) 
     bnorm_kernel<<<1, CHECK_THREADS, 0, st>>>(partial, n, ctl);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
+}
+
+int current_device() {
+    int dev = 0;
+    MHS_CUDA(cudaGetDevice(&dev));
+    return dev;
+}
+
+void allow_smem(const void* kernel, size_t bytes) {
+    static PerDevice<const void*, size_t> limits;
+    limits.get(current_device(), kernel, [&] {
+        MHS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+        return bytes;
+    });
 }
 
 size_t subcycle_smem_limit() { return 220 * 1024; }

@@ -166,11 +166,7 @@ void dst_shape(DstArgs<T>& a, dim3& grid, int& threads, size_t& smem) {
 
 template <typename T>
 void launch_dst_stage(const SepStage<T>& s, cudaStream_t st) {
-    static bool configured = false;   // per template instance
-    if (!configured) {
-        MHS_CUDA(cudaFuncSetAttribute(dst_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(DST_SMEM_MAX)));
-        configured = true;
-    }
+    allow_smem(dst_kernel<T>, DST_SMEM_MAX);
     dst_kernel<T><<<s.grid, s.threads, s.smem, st>>>(s.dst);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
@@ -179,12 +175,7 @@ void launch_dst_stage(const SepStage<T>& s, cudaStream_t st) {
 template <typename T>
 void glaunch_dst(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st) {
     if (t.n == 0) return;
-    static bool configured = false;
-    if (!configured) {
-        MHS_CUDA(
-            cudaFuncSetAttribute(g_dst_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(DST_SMEM_MAX)));
-        configured = true;
-    }
+    allow_smem(g_dst_kernel<T>, DST_SMEM_MAX);
     g_dst_kernel<T><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());

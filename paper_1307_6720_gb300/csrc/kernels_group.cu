@@ -285,12 +285,8 @@ template <typename T>
 void glaunch_zline(const GTable& t, int colour, int sweep, int fmg_step, int gate, cudaStream_t st) {
     if (!t.n) return;
     if constexpr (sizeof(T) == 4) {
-        static bool attr = false;
-        if (!attr) {
-            MHS_CUDA(cudaFuncSetAttribute(g_zline_part_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            MHS_CUDA(cudaFuncSetAttribute(g_zline_part_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            attr = true;
-        }
+        if (t.ty <= 8) allow_smem(g_zline_part_kernel<8>, 227 * 1024);
+        else allow_smem(g_zline_part_kernel<32>, 227 * 1024);
         const dim3 blk(32, t.ty);
         if (t.ty <= 8) g_zline_part_kernel<8><<<t.blocks, blk, t.smem, st>>>(t.items, t.n, colour, sweep, fmg_step, gate);
         else g_zline_part_kernel<32><<<t.blocks, blk, t.smem, st>>>(t.items, t.n, colour, sweep, fmg_step, gate);

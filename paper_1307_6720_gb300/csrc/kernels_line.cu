@@ -34,12 +34,8 @@ void launch_zline(const Geom& g, const PlaneCoef<T>* coef, T* u, const T* f, T* 
     if constexpr (sizeof(T) == 4) {
         const int n = g.nz - 2, S = zpart_segments(n);
         const size_t smem = zpart_smem(n, S);   // up to 172 KB (1024 planes, 32 segments)
-        static bool attr = false;
-        if (!attr) {
-            MHS_CUDA(cudaFuncSetAttribute(zline_part_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            MHS_CUDA(cudaFuncSetAttribute(zline_part_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            attr = true;
-        }
+        if (S <= 8) allow_smem(zline_part_kernel<8>, 227 * 1024);
+        else allow_smem(zline_part_kernel<32>, 227 * 1024);
         const dim3 grid = zline_part_grid(g);
         for (int colour = 0; colour < 2; ++colour) {
             if (S <= 8) zline_part_kernel<8><<<grid, dim3(32, S), smem, st>>>(g, coef, u, f, colour, hx);

@@ -289,11 +289,7 @@ template <int NW>
 void launch_pair(const Geom& g, const CUtensorMap& tm_u, const CUtensorMap& tm_f, const PlaneCoef<float>* coef,
                  float* uout, int* err, cudaStream_t st) {
     using S = PairShape<NW>;
-    static bool attr = false;
-    if (!attr) {
-        MHS_CUDA(cudaFuncSetAttribute(rb_pair_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::BYTES)));
-        attr = true;
-    }
+    allow_smem(rb_pair_kernel<NW>, S::BYTES);
     static_assert(S::H == PAIR_ROWS, "the rows that the rule counts with");
     const PairShapeOf p = pair_shape(g.nx, g.ny, g.nz);
     const int kchunk = p.chunk;

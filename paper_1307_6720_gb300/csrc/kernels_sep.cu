@@ -27,8 +27,7 @@
 
 #include <algorithm>
 #include <cmath>
-#include <map>
-#include <mutex>
+#include <utility>
 #include <vector>
 
 #include "device_util.cuh"
@@ -36,6 +35,7 @@
 #include "group.h"
 #include "launch_rules.h"
 #include "mhs_internal.h"
+#include "per_device.h"
 #include "solver.h"
 
 namespace mhs {
@@ -906,27 +906,15 @@ void launch_stage(const SepStage<T>& s, cudaStream_t st) {
     case SEP_GEMM:
         if constexpr (sizeof(T) == 4) gemm_kernel<T><<<s.grid, s.threads, 0, st>>>(s.gemm);
         break;
-    case SEP_SCAN: {
-        static bool configured = false;   // per template instance
-        if (!configured) {
-            MHS_CUDA(cudaFuncSetAttribute(sep_scan_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          int(SCAN_SMEM_MAX)));
-            configured = true;
-        }
+    case SEP_SCAN:
+        allow_smem(sep_scan_kernel<T>, SCAN_SMEM_MAX);
         sep_scan_kernel<T><<<s.grid, s.threads, s.smem, st>>>(s.mode);
         break;
-    }
     case SEP_THOMAS: sep_thomas_kernel<T><<<s.grid, s.threads, 0, st>>>(s.mode); break;
-    case SEP_PLANE: {
-        static bool configured = false;
-        if (!configured) {
-            MHS_CUDA(cudaFuncSetAttribute(sep_dense_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          int(PLANE_SMEM)));
-            configured = true;
-        }
+    case SEP_PLANE:
+        allow_smem(sep_dense_kernel<T>, PLANE_SMEM);
         sep_dense_kernel<T><<<s.grid, s.threads, s.smem, st>>>(s.plane);
         break;
-    }
     default: sep_divide_kernel<T><<<s.grid, s.threads, 0, st>>>(s.mode); break;
     }
     count_launches(1);
@@ -984,39 +972,32 @@ bool dense2d_solve(const std::vector<SepStage<T>>& st, cudaStream_t stream) {
     const ModeArgs<T>& m = st[1].mode;
     const int Kox = (f.M1 + 1) / 2, Koy = (f.A + 1) / 2, r = plane_r<T>();
     const void* fn = reinterpret_cast<const void*>(&sep_dense2d_kernel<T>);
-    static std::mutex mu;
-    static std::map<std::pair<int, int>, int> known;   // cluster size of (nxi, nyi), 0: none
     auto slab = [&](int K, int c) { return ((K + c - 1) / c + r - 1) / r * r; };
-    int c = 0;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        const auto it = known.find({f.M1, f.A});
-        if (it != known.end()) {
-            c = it->second;
-        } else {
-            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PLANE_SMEM)) == cudaSuccess &&
-                cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
-                for (int n = 16; n >= 1 && !c; n /= 2) {
-                    const size_t smem = dense2d_smem<T>(f.M1, f.A, slab(Kox, n), slab(Koy, n));
-                    if (smem > PLANE_SMEM) break;
-                    if (n > 1 && (n / 2) * r >= std::max(Kox, Koy)) continue;   // fewer CTAs suffice
-                    cudaLaunchConfig_t cfg{};
-                    cudaLaunchAttribute attr{};
-                    attr.id = cudaLaunchAttributeClusterDimension;
-                    attr.val.clusterDim.x = n;
-                    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-                    cfg.gridDim = dim3(n, 1, 1);
-                    cfg.blockDim = dim3(PLANE_T, 1, 1);
-                    cfg.dynamicSmemBytes = smem;
-                    cfg.attrs = &attr;
-                    cfg.numAttrs = 1;
-                    int clusters = 0;
-                    if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) c = n;
-                }
-            (void)cudaGetLastError();
-            known[{f.M1, f.A}] = c;
-        }
-    }
+    static PerDevice<std::pair<int, int>, int> sizes;   // cluster size of (nxi, nyi), 0: none
+    const int c = sizes.get(current_device(), {f.M1, f.A}, [&] {
+        int size = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PLANE_SMEM)) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+            for (int n = 16; n >= 1 && !size; n /= 2) {
+                const size_t smem = dense2d_smem<T>(f.M1, f.A, slab(Kox, n), slab(Koy, n));
+                if (smem > PLANE_SMEM) break;
+                if (n > 1 && (n / 2) * r >= std::max(Kox, Koy)) continue;   // fewer CTAs suffice
+                cudaLaunchConfig_t cfg{};
+                cudaLaunchAttribute attr{};
+                attr.id = cudaLaunchAttributeClusterDimension;
+                attr.val.clusterDim.x = n;
+                attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+                cfg.gridDim = dim3(n, 1, 1);
+                cfg.blockDim = dim3(PLANE_T, 1, 1);
+                cfg.dynamicSmemBytes = smem;
+                cfg.attrs = &attr;
+                cfg.numAttrs = 1;
+                int clusters = 0;
+                if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0) size = n;
+            }
+        (void)cudaGetLastError();
+        return size;
+    });
     if (c == 0) return false;
     f.sp = slab(Kox, c);
     b.sp = slab(Koy, c);
@@ -1234,27 +1215,15 @@ void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st)
         if constexpr (sizeof(T) == 4)
             g_sep_kernel<T, SEP_GEMM><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate);
         break;
-    case SEP_SCAN: {
-        static bool configured = false;
-        if (!configured) {
-            MHS_CUDA(cudaFuncSetAttribute(g_sep_kernel<T, SEP_SCAN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          int(SCAN_SMEM_MAX)));
-            configured = true;
-        }
+    case SEP_SCAN:
+        allow_smem(g_sep_kernel<T, SEP_SCAN>, SCAN_SMEM_MAX);
         g_sep_kernel<T, SEP_SCAN><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);
         break;
-    }
     case SEP_THOMAS: g_sep_kernel<T, SEP_THOMAS><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate); break;
-    case SEP_PLANE: {
-        static bool configured = false;
-        if (!configured) {
-            MHS_CUDA(cudaFuncSetAttribute(g_sep_kernel<T, SEP_PLANE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          int(PLANE_SMEM)));
-            configured = true;
-        }
+    case SEP_PLANE:
+        allow_smem(g_sep_kernel<T, SEP_PLANE>, PLANE_SMEM);
         g_sep_kernel<T, SEP_PLANE><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);
         break;
-    }
     case SEP_SPLIT_PLANE:
         if constexpr (sizeof(T) == 8) glaunch_split_plane(t, fmg_step, gate, st);
         break;

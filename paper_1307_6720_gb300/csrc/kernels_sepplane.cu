@@ -26,12 +26,11 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
+#include <utility>
 
 #include "dst_body.cuh"
 #include "mhs_internal.h"
+#include "per_device.h"
 #include "solver.h"
 
 namespace cg = cooperative_groups;
@@ -212,32 +211,29 @@ void* kernel_of() { return reinterpret_cast<void*>(&sep_plane_kernel<T, MODE>); 
 // clusters of this shape and shared memory can run on the device (queried once per configuration)
 template <typename T, int MODE>
 bool cluster_fits(int csize, size_t smem) {
-    static std::mutex mu;
-    static std::map<std::pair<int, size_t>, bool> known;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = known.find({csize, smem});
-    if (it != known.end()) return it->second;
-    bool ok = false;
-    const void* fn = kernel_of<T, MODE>();
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PLANE_SMEM_MAX)) == cudaSuccess &&
-        (csize <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = csize;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.gridDim = dim3(csize, 1, 1);
-        cfg.blockDim = dim3(PLANE_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int clusters = 0;
-        ok = cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0;
-    }
-    (void)cudaGetLastError();
-    known[{csize, smem}] = ok;
-    return ok;
+    static PerDevice<std::pair<int, size_t>, bool> known;
+    return known.get(current_device(), {csize, smem}, [&] {
+        bool ok = false;
+        const void* fn = kernel_of<T, MODE>();
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(PLANE_SMEM_MAX)) == cudaSuccess &&
+            (csize <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = csize;
+            attr.val.clusterDim.y = 1;
+            attr.val.clusterDim.z = 1;
+            cfg.gridDim = dim3(csize, 1, 1);
+            cfg.blockDim = dim3(PLANE_THREADS, 1, 1);
+            cfg.dynamicSmemBytes = smem;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            ok = cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters > 0;
+        }
+        (void)cudaGetLastError();
+        return ok;
+    });
 }
 
 template <typename T, int MODE>

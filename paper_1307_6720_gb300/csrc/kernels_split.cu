@@ -342,12 +342,8 @@ __global__ void __launch_bounds__(SP_T) g_split_plane_kernel(const GSepItem<doub
 
 template <int KS>
 void launch_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
-    static bool attr = false;
     constexpr int smem = SW / 2 * KS * STEP * 4;
-    if (!attr) {
-        MHS_CUDA(cudaFuncSetAttribute(dst_split_kernel<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr = true;
-    }
+    allow_smem(dst_split_kernel<KS>, smem);
     const long long total = (long long)a.lines * a.planes;
     const unsigned blocks = unsigned((total + 8 * SW - 1) / (8 * SW));
     // up to a block per SM (4864 lines): a group of results per block, their lines' digits made by each

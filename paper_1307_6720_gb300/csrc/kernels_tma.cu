@@ -264,12 +264,7 @@ template <int TY, int NS>
 void launch_tma(const Geom& g, const CUtensorMap& tm_in, const CUtensorMap& tm_f, const PlaneCoef<float>* coef,
                 float* uout, int* err, cudaStream_t st) {
     using S = TmaShape<TY, NS>;
-    static bool attr = false;
-    if (!attr) {
-        MHS_CUDA(cudaFuncSetAttribute(rb_sweep_tma_kernel<TY, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      int(S::BYTES)));
-        attr = true;
-    }
+    allow_smem(rb_sweep_tma_kernel<TY, NS>, S::BYTES);
     int per_sm = 0;
     MHS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rb_sweep_tma_kernel<TY, NS>, 32 * TY, S::BYTES));
     const int gx = (g.nx - 2 + TX - 1) / TX, gy = (g.ny - 2 + TY - 1) / TY;

@@ -471,6 +471,14 @@ void launch_lower_pair(const Geom& g, const PlaneCoef<T>* coef, const T* u, cons
                        const T* uc, cudaStream_t st);
 
 // ---- control and sub-cycle (kernels_ctl.cu) ----
+int current_device();
+// lets a kernel take `bytes` of dynamic shared memory on the current device (set once per
+// device; a kernel is always given the same bytes)
+void allow_smem(const void* kernel, size_t bytes);
+template <typename... A>
+void allow_smem(void (*kernel)(A...), size_t bytes) {
+    allow_smem(reinterpret_cast<const void*>(kernel), bytes);
+}
 void launch_bnorm(const double* partial, int n, SolveCtl* ctl, cudaStream_t st);
 size_t subcycle_smem_limit();
 // rows of 32 threads of the sub-cycle CTA of a hierarchy cut at a level with
