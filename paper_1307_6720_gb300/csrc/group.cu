@@ -92,13 +92,17 @@ std::vector<GSepTable<double>>& exact_tables<double>(GDim& D) { return D.exact64
 
 // stage tables of the exact coarse-grid solves: items of stage s and kind k
 // share a launch; block shapes of the plain mode solves follow the launch's
-// thread count
+// thread count.  Dense products (SEP_GEMM) and transforms of long lines by digits
+// (SEP_SPLIT) serve only direct solves, which groups do not take.
 template <typename T>
 void upload_exact(GPart* G, GDim& D, std::vector<std::vector<GSepItem<T>>>& by_stage) {
     std::vector<GSepTable<T>>& out = exact_tables<T>(D);
     out.clear();
     for (auto& items : by_stage) {
-        for (int kind = SEP_DST; kind <= SEP_SPLIT_PLANE; ++kind) {
+        for (const GSepItem<T>& it : items)
+            if (it.st.kind == SEP_GEMM || it.st.kind == SEP_SPLIT)
+                throw Error(MHS_ERR_BAD_STATE, "group: a stage of an exact coarse-grid solve has no grouped form");
+        for (int kind : {SEP_DST, SEP_SCAN, SEP_THOMAS, SEP_DIVIDE, SEP_PLANE, SEP_SPLIT_PLANE}) {
             std::vector<GSepItem<T>> v;
             for (const GSepItem<T>& it : items)
                 if (it.st.kind == kind) v.push_back(it);

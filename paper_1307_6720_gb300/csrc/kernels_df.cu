@@ -26,9 +26,9 @@ __global__ void df_residual_kernel(Geom g, const PlaneCoefDF* __restrict__ cdf, 
     check_last_block(ck, partial);
 }
 
-__global__ void df_correct_kernel(Geom g, int d3, const float* __restrict__ e, float* __restrict__ hi,
+__global__ void df_correct_kernel(Geom g, const float* __restrict__ e, float* __restrict__ hi,
                                   float* __restrict__ lo) {
-    df_correct_body(g, d3, e, hi, lo, blockIdx, gridDim);
+    df_correct_body(g, 1, e, hi, lo, blockIdx, gridDim);
 }
 
 template <bool FZ>
@@ -182,9 +182,8 @@ int launch_df_step(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* 
     return int(grid.x * grid.y * grid.z);
 }
 
-void launch_df_correct(const Geom& g, int dim, const float* e, float* hi, float* lo, cudaStream_t st) {
-    const int d3 = dim == 3;
-    df_correct_kernel<<<df_grid(g, d3, 0), dim3(DF_BX, DF_BY), 0, st>>>(g, d3, e, hi, lo);
+void launch_df_correct(const Geom& g, const float* e, float* hi, float* lo, cudaStream_t st) {
+    df_correct_kernel<<<df_grid(g, 1, 0), dim3(DF_BX, DF_BY), 0, st>>>(g, e, hi, lo);
     count_launches(1);
     MHS_CUDA(cudaGetLastError());
 }

@@ -710,9 +710,8 @@ __global__ void __launch_bounds__(1024) g_sep_kernel(const GSepItem<T>* items, i
     int lb;
     const GSepItem<T>* it = glocate(items, n, gate, fmg_step, lb);
     if (!it) return;
-    const int bx = lb % it->gx, by = (lb / it->gx) % it->gy, bz = lb / (it->gx * it->gy);
-    if constexpr (KIND == SEP_GEMM && sizeof(T) == 4) gemm_body(it->st.gemm, bx, by, bz);
-    else if constexpr (KIND == SEP_SCAN) scan_body(it->st.mode, bx, by);
+    const int bx = lb % it->gx, by = lb / it->gx;
+    if constexpr (KIND == SEP_SCAN) scan_body(it->st.mode, bx, by);
     else if constexpr (KIND == SEP_THOMAS) thomas_body(it->st.mode, bx, by);
     else if constexpr (KIND == SEP_PLANE) plane_body(it->st.plane, bx, by);
     else divide_body(it->st.mode, bx, by);
@@ -1211,10 +1210,6 @@ void glaunch_sep(const GSepTable<T>& t, int fmg_step, int gate, cudaStream_t st)
     if (t.n == 0) return;
     switch (t.kind) {
     case SEP_DST: glaunch_dst<T>(t, fmg_step, gate, st); return;
-    case SEP_GEMM:
-        if constexpr (sizeof(T) == 4)
-            g_sep_kernel<T, SEP_GEMM><<<t.blocks, t.threads, 0, st>>>(t.items, t.n, fmg_step, gate);
-        break;
     case SEP_SCAN:
         allow_smem(g_sep_kernel<T, SEP_SCAN>, SCAN_SMEM_MAX);
         g_sep_kernel<T, SEP_SCAN><<<t.blocks, t.threads, t.smem, st>>>(t.items, t.n, fmg_step, gate);

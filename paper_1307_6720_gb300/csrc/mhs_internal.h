@@ -497,13 +497,13 @@ void launch_df_split(const Geom& g, int dim, const double* f, float* hi, float* 
 int launch_df_residual(const Geom& g, int dim, const PlaneCoefDF* cdf, const float* hi, const float* lo,
                        const float* fh, const float* fl, float* r32, double* partial, int max_blocks, cudaStream_t st,
                        const CheckArgs& ck = CheckArgs());
-// (hi, lo) += e at interior nodes
-// the two double-float iterates and which is current (DFState); flip == nullptr: the first
+// the two double-float iterates and, in device memory, which is current (DFState)
 struct DFPair {
     float *hi[2], *lo[2];
     const int* flip;
 };
-void launch_df_correct(const Geom& g, int dim, const float* e, float* hi, float* lo, cudaStream_t st);
+// (hi, lo) += e at the interior nodes of a 3D level that df_step_available does not serve
+void launch_df_correct(const Geom& g, const float* e, float* hi, float* lo, cudaStream_t st);
 // the lower boundary, and 3D levels wide enough for the pass: correction and residual in one launch
 bool df_step_available(const Geom& g, int dim);
 // current pair + e into the other pair (faces copied), and its residual as launch_df_residual's

@@ -643,7 +643,7 @@ static void correct_and_residual(mhs_ctx* c, Hierarchy& H, CheckArgs ck) {
     if (!df_step_available(g, H.dim)) {
         TimedScope t(c->timer, MHS_KT_CORRECT, double(g.interior()) * 20.0, double(g.interior()) * 8.0, c->stream,
                      H.dim == 3);
-        launch_df_correct(g, H.dim, H.s[0].u, H.df.hi, H.df.lo, c->stream);
+        launch_df_correct(g, H.s[0].u, H.df.hi, H.df.lo, c->stream);
         t.stop();
         residual_partials(c, H, MHS_MIXED, false, ck);
         return;
