@@ -514,6 +514,21 @@ static bool fused_level(const mhs_ctx* c, const Hierarchy& H, int l) {
                           : H.g[l].interior() >= size_t(c->opts.fused_min);
 }
 
+// FP32 levels (one bit each) that a mixed V-cycle sweeps in the fused form: at
+// least fused_min interior nodes, no pairs, above the coarse-grid solve
+unsigned fused_levels(const mhs_ctx* c) {
+    const Hierarchy& H = c->h3;
+    if (c->opts.flags & MHS_FLAG_SEPARABLE) return 0;
+    int end = std::min(cut_of<float>(H), H.nlev());
+    if (exact_of<float>(H) >= 0) end = std::min(end, exact_of<float>(H));
+    unsigned m = 0;
+    for (int l = 0; l < end; ++l) {
+        const PairPasses p = pair_passes<float>(c, H, l);
+        if (fused_level<float>(c, H, l) && p.pre + p.post == 0) m |= 1u << l;
+    }
+    return m;
+}
+
 // An out-of-place sweep writes interior nodes only and reads t as the old
 // iterate on every second sweep, so t's boundary faces must hold u's.  t is
 // also scratch of the separable solver (a coarse-grid solve, or the inner

@@ -57,6 +57,7 @@ template <typename T>
 void vcycle(mhs_ctx* c, Hierarchy& H, int l);
 template <typename T>
 void smooth_hook(mhs_ctx* c, Hierarchy& H, int l);   // one sweep as the V-cycle runs it
+unsigned fused_levels(const mhs_ctx* c);   // FP32 levels swept in the fused form by the handle's options
 double read_norm2(mhs_ctx* c, int slot);
 bool is_device_ptr(const void* p);
 // field recovery of the resident P into dense host or device arrays (B_x, B_y, B_z, p, rho; NULL

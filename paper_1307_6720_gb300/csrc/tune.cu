@@ -12,7 +12,8 @@
 //   - the sub-cycle cut-off (cut64 in FP64 mode, cut32 in mixed mode), one
 //     candidate per level that the sub-cycle could start from,
 //   - the fused TMA sweep threshold on FP32 levels (mixed mode, point smoother)
-//     and the height of its tiles (tma_rows),
+//     and the height of its tiles (tma_rows), where levels exist that it decides
+//     about (sweeps that run in pairs do not ask it),
 //   - the full-multigrid first cycle (MHS_FLAG_NO_FMG),
 //   - the thread-block shape of the red-black point passes (tile),
 // at most two rounds, a change kept only when it saves at least 3 %.  The
@@ -143,13 +144,18 @@ void autotune(mhs_ctx* c, double tol, int mode, int repeats, mhs_tune_result* ou
         }
         const bool line = (best.flags & MHS_FLAG_ZLINE) || (!(best.flags & MHS_FLAG_POINT) && c->aniso >= 5);
         if (mode == MHS_MIXED && !line && c->h3.nlev() > 1) {
-            // fused sweep on the finest FP32 level, on the two finest, or nowhere
+            // fused sweep on the finest FP32 level, on the two finest, or nowhere; a threshold that
+            // leaves every level as it is would be timed for its noise
+            auto swept = [&](const mhs_solver_opts& o) {
+                apply_opts(c, o);
+                return fused_levels(c);
+            };
             for (int fm : {clamp_int(c->h3.g[0].interior()), clamp_int(c->h3.g[1].interior()), INT_MAX}) {
                 mhs_solver_opts o = best;
                 o.fused_min = fm;
-                consider(o);
+                if (swept(o) != swept(best)) consider(o);
             }
-            if (best.fused_min != INT_MAX)
+            if (swept(best))
                 for (int rows : {8, 16}) {   // tile height of the fused sweep
                     mhs_solver_opts o = best;
                     o.tma_rows = rows;

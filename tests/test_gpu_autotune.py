@@ -67,6 +67,28 @@ def test_autotune_isotropic_mixed_never_slower_and_clear(M):
     M.mhs_destroy(h)
 
 
+def test_autotune_times_no_threshold_that_decides_nothing(M):
+    """On 129 x 129 x 97 nodes every sweep of the finest level runs in a pair and
+    the coarser levels are small: neither the threshold of the fused sweep nor
+    its tile height is a candidate.  (Candidates of a round: two smoothers, five
+    sweep counts, the coarse-grid solve and the cut-off per level and none, the
+    first cycle, five block shapes; a second round when something was kept.)"""
+    M.mhs_tune_clear()
+    nx, ny, nz = 129, 129, 97
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=1.0, Lz=0.75, alpha=0.3, xi_kind=1, xi_a=0.5, xi_kappa=1.0)
+    h = _handle(M, pr, S.magnetogram_random(nx, ny, 1.0, 1.0, seed=44))
+    M.mhs_set_options(h, nu1=2, nu2=2)
+    res = M.mhs_autotune(h, 1e-10, M.MHS_MIXED, repeats=1)
+    levels = M.mhs_num_levels(h, 3)
+    per_round = 2 + 5 + levels + levels + 1 + 5
+    o = res["opts"]
+    paired = o["nu1"] >= 2 and o["nu2"] >= 2   # else the threshold decides after all
+    assert not paired or (o["fused_min"] == 12000000 and o["tma_rows"] == 8)
+    one = (o["nu1"], o["nu2"], o["flags"], o["cut32"], o["sep_coarse"], o["tile"]) == (2, 2, 0, 4000, 300000, 1)
+    assert res["candidates"] <= 1 + (per_round - 2 if one else 2 * per_round + (0 if paired else 10))
+    M.mhs_destroy(h)
+
+
 def test_autotune_requires_bz(M):
     h = M.mhs_create(33, 33, 33, 1.0, 1.0, 1.0, 0.0, None)
     with pytest.raises(M.MhsError) as e:
