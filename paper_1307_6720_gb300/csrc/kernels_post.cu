@@ -36,21 +36,6 @@ __device__ __forceinline__ double num1(const double* __restrict__ f, size_t c, p
     return v;
 }
 
-// sqrt(m): an FP32 reciprocal square root refined by one coupled Newton
-// (Goldschmidt) step for g ~ sqrt(m), h ~ 1/(2 sqrt(m)) and one correction of
-// g by its residual, 8 FP64 instructions instead of about 22; the relative
-// error before the last rounding is below 2^-80.  Arguments outside the FP32
-// range (and 0, NaN) take the library's sqrt.
-__device__ __forceinline__ double sqrt_mid(double m) {
-    if (!(m > 1e-30 && m < 1e30)) return sqrt(m);
-    const float y = rsqrtf(float(m));
-    double g = m * double(y), h = double(0.5f * y);
-    const double r = fma(-g, h, 0.5);
-    g = fma(g, r, g);
-    h = fma(h, r, h);
-    return fma(fma(-g, g, m), h, g);
-}
-
 // j and the magnitudes on dense arrays; wx, wy, wz = 1/(2 h mu0).  A block
 // owns 256 consecutive nodes of a plane and `per` consecutive planes.  Bound
 // by the FP64 pipe (12 instructions per node for j, 22 for the two

@@ -137,3 +137,32 @@ def test_field_lines_do_not_depend_on_the_number_of_lines(M, extra):
         pq, lq = trace(seeds[a:b])
         assert torch.equal(pq, p[a:b]) and torch.equal(lq, l[a:b])
     assert int(l[3]) == 0 and int((l > 1).sum()) > n // 2 and int((l < steps + 1).sum()) > 100
+
+
+def test_magnitudes_equal_the_root_of_their_components(M):
+    """|j| and |B| node by node against the square root of the returned components
+    in extended precision, with P over sixty decades (squares far below and above
+    the range in which the root is refined from FP32, and on both sides of its
+    limits) and a part of the box where it vanishes.  Bound: three rounded
+    operations in the sum of squares, halved by the root, and the root's own
+    rounding, 2.5 units of 2^-53; four allowed."""
+    import torch
+    nx, ny, nz = 17, 13, 65
+    h = M.mhs_create(nx, ny, nz, 1.0, 0.75, 4.0, 0.4, None)
+    M.mhs_set_stream(h, torch.cuda.current_stream())
+    M.mhs_set_lower_bz(h, S.magnetogram_random(nx, ny, 1.0, 0.75, seed=3))
+    M.mhs_solve(h, 1e-8, M.MHS_FP64)
+    rng = np.random.default_rng(9)
+    P = rng.standard_normal((nz, ny, nx)) * 10.0 ** np.linspace(-32, 28, nz)[:, None, None]
+    P[20:30] = 0.0
+    M.mhs_level_write(h, 3, 0, M.MHS_FIELD_U, 0, P)
+    B = [np.zeros((nz, ny, nx)) for _ in range(3)]
+    M.mhs_fields(h, *B)
+    j = [np.zeros((nz, ny, nx)) for _ in range(5)]
+    M.mhs_current(h, *j)
+    for comp, mag in ((B, j[4]), (j[:3], j[3])):
+        want = np.sqrt(sum(c.astype(np.longdouble) ** 2 for c in comp))
+        assert np.all(np.abs(mag - want) <= 4 * 2.0**-53 * want)
+        sq = want**2
+        assert (sq == 0).any() and ((sq > 0) & (sq < 1e-30)).any() and ((sq > 1e-30) & (sq < 1e30)).any() and (sq > 1e30).any()
+    M.mhs_destroy(h)
