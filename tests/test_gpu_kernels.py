@@ -610,10 +610,10 @@ def test_zline_vcycle_parity(M, prec, cut):
 
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("shape", [(19, 35, 9), (35, 19, 21), (57, 57, 89), (41, 41, 321), (11, 7, 5)])
-def test_dense_transform_tiles(M, shape, prec):
-    """Dense sine transforms at the edges of their output tiles (16, 32 and 64:
-    one interior node past a tile, ragged ends, batches that select each
-    tile), against the separable direct solution formed with plain products."""
+def test_ragged_plane_transforms(M, shape, prec):
+    """Plane transforms of lengths that are no powers of two, few and many
+    planes (one result of either parity per block up to sixteen), against the
+    separable direct solution formed with plain products."""
     from oracle import exact
     nx, ny, nz = shape
     pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
@@ -674,13 +674,14 @@ def test_levels_and_counts_without_pairs(M, shape, nu):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("shape", [(5, 5, 5), (7, 5, 9), (9, 33, 5), (35, 19, 5), (67, 67, 9), (65, 63, 9), (129, 9, 5),
-                                   (129, 129, 5), (127, 67, 5), (65, 17, 5), (65, 19, 5), (19, 65, 7), (35, 33, 5)])
+@pytest.mark.parametrize("shape", [(5, 5, 5), (7, 5, 9), (9, 33, 5), (35, 19, 5), (33, 65, 9), (65, 63, 9), (129, 9, 5),
+                                   (129, 129, 5), (65, 17, 5), (65, 19, 5), (19, 65, 7), (35, 33, 5)])
 def test_plane_transforms_of_folded_matrices(M, shape, prec):
     """The plane transforms with folded sine matrices (one pair of lines up to
-    128 cells, odd and even lengths, ragged slabs of results), 2D and 3D,
-    against the separable direct solution; the staged form, one transform per
-    launch, gives the same bits.  Bounds: those of test_exact_op_parity."""
+    128 cells, ragged slabs of results), 2D and 3D, against the separable direct
+    solution; the staged form, one transform per launch, gives the same bits.
+    Bounds: those of test_exact_op_parity.  (Longer sides that are no powers of
+    two: test_direct_mixed_solves_of_ragged_boxes.)"""
     from oracle import exact
     nx, ny, nz = shape
     pr, h = _make(M, nx, ny, nz, Lx=1.0, Ly=0.6, Lz=0.8)
@@ -689,9 +690,6 @@ def test_plane_transforms_of_folded_matrices(M, shape, prec):
         f = np.random.default_rng(nx + dim).standard_normal(shape_l)
         if prec == 1:
             f = f.astype(np.float32).astype(np.float64)
-        fast = (nx - 1) & (nx - 2) == 0 and (ny - 1) & (ny - 2) == 0
-        if not (fast or (nx <= 66 and ny <= 66)):
-            continue
         got = []
         for flags in (0, M.MHS_FLAG_STAGED_TRANSFORMS):
             M.mhs_set_options(h, flags=flags)

@@ -448,7 +448,7 @@ def test_separable_inner_solver_reaches_exact_solution(M, case, mode):
     elif case == "small":
         pr = S.problem(5, 9, 5, Ly=2.0, alpha=0.4)
         bz = S.magnetogram_random(5, 9, 1.0, 2.0, seed=54)
-    else:   # nx - 1 = 48, ny - 1 = 96: not powers of two, the sine transforms run as matrix products
+    else:   # nx - 1 = 48, ny - 1 = 96: not powers of two, the mixed solve's transforms run as dense planes
         pr = S.problem(49, 97, 25, Ly=2.0, Lz=0.5, alpha=0.4, xi_kind=1, xi_a=0.6, xi_kappa=1.0)
         bz = S.magnetogram_random(49, 97, 1.0, 2.0, seed=55)
     tol = 5e-12 if mode == 1 else 1e-13
@@ -459,6 +459,44 @@ def test_separable_inner_solver_reaches_exact_solution(M, case, mode):
         # FP64 direct solves: one step leaves only rounding, a second at most
         assert info["cycles_3d"] <= 3 and info["cycles_2d"] <= 3, info
     _compare(got, _oracle(pr, bz), 1e-10)
+
+
+@pytest.mark.parametrize("shape,per_solve", [((67, 67, 9), (3, 1)), ((127, 67, 5), (3, 1)), ((113, 97, 9), (3, 1)),
+                                             ((161, 145, 9), (5, 5)), ((161, 145, 25), (5, 5)), ((145, 161, 73), (5, 5)),
+                                             ((137, 9, 17), (5, 5))])
+def test_direct_mixed_solves_of_ragged_boxes(M, shape, per_solve):
+    """Mixed MHS_FLAG_SEPARABLE solves of boxes whose sides are no powers of two:
+    dense planes up to 128 cells a side (3 launches per volume solve, one cluster
+    per lower-boundary solve), past that batched products (5 launches each) in
+    output tiles of 16 (one plane, 7 planes), 32 (23 planes) and 64 (71 planes).
+    Every step cuts the error by about the FP32 rounding level, so a wrong
+    transform shows in the number of steps; the potential to the FP64 bar, the
+    fields to the mixed one."""
+    nx, ny, nz = shape
+    pr = S.problem(nx, ny, nz, Lx=1.0, Ly=(ny - 1) / (nx - 1), Lz=(nz - 1) / (nx - 1), alpha=0.4, xi_kind=1, xi_a=0.6,
+                   xi_kappa=1.0)
+    bz = S.magnetogram_random(nx, ny, 1.0, pr["Ly"], seed=nx + nz)
+    info, got = _gpu_solve(M, pr, bz, 5e-12, 1, opts=dict(flags=M.MHS_FLAG_SEPARABLE))
+    assert 2 <= info["cycles_3d"] <= 4 and 2 <= info["cycles_2d"] <= 4, info
+    want = _oracle(pr, bz)
+    assert rel(got["phi"], want["phi"]) < 1e-10
+    _compare(got, want, 1e-8)
+    # launches of the steps that a tighter tolerance adds: the forms of the transforms
+    h = M.mhs_create(nx, ny, nz, pr["Lx"], pr["Ly"], pr["Lz"], pr["alpha"], _xi(M, pr))
+    M.mhs_set_lower_bz(h, bz)
+    M.mhs_set_options(h, flags=M.MHS_FLAG_SEPARABLE | M.MHS_FLAG_NO_FMG)
+    counts = {}
+    M.mhs_solve(h, 1e-3, 1)   # (the first solve also makes the elimination factors)
+    for tol in (1e-3, 1e-9, 5e-12):
+        n0 = M.mhs_kernel_launches()
+        i = M.mhs_solve(h, tol, 1)
+        counts[i["cycles_2d"], i["cycles_3d"]] = M.mhs_kernel_launches() - n0
+    (a2, a3), (b2, b3) = min(counts), max(counts)
+    assert b3 > a3 and b2 > a2
+    step3 = 1 if nx >= 95 else 2   # correction and residual, one launch or two (test_mixed_step_on_wide_levels)
+    more = (b3 - a3) * (per_solve[0] + step3) + (b2 - a2) * (per_solve[1] + 1)
+    assert counts[b2, b3] - counts[a2, a3] == more, counts
+    M.mhs_destroy(h)
 
 
 @pytest.mark.parametrize("mode", [0, 1])
