@@ -66,14 +66,18 @@ inline bool dense_planes_faster(bool fp64, int dim, int cx, int cy, int planes) 
 // Chunks of the nzi inner planes of the double-float march (df_march_body) over
 // `tiles` tiles: the count with the least waves of resident blocks (two per
 // SM) times planes, three of them start-up; at most max_blocks blocks (0: any)
-// unless the tiles alone are more.  Down to single planes, or a shallow level
-// is marched by its few tiles (129 x 129 x 9 in one chunk of seven planes: 16
-// blocks; a direct mixed solve 205 us, with single planes 190 us).
+// unless the tiles alone are more.  Chunks of four planes or more, and two of
+// levels of five to seven planes (a direct mixed solve of 129 x 129 x 9: 205 us in
+// one chunk, 196 in two; as two launches per step 198).  Shorter chunks fill the
+// chip better on shallow levels by themselves (190 us with single planes) but groups
+// keep the decomposition, which orders the sums, and have blocks enough: 32 of
+// them 3.70 ms, in two chunks 3.75, in single planes 4.08; 16 of 129 x 33 x 33
+// 1.89 and, in single planes, 2.10 ms.
 inline int df_march_chunks(long long tiles, int nzi, int max_blocks) {
     const long long resident = 2 * RULE_SMS;
     long long best = 0;
     int chunks = 1;
-    for (int n = 1; n <= nzi; ++n) {
+    for (int n = 1; n <= std::max(nzi > 4 ? 2 : 1, nzi / 4); ++n) {
         const int per = (nzi + n - 1) / n, m = (nzi + per - 1) / per;
         if (n > 1 && max_blocks > 0 && tiles * m > max_blocks) break;
         const long long cost = (tiles * m + resident - 1) / resident * (per + 3);

@@ -81,22 +81,23 @@ def test_transforms_of_a_level_take_the_faster_form(rules, prec, cx, cy, planes,
     assert bool(pick) == (dense < fast)
 
 
-def test_double_float_march_fills_the_chip_on_shallow_levels(rules):
+def test_double_float_march_splits_shallow_levels(rules):
     """Chunks of the double-float march: never empty, never over the limit of
-    partial sums, never slower by the rule's own measure than any other
-    count, and single planes where the tiles are few."""
+    partial sums, of four planes or more but for two of five to seven planes, and
+    by the rule's own measure never slower than another such count."""
     for tiles in (1, 2, 3, 5, 16, 33, 64, 110, 152, 305, 1024):
-        for nzi in (1, 2, 3, 5, 7, 9, 15, 31, 63, 127, 255, 511):
+        for nzi in (1, 2, 3, 4, 5, 7, 8, 9, 15, 31, 63, 127, 255, 511):
             n = rules.df_march_chunks(tiles, nzi, 65536)
             per = -(-nzi // n)
             assert 1 <= n <= nzi and (n - 1) * per < nzi
             assert n == 1 or tiles * n <= 65536
+            assert per >= 4 or nzi < 8 and n == (2 if nzi > 4 else 1)
             cost = -(-tiles * n // 304) * (per + 3)
-            for p in range(1, nzi + 1):
+            for p in range(4, nzi + 1):
                 m = -(-nzi // p)
-                if tiles * m <= 65536:
+                if m * 4 <= nzi and tiles * m <= 65536:
                     assert cost <= -(-tiles * m // 304) * (p + 3), (tiles, nzi, n, m)
-    assert rules.df_march_chunks(16, 7, 65536) == 7
+    assert rules.df_march_chunks(16, 7, 65536) == 2 and rules.df_march_chunks(16, 3, 65536) == 1
     assert rules.df_march_chunks(300, 200, 700) * 300 <= 700 and rules.df_march_chunks(1000, 200, 700) == 1
 
 
