@@ -108,7 +108,7 @@ typedef struct {
     int cut32;           /* same for FP32 levels [4000] */
     int fused_min;       /* FP32 3D levels with at least this many interior nodes use the fused, TMA-staged
                             red-black sweep (one pass per sweep) when no two sweeps of theirs run as one pass,
-                            which levels of nx = 4m + 1 and some 1.2 million nodes do with nu1, nu2 of two and
+                            which levels of nx = 4m + 1 and about a million nodes do with nu1, nu2 of two and
                             more (a sweep left over there runs as colour passes); smaller levels use the two
                             colour passes, which have less latency; results do not depend on it [12000000] */
     int sep_coarse;      /* coarse-grid solve of the V-cycles: the first level below the finest with at most this

@@ -650,7 +650,7 @@ def _vcycles_with_and_without_pairs(M, shape, nu):
 
 
 @pytest.mark.parametrize("nu", [(2, 2), (4, 2), (3, 3), (3, 2), (2, 4)])
-@pytest.mark.parametrize("shape", [(129, 129, 97), (249, 161, 49), (193, 97, 129), (129, 33, 1025), (73, 145, 97)])
+@pytest.mark.parametrize("shape", [(129, 129, 65), (249, 161, 49), (193, 97, 129), (129, 33, 1025), (73, 145, 97)])
 def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
     """FP32 V-cycles whose pairs of sweeps run as one out-of-place pass (tiles
     in x, y and z with ragged ends, boundary values that are not zero, odd
@@ -663,10 +663,10 @@ def test_paired_sweeps_equal_colour_passes_fp32(M, shape, nu):
     assert not np.array_equal(got[0], u)
 
 
-@pytest.mark.parametrize("shape,nu", [((129, 129, 65), (2, 2)), ((33, 129, 257), (2, 2)), ((17, 33, 2049), (2, 2)),
+@pytest.mark.parametrize("shape,nu", [((257, 129, 33), (2, 2)), ((33, 129, 257), (2, 2)), ((17, 33, 2049), (2, 2)),
                                       ((65, 65, 257), (2, 2)), ((129, 129, 97), (2, 1)), ((129, 129, 97), (1, 1))])
 def test_levels_and_counts_without_pairs(M, shape, nu):
-    """Levels on which the pass of two sweeps would be the slower form, and
+    """Levels on which the pass of two sweeps would be far the slower form, and
     sweep counts without an even number of pairs, run colour passes."""
     got, launches, u = _vcycles_with_and_without_pairs(M, shape, nu)
     assert launches[0] == launches[1]
