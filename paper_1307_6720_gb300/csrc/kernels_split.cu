@@ -130,6 +130,7 @@ __device__ __forceinline__ int line_max(int e) {
 template <int KS>
 __device__ __forceinline__ void products(const unsigned* A, const uint2* __restrict__ bt, int lane,
                                          float (&acc)[TILES][ORDERS][4]) {
+    static_assert(DIG * 16LL * KS * 128 * 128 < 1LL << 24, "sums of digit products must be exact in FP32");
 #pragma unroll
     for (int n = 0; n < TILES; ++n)
 #pragma unroll
@@ -360,8 +361,9 @@ void launch_split(const DstArgs<double>& a, const void* tab, cudaStream_t st) {
 // transforms serve smaller ones
 bool split_planes(const Geom& g) { return g.nx - 1 == SP_CELLS && g.ny - 1 == SP_CELLS; }
 
-// direct corrections.  512 cells: the digits of a parity (58 KB for 16 lines) would leave one block per SM; 64: direct
-// corrections keep the fast transforms (their error, 2.3e-15 to 3.5e-15 at 65 x 65 x 33, is the tridiagonal solves')
+// direct corrections, where both axes are of such lengths.  512 cells: 7 x 256 digit products of up to 2^14 pass 2^24, so
+// FP32 sums of them would not be exact (and the digits of a parity, 58 KB for 16 lines, would leave one block per SM); 64:
+// direct corrections keep the fast transforms (their error, 2.3e-15 to 3.5e-15 at 65 x 65 x 33, is the tridiagonal solves')
 bool split_length(int N) { return N == 128 || N == 256; }
 
 // sin(pi q / N) 2^55 as an integer
