@@ -13,16 +13,20 @@
 //   D_k = (alpha^2 - 2 cz) + cx_k mu_x(m) + cy_k mu_y(n),
 // and the lower-boundary problem (eq. lower_bound) into a division per mode.
 // Every multigrid level is a rediscretisation with the same structure, so
-// the same solver applies on any level.  The sine transforms are fast
-// transforms (kernels_dst.cu) on large planes whose nx - 1 and ny - 1 are powers
-// of two, dense products with folded sine matrices, both transforms of a plane
-// in one launch, on planes of at most 128 cells a side (plane_body), exact
-// digit products on the tensor cores in the FP64 direct correction of 128 and
-// 256 cells and on coarse FP64 levels of 64 x 64 cells, where the FP64 pipe
-// bounds the fast transforms (kernels_split.cu), and in FP32 batched GEMMs with the (symmetric)
-// sine matrices otherwise (in FP64 such levels are refused, sep_level_ok); the
-// inverse is the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the solve is accurate to about 1e-6
-// relative, which the double-float outer loop of mixed mode then corrects.
+// the same solver applies on any level.  The sine transforms are
+// - dense products with folded sine matrices, both transforms of a plane in one
+//   launch (plane_body), on planes of at most 128 cells a side that have no fast
+//   transform or a slower one (dense_planes_faster in launch_rules.h);
+// - exact digit products on the tensor cores in the FP64 direct correction of 128
+//   and 256 cells and on coarse FP64 levels of 64 x 64 cells, where the FP64 pipe
+//   bounds the fast transforms (kernels_split.cu);
+// - fast transforms (kernels_dst.cu) on other planes whose nx - 1 and ny - 1 are
+//   powers of two;
+// - in FP32 batched GEMMs with the (symmetric) sine matrices otherwise (in FP64
+//   such levels are refused, sep_level_ok).
+// The inverse is the same transform scaled by (2/(nx-1)) (2/(ny-1)).  In FP32 the
+// solve is accurate to about 1e-6 relative, which the double-float outer loop of
+// mixed mode then corrects.
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -1,8 +1,9 @@
 // Separable solve of one level with the sine transforms of each plane fused
 // into one kernel: the coarse-grid solves of the V-cycles (and any other
 // single-level separable solve whose planes fit the shared memory of a
-// thread-block cluster) on levels with fast transforms: those of at most 128
-// cells a side take dense planes (FP64: smaller ones, or digit products).
+// thread-block cluster) on levels whose fast transforms are the fastest: most
+// planes of at most 128 cells a side take dense planes (FP64: of at most 32, or
+// digit products; dense_planes_faster in launch_rules.h).
 //
 // The staged separable solve (kernels_sep.cu) runs one launch per transform
 // pass (x, y, mode solves, inverse y, inverse x) with the transformed data
