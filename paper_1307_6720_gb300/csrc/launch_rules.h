@@ -117,23 +117,24 @@ inline PairShapeOf pair_shape(int nx, int ny, int nz) {
 
 // Levels whose pairs of sweeps run as one pass: those where its march takes less
 // time than four colour passes, or up to 2.5 us more.  nx = 4m + 1: see PairTile.  A
-// step takes 1.04 us; the colour passes, up to three million nodes, 7.45 us more than
+// step takes 1.04 us; the colour passes, up to four million nodes, 7.45 us more than
 // the march's start and 5.57 us per million nodes, rows counted in whole warps of 64
-// nodes (fitted to whole mixed solves of 62 boxes of 0.9 to 2.9 million nodes, within
-// 0.8 us).  Four passes against one, us more (+) or less (-) for the one: 129^3 -1.4,
-// 113^3 -2.1, 97 x 97 x 193 -4.1; 129 x 129 x 65 +1.4, 65 x 65 x 513 +4.1, 33 x 33 x 1025
-// +6.9, 17 x 33 x 2049 +9.6 (17 of 128 columns of its tiles used).  The passes are ahead
-// while u and f stay in cache, of which the one pass needs a quarter of the traffic: past
-// three million nodes it wins (257 x 129 x 129 -8.2, 33 x 129 x 1025 -36), and beside other
-// solves it wins earlier (an uneven group with 129 x 129 x 65 members 11.16 ms, with
-// passes for these 11.43; eight solves of 257 x 257 x 33 4.72 and 5.43 ms), hence the 2.5
-// us.  Levels of less than 800,000 nodes keep the passes (65^3 mixed solves 1.04 ms with
-// them, 1.15 ms with pairs).
+// nodes (fitted to whole mixed solves of 82 boxes of 0.9 to 4 million nodes: within
+// 2.5 us but on three of the longest).  Four passes against one, us more (+) or less
+// (-) for the one: 129^3 -1.4, 113^3 -2.1, 97 x 97 x 193 -4.1, 193 x 193 x 97 -5.1; 129 x
+// 129 x 65 +1.4, 65 x 65 x 513 +4.1, 33 x 33 x 1025 +6.9, 17 x 33 x 2049 +9.6 (17 of 128
+// columns of its tiles used), 33 x 33 x 4097 +22.  The passes are ahead while u and f stay
+// in cache, of which the one pass needs a quarter of the traffic: from four million
+// nodes, where they run in their vector form, it wins on every box (257 x 129 x 129 -8.2,
+// 33 x 129 x 1025 -36), and beside other solves it wins earlier (an uneven group with 129
+// x 129 x 65 members 11.16 ms, with passes for these 11.43; eight solves of 257 x 257 x 33
+// 4.72 and 5.43 ms), hence the 2.5 us.  Levels of less than 800,000 nodes keep the
+// passes (65^3 mixed solves 1.04 ms with them, 1.15 ms with pairs).
 inline bool pair_pays(int nx, int ny, int nz) {
     const long long rows = (long long)(ny - 2) * (nz - 2), nodes = rows * (nx - 2);
     if ((nx & 3) != 1 || nodes < 800000) return false;
     const double padded = double((nx - 2 + 63) / 64 * 64) * double(rows);
-    return nodes >= 3000000 || 1.04 * double(pair_shape(nx, ny, nz).steps) < 7.45 + 5.57e-6 * padded + 2.5;
+    return nodes >= 4000000 || 1.04 * double(pair_shape(nx, ny, nz).steps) < 7.45 + 5.57e-6 * padded + 2.5;
 }
 
 }  // namespace mhs
